@@ -64,9 +64,13 @@ __global__ void mark_done_kernel(SolverCtl* ctl) {
   ctl->done = 1;
 }
 
-// ---- gauge field: host layout -> even-odd structure of arrays (S1)
-__global__ void gauge_pack_f64_kernel(Geom g, const double* lex, double2* out, int nc) {
+// ---- gauge field: host layout -> even-odd structure of arrays (S1), the
+// elements as fixed-point numbers (nbad counts the links with an element the
+// fixed-point form does not take, row c of 12-real storage included) or, with
+// nbad null, as the doubles they are
+__global__ void gauge_pack_f64_kernel(Geom g, const double* lex, double2* out, int nc, unsigned* nbad) {
   const int n = 2 * g.Vh;
+  unsigned bad = 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int parity = i / g.Vh, h = i - parity * g.Vh;
     int x, y, z, t;
@@ -75,9 +79,40 @@ __global__ void gauge_pack_f64_kernel(Geom g, const double* lex, double2* out, i
     for (int mu = 0; mu < 4; ++mu) {
       const double2* src = reinterpret_cast<const double2*>(lex + (s * 4 + mu) * 18);
       double2* dst = out + (size_t)(parity * 4 + mu) * nc * g.stride + h;
-      for (int c = 0; c < nc; ++c) dst[(size_t)c * g.stride] = src[c];
+      if (!nbad) {
+        for (int c = 0; c < nc; ++c) dst[(size_t)c * g.stride] = src[c];
+        continue;
+      }
+      double2 u[9];
+#pragma unroll
+      for (int c = 0; c < 6; ++c) u[c] = src[c];
+      if (nc == 9) {
+#pragma unroll
+        for (int c = 6; c < 9; ++c) u[c] = src[c];
+      } else {
+        double r[18];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+          r[2 * c] = u[c].x;
+          r[2 * c + 1] = u[c].y;
+        }
+        reconstruct_row3(r);
+#pragma unroll
+        for (int c = 6; c < 9; ++c) u[c] = make_double2(r[2 * c], r[2 * c + 1]);
+      }
+      bool ok = true;
+#pragma unroll
+      for (int c = 0; c < 9; ++c) {
+        ok = ok && fabs(u[c].x) <= kFixedLinkMax && fabs(u[c].y) <= kFixedLinkMax;  // false for a NaN
+        if (c < nc) {
+          const int2 re = fx_link(u[c].x), im = fx_link(u[c].y);
+          reinterpret_cast<int4*>(dst)[(size_t)c * g.stride] = make_int4(re.x, re.y, im.x, im.y);
+        }
+      }
+      bad += !ok;
     }
   }
+  if (bad) atomicAdd(nbad, bad);
 }
 
 // ---- temporal gauge (Sec. 4.3), FP64 on the host-layout links in place.
@@ -174,13 +209,13 @@ __global__ void temporal_gauge_pack_kernel(Geom g, const double2* G, double2* ou
 }
 
 // FP64 copy (first two rows) -> FP32 / 16-bit copies
-__global__ void gauge_f64_to_f32_kernel(Geom g, const double2* in, int nc, float4* out) {
+__global__ void gauge_f64_to_f32_kernel(Geom g, const double2* in, int nc, bool fixed, float4* out) {
   const int n = 8 * g.Vh;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int pm = i / g.Vh, h = i - pm * g.Vh;
     double r[12];
     for (int c = 0; c < 6; ++c) {
-      double2 d = in[((size_t)pm * nc + c) * g.stride + h];
+      double2 d = link_value(in[((size_t)pm * nc + c) * g.stride + h], fixed);
       r[2 * c] = d.x;
       r[2 * c + 1] = d.y;
     }
@@ -200,13 +235,13 @@ __device__ __forceinline__ uint32_t link16(double u) {
 }
 
 template <Fmt16 F>
-__global__ void gauge_f64_to_16_kernel(Geom g, const double2* in, int nc, uint4* out8, uint2* out4) {
+__global__ void gauge_f64_to_16_kernel(Geom g, const double2* in, int nc, bool fixed, uint4* out8, uint2* out4) {
   const int n = 8 * g.Vh;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int pm = i / g.Vh, h = i - pm * g.Vh;
     uint32_t w[6];
     for (int c = 0; c < 6; ++c) {
-      double2 d = in[((size_t)pm * nc + c) * g.stride + h];
+      double2 d = link_value(in[((size_t)pm * nc + c) * g.stride + h], fixed);
       w[c] = link16<F>(d.x) | (link16<F>(d.y) << 16);
     }
     out8[(size_t)pm * g.stride + h] = make_uint4(w[0], w[1], w[2], w[3]);
@@ -344,16 +379,16 @@ int grid_for(const Ctx& c, int n, int block) {
 // singularity |a1| = 1 (N = sqrt(|a2|^2 + |a3|^2) below 1e-6); temporal links
 // of the temporal gauge off the last slice are never read.
 template <int P>
-__global__ void gauge_f64_to_8_kernel(Geom g, const double2* in, int nc, void* out, unsigned* nsing) {
+__global__ void gauge_f64_to_8_kernel(Geom g, const double2* in, int nc, bool fixed, void* out, unsigned* nsing) {
   const int n = 8 * g.Vh;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int pm = i / g.Vh, h = i - pm * g.Vh;
     const int parity = pm >> 2, mu = pm & 3;
     double2 r[6];
-    for (int c = 0; c < 6; ++c) r[c] = in[((size_t)pm * nc + c) * g.stride + h];
+    for (int c = 0; c < 6; ++c) r[c] = link_value(in[((size_t)pm * nc + c) * g.stride + h], fixed);
     double2 c1;
     if (nc == 9) {
-      c1 = in[((size_t)pm * nc + 6) * g.stride + h];
+      c1 = link_value(in[((size_t)pm * nc + 6) * g.stride + h], fixed);
     } else {  // c1 = conj(a2 b3 - a3 b2)
       const double re = r[1].x * r[5].x - r[1].y * r[5].y - (r[2].x * r[4].x - r[2].y * r[4].y);
       const double im = r[1].x * r[5].y + r[1].y * r[5].x - (r[2].x * r[4].y + r[2].y * r[4].x);
@@ -388,6 +423,7 @@ wd_status ensure_gauge(wd_ctx* ctx, int prec) {
   const size_t links = (size_t)8 * c.g.stride;
   const int nc = c.recon / 2;
   const double2* src = (const double2*)c.gauge[WD_F64];
+  const bool fx = c.gauge_fixed;
   const int grid = grid_for(c, 8 * c.g.Vh, 256);
   wd_status st;
   if (c.low_recon == 8 && prec != WD_F64) {
@@ -395,10 +431,10 @@ wd_status ensure_gauge(wd_ctx* ctx, int prec) {
     if ((st = dev_alloc(ctx, &c.gauge[prec], bytes)) != WD_OK) return st;
     unsigned* nsing = reinterpret_cast<unsigned*>(c.scalars);
     WD_CK(ctx, cudaMemsetAsync(nsing, 0, sizeof(unsigned), c.stream));
-    if (prec == WD_F32) gauge_f64_to_8_kernel<WD_F32><<<grid, 256, 0, c.stream>>>(c.g, src, nc, c.gauge[prec], nsing);
-    else if (prec == WD_Q16) gauge_f64_to_8_kernel<WD_Q16><<<grid, 256, 0, c.stream>>>(c.g, src, nc, c.gauge[prec], nsing);
-    else if (prec == WD_H16N) gauge_f64_to_8_kernel<WD_H16N><<<grid, 256, 0, c.stream>>>(c.g, src, nc, c.gauge[prec], nsing);
-    else gauge_f64_to_8_kernel<WD_B16N><<<grid, 256, 0, c.stream>>>(c.g, src, nc, c.gauge[prec], nsing);
+    if (prec == WD_F32) gauge_f64_to_8_kernel<WD_F32><<<grid, 256, 0, c.stream>>>(c.g, src, nc, fx, c.gauge[prec], nsing);
+    else if (prec == WD_Q16) gauge_f64_to_8_kernel<WD_Q16><<<grid, 256, 0, c.stream>>>(c.g, src, nc, fx, c.gauge[prec], nsing);
+    else if (prec == WD_H16N) gauge_f64_to_8_kernel<WD_H16N><<<grid, 256, 0, c.stream>>>(c.g, src, nc, fx, c.gauge[prec], nsing);
+    else gauge_f64_to_8_kernel<WD_B16N><<<grid, 256, 0, c.stream>>>(c.g, src, nc, fx, c.gauge[prec], nsing);
     WD_CK_LAUNCH(ctx, "gauge conversion (8 numbers)");
     unsigned h_nsing = 0;
     WD_CK(ctx, cudaMemcpyAsync(&h_nsing, nsing, sizeof(unsigned), cudaMemcpyDeviceToHost, c.stream));
@@ -413,15 +449,15 @@ wd_status ensure_gauge(wd_ctx* ctx, int prec) {
   }
   if (prec == WD_F32) {
     if ((st = dev_alloc(ctx, &c.gauge[prec], links * 3 * sizeof(float4))) != WD_OK) return st;
-    gauge_f64_to_f32_kernel<<<grid, 256, 0, c.stream>>>(c.g, src, nc, (float4*)c.gauge[prec]);
+    gauge_f64_to_f32_kernel<<<grid, 256, 0, c.stream>>>(c.g, src, nc, fx, (float4*)c.gauge[prec]);
   } else {
     if ((st = dev_alloc(ctx, &c.gauge[prec], links * sizeof(uint4))) != WD_OK) return st;
     if ((st = dev_alloc(ctx, &c.gauge4[prec], links * sizeof(uint2))) != WD_OK) return st;
     uint4* o8 = (uint4*)c.gauge[prec];
     uint2* o4 = (uint2*)c.gauge4[prec];
-    if (prec == WD_Q16) gauge_f64_to_16_kernel<Fmt16::Q16><<<grid, 256, 0, c.stream>>>(c.g, src, nc, o8, o4);
-    else if (prec == WD_H16N) gauge_f64_to_16_kernel<Fmt16::H16><<<grid, 256, 0, c.stream>>>(c.g, src, nc, o8, o4);
-    else gauge_f64_to_16_kernel<Fmt16::B16><<<grid, 256, 0, c.stream>>>(c.g, src, nc, o8, o4);
+    if (prec == WD_Q16) gauge_f64_to_16_kernel<Fmt16::Q16><<<grid, 256, 0, c.stream>>>(c.g, src, nc, fx, o8, o4);
+    else if (prec == WD_H16N) gauge_f64_to_16_kernel<Fmt16::H16><<<grid, 256, 0, c.stream>>>(c.g, src, nc, fx, o8, o4);
+    else gauge_f64_to_16_kernel<Fmt16::B16><<<grid, 256, 0, c.stream>>>(c.g, src, nc, fx, o8, o4);
   }
   WD_CK_LAUNCH(ctx, "gauge conversion");
   return WD_OK;
@@ -611,12 +647,11 @@ wd_status solve_device(wd_ctx* ctx, void* x_full, const void* b_full, double kap
     // kept in the FP64 residual buffer, which BiCGstab does not use otherwise
     using T64 = Tr<WD_F64>;
     WD_CK(ctx, cudaMemcpyAsync(sb.x, x_e, f64, cudaMemcpyDeviceToDevice, s));
-    EpiStore<SpinorF64> e0{T64::view(sb.tmp64, c.g)};
-    launch_dslash<double>(c, T64::view(sb.x, c.g), T64::gauge(c), 1, 0, e0, s);
+    o64->dslash(c, sb.tmp64, sb.x, 1, 0, s);
     EpiResid<SpinorF64, SpinorF64, SpinorF64, FinStore> e1{T64::view(sb.r, c.g), true, T64::view(sb.b_hat, c.g),
                                                            T64::view(sb.x, c.g), Coef{-kappa * kappa, nullptr},
                                                            c.red, FinStore{c.scalars + 6, 1}};
-    launch_dslash<double>(c, T64::view(sb.tmp64, c.g), T64::gauge(c), 0, 0, e1, s);
+    launch_dslash<double>(c, T64::view(sb.tmp64, c.g), T64::gauge(c), 0, kPlain, e1, s);
     setup_src = sb.r;
   } else {
     o64->zero(c, sb.x, s);
@@ -690,11 +725,11 @@ wd_status solve_device(wd_ctx* ctx, void* x_full, const void* b_full, double kap
     using T64 = Tr<WD_F64>;
     EpiReconResid<FinStore> eo{T64::view(x_o, c.g), T64::view(b_o, c.g), Coef{kappa, nullptr}, c.red,
                                FinStore{c.scalars + 5, 1}};
-    launch_dslash<double>(c, T64::view(x_e, c.g), T64::gauge(c), 1, 0, eo, s);
+    launch_dslash<double>(c, T64::view(x_e, c.g), T64::gauge(c), 1, kPlain, eo, s);
     const Coef ck{-kappa, nullptr};
     EpiResid<SpinorF64, SpinorF64, SpinorF64, FinStore> ee{T64::view(nullptr, c.g), false, T64::view(b_e, c.g),
                                                            T64::view(x_e, c.g), ck, c.red, FinStore{c.scalars + 4, 1}};
-    launch_dslash<double>(c, T64::view(x_o, c.g), T64::gauge(c), 0, 0, ee, s);
+    launch_dslash<double>(c, T64::view(x_o, c.g), T64::gauge(c), 0, kPlain, ee, s);
   }
   WD_CK_LAUNCH(ctx, "reconstruction");
   WD_CK(ctx, cudaMemcpyAsync(&hc, sb.ctl, sizeof(hc), cudaMemcpyDeviceToHost, s));
@@ -949,10 +984,23 @@ wd_status wd_load_gauge_opt(wd_ctx* ctx, const double* U, int is_device, int rec
   const int nc = recon / 2;
   if (st == WD_OK) st = dev_alloc(ctx, &c.gauge[WD_F64], (size_t)8 * nc * c.g.stride * sizeof(double2));
   if (st == WD_OK) {
-    gauge_pack_f64_kernel<<<grid_for(c, 2 * c.g.Vh, 256), 256, 0, c.stream>>>(c.g, src, (double2*)c.gauge[WD_F64],
-                                                                               nc);
-    cudaError_t e = cudaGetLastError();
+    // fixed-point links; a field with an element above kFixedLinkMax (not
+    // SU(3)) or not finite is packed again as doubles
+    unsigned* nbad = reinterpret_cast<unsigned*>(c.scalars);
+    unsigned h_nbad = 0;
+    const int grid = grid_for(c, 2 * c.g.Vh, 256);
+    cudaError_t e = cudaMemsetAsync(nbad, 0, sizeof(unsigned), c.stream);
+    gauge_pack_f64_kernel<<<grid, 256, 0, c.stream>>>(c.g, src, (double2*)c.gauge[WD_F64], nc, nbad);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(&h_nbad, nbad, sizeof(unsigned), cudaMemcpyDeviceToHost, c.stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c.stream);
+    c.gauge_fixed = h_nbad == 0;
+    if (e == cudaSuccess && h_nbad) {
+      gauge_pack_f64_kernel<<<grid, 256, 0, c.stream>>>(c.g, src, (double2*)c.gauge[WD_F64], nc, nullptr);
+      e = cudaGetLastError();
+      if (e == cudaSuccess) e = cudaStreamSynchronize(c.stream);
+    }
     if (e != cudaSuccess) st = cuda_err(ctx, e, "gauge pack");
   }
   if (staging) cudaFree(staging);

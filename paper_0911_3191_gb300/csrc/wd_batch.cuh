@@ -50,19 +50,6 @@ __device__ __forceinline__ bool rhs_active(const BatchArgs& a, int r) {
   return !c->done && (a.mode == 0 || c->do_update);
 }
 
-// even-odd indices of the 8 neighbours of site h (forward, backward per mu)
-__device__ __forceinline__ void neighbours(const Geom& g, int h, int x, int y, int z, int t, int (&nb)[8]) {
-  const int xo = x & 1;
-  nb[0] = (x == g.X - 1) ? h - (g.Xh - 1) : h + xo;
-  nb[1] = (x == 0) ? h + (g.Xh - 1) : h - (xo ^ 1);
-  nb[2] = (y == g.Y - 1) ? h - g.wy : h + g.Xh;
-  nb[3] = (y == 0) ? h + g.wy : h - g.Xh;
-  nb[4] = (z == g.Z - 1) ? h - g.wz : h + g.XhY;
-  nb[5] = (z == 0) ? h + g.wz : h - g.XhY;
-  nb[6] = (t == g.T - 1) ? h - g.wt : h + g.XhYZ;
-  nb[7] = (t == 0) ? h + g.wt : h - g.XhYZ;
-}
-
 // one hop with the link taken from the shared-memory tile (column sx)
 template <int MU, bool FWD, bool DAGGER, typename R, class In>
 __device__ __forceinline__ void hop_tile(const In& in, const R* lk, int sx, int h_nbr, bool flip, R (&acc)[24]) {
@@ -502,12 +489,7 @@ __global__ void __launch_bounds__(kDslashBlock, (DslashOccupancy<R, In, Epi::NRE
   double red[NR];
 #pragma unroll
   for (int k = 0; k < NR; ++k) red[k] = 0.0;
-  for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < g.Vh; h += gridDim.x * blockDim.x) {
-    R acc[24];
-    if constexpr (UseAsync<In, R8>::value) dslash_site_async<DAGGER, TFIX>(g, v, gauge, h, parity, acc);
-    else dslash_site<DAGGER, TFIX, R8, Epi::NRED == 0>(g, v, gauge, h, parity, acc);
-    e(h, acc, red);
-  }
+  dslash_sites<DAGGER, TFIX, R8>(g, v, gauge, 0, g.Vh, parity, e, red);
   if constexpr (Epi::NRED > 0) {
     __shared__ double sm[32][NR];
     block_sum<NR>(red, sm);
@@ -610,11 +592,16 @@ inline int mrhs_grid(const BatchLaunch& bl) {
   return (sizeof(R) == 8 && bl.grid64 > 0) ? bl.grid64 : bl.grid;
 }
 
-template <typename R, class In, class G, class Epi>
-void launch_dslash_mrhs(const Geom& g, const BatchLaunch& bl, const In& in, const G& gauge, int parity, int dagger,
+template <typename R, class In, class G, class Dag, class Epi>
+void launch_dslash_mrhs(const Geom& g, const BatchLaunch& bl, const In& in, const G& gauge, int parity, Dag dagger,
                         const Epi& epi, const BatchArgs& ba, cudaStream_t s) {
-  constexpr int NR = Epi::NRED > 0 ? Epi::NRED : 1;
-  const size_t smem = tile_link_bytes<R>() + (size_t)bl.nrhs * NR * sizeof(double);
+  if constexpr (std::is_same<G, GaugeF64>::value) {
+    if (gauge.fixed) {
+      launch_dslash_mrhs<R>(g, bl, in, GaugeX64{(const int4*)gauge.p, gauge.stride, gauge.recon}, parity, dagger, epi,
+                            ba, s);
+      return;
+    }
+  }
   const int grid = mrhs_grid<R>(bl);
   if (sizeof(R) == 8 || bl.tr == 0) {
     const dim3 gr(grid, bl.nrhs);
@@ -622,57 +609,50 @@ void launch_dslash_mrhs(const Geom& g, const BatchLaunch& bl, const In& in, cons
       launch_pdl(dslash_rhs_kernel<decltype(dag)::value, decltype(tfix)::value, decltype(rec8)::value, R, In, G, Epi>,
                  gr, dim3(kDslashBlock), 0, s, g, in, gauge, parity, epi, ba);
     };
-    using T_ = std::true_type;
-    using F_ = std::false_type;
-    if constexpr (sizeof(R) == 4) {
-      if (gauge.recon == 8) {
-        if (g.tfix) dagger ? go(T_{}, T_{}, T_{}) : go(F_{}, T_{}, T_{});
-        else dagger ? go(T_{}, F_{}, T_{}) : go(F_{}, F_{}, T_{});
-        return;
+    pick_dagger(dagger, [&](auto dag) {
+      using T_ = std::true_type;
+      using F_ = std::false_type;
+      if constexpr (sizeof(R) == 4) {
+        if (gauge.recon == 8) {
+          if (g.tfix) go(dag, T_{}, T_{});
+          else go(dag, F_{}, T_{});
+          return;
+        }
       }
-    }
-    if (g.tfix) dagger ? go(T_{}, T_{}, F_{}) : go(F_{}, T_{}, F_{});
-    else dagger ? go(T_{}, F_{}, F_{}) : go(F_{}, F_{}, F_{});
+      if (g.tfix) go(dag, T_{}, F_{});
+      else go(dag, F_{}, F_{});
+    });
     return;
   }
-  const int tr = bl.tr;
-  if constexpr (sizeof(R) == 4) {
-    if (bl.pack) {
-      const size_t smem2 = tile_link_bytes2<R>() + (size_t)bl.nrhs * NR * sizeof(double);
-#define WD_MRHS2_CASE(TRV)                                                                                  \
-  case TRV:                                                                                                 \
-    if (dagger)                                                                                             \
-      launch_pdl(dslash_mrhs2_kernel<true, In, G, Epi, TRV / 2>, dim3(grid), dim3(32, TRV / 2), smem2, s, g, \
-                 in, gauge, parity, epi, ba);                                                               \
-    else                                                                                                    \
-      launch_pdl(dslash_mrhs2_kernel<false, In, G, Epi, TRV / 2>, dim3(grid), dim3(32, TRV / 2), smem2, s,   \
-                 g, in, gauge, parity, epi, ba);                                                            \
-    break;
-      switch (tr) {
-        WD_MRHS2_CASE(2)
-        WD_MRHS2_CASE(4)
-        WD_MRHS2_CASE(8)
+  if constexpr (sizeof(R) == 4) {  // FP64 has returned above
+    constexpr int NR = Epi::NRED > 0 ? Epi::NRED : 1;
+    const size_t smem = tile_link_bytes<R>() + (size_t)bl.nrhs * NR * sizeof(double);
+    const int tr = bl.tr;
+    pick_dagger(dagger, [&](auto dag) {
+      constexpr bool kDag = decltype(dag)::value;
+      if (bl.pack) {
+        const size_t smem2 = tile_link_bytes2<R>() + (size_t)bl.nrhs * NR * sizeof(double);
+        auto go2 = [&](auto tp) {
+          constexpr int TP = decltype(tp)::value;
+          launch_pdl(dslash_mrhs2_kernel<kDag, In, G, Epi, TP>, dim3(grid), dim3(32, TP), smem2, s, g, in, gauge,
+                     parity, epi, ba);
+        };
+        if (tr == 2) go2(std::integral_constant<int, 1>{});
+        else if (tr == 4) go2(std::integral_constant<int, 2>{});
+        else if (tr == 8) go2(std::integral_constant<int, 4>{});
+        return;
       }
-#undef WD_MRHS2_CASE
-      return;
-    }
+      auto go1 = [&](auto trv) {
+        constexpr int TR = decltype(trv)::value;
+        launch_pdl(dslash_mrhs_kernel<kDag, R, In, G, Epi, TR>, dim3(grid), dim3(32, TR), smem, s, g, in, gauge,
+                   parity, epi, ba);
+      };
+      if (tr == 1) go1(std::integral_constant<int, 1>{});
+      else if (tr == 2) go1(std::integral_constant<int, 2>{});
+      else if (tr == 4) go1(std::integral_constant<int, 4>{});
+      else if (tr == 8) go1(std::integral_constant<int, 8>{});
+    });
   }
-#define WD_MRHS_CASE(TRV)                                                                                   \
-  case TRV:                                                                                                 \
-    if (dagger)                                                                                             \
-      launch_pdl(dslash_mrhs_kernel<true, R, In, G, Epi, TRV>, dim3(grid), dim3(32, TRV), smem, s, g, in,    \
-                 gauge, parity, epi, ba);                                                                   \
-    else                                                                                                    \
-      launch_pdl(dslash_mrhs_kernel<false, R, In, G, Epi, TRV>, dim3(grid), dim3(32, TRV), smem, s, g, in,   \
-                 gauge, parity, epi, ba);                                                                   \
-    break;
-  switch (tr) {
-    WD_MRHS_CASE(1)
-    WD_MRHS_CASE(2)
-    WD_MRHS_CASE(4)
-    WD_MRHS_CASE(8)
-  }
-#undef WD_MRHS_CASE
 }
 
 template <class Op>
@@ -720,6 +700,12 @@ struct ImplBatch {
     launch_dslash_mrhs<R>(c.g, bl, v(in, c.g), T::gauge(c), parity, dagger, e, ba, s);
   }
 
+  static void dslash_args(const Ctx& c, const BatchLaunch& bl, void* out, const void* in, int parity,
+                          const BatchArgs& ba, cudaStream_t s) {
+    EpiStore<S> e{v(out, c.g)};
+    launch_dslash_mrhs<R>(c.g, bl, v(in, c.g), T::gauge(c), parity, kPlain, e, ba, s);
+  }
+
   // ---- batched BiCGstab (Sec. 5.1) with Alg. 2 reliable updates; one
   // SolverCtl per system, all systems step together, converged ones masked
   static void setup(const Ctx& c, const BatchLaunch& bl, BatchBufs& b, cudaStream_t s) {
@@ -740,14 +726,14 @@ struct ImplBatch {
     const Coef nk2{0.0, &b.ctl->neg_kappa2, (long)(sizeof(SolverCtl) / sizeof(double))};
     launch_sites_batch(g, bl, OpBicgP<S>{v(b.r_hat, g), v(b.p, g), v(b.v, g), b.ctl}, ba, s);
     EpiStore<S> e0{v(b.tmp, g)};
-    launch_dslash_mrhs<R>(g, bl, v(b.p, g), T::gauge(c), 1, 0, e0, ba, s);
+    launch_dslash_mrhs<R>(g, bl, v(b.p, g), T::gauge(c), 1, kPlain, e0, ba, s);
     EpiXpayDot<S, S, S, FinBicgAlpha> e1{v(b.v, g), v(b.p, g), v(b.r_tilde, g), nk2, c.red, FinBicgAlpha{b.ctl}};
-    launch_dslash_mrhs<R>(g, bl, v(b.tmp, g), T::gauge(c), 0, 0, e1, ba, s);
+    launch_dslash_mrhs<R>(g, bl, v(b.tmp, g), T::gauge(c), 0, kPlain, e1, ba, s);
     launch_finalize<2>(bl, ba, mrhs_grid<R>(bl), FinBicgAlpha{b.ctl}, b.bc, 0, 0, s);
     launch_sites_batch(g, bl, OpBicgS<S>{v(b.r_hat, g), v(b.v, g), b.ctl}, ba, s);
-    launch_dslash_mrhs<R>(g, bl, v(b.r_hat, g), T::gauge(c), 1, 0, e0, ba, s);
+    launch_dslash_mrhs<R>(g, bl, v(b.r_hat, g), T::gauge(c), 1, kPlain, e0, ba, s);
     EpiXpayTS<S, S, FinBicgOmega> e2{v(b.t, g), v(b.r_hat, g), nk2, c.red, FinBicgOmega{b.ctl}};
-    launch_dslash_mrhs<R>(g, bl, v(b.tmp, g), T::gauge(c), 0, 0, e2, ba, s);
+    launch_dslash_mrhs<R>(g, bl, v(b.tmp, g), T::gauge(c), 0, kPlain, e2, ba, s);
     launch_finalize<3>(bl, ba, mrhs_grid<R>(bl), FinBicgOmega{b.ctl}, b.bc, 1, 0, s);
     OpBicgFinal<S> fo{v(b.x_hat, g), v(b.p, g), v(b.r_hat, g), v(b.t, g), v(b.r_tilde, g), b.ctl, c.red,
                       FinBicgIter{b.ctl}};
@@ -761,11 +747,10 @@ struct ImplBatch {
     BatchArgs ba{bl.nrhs, b.ctl, 1, b.partials, b.bc};
     const Coef nk2{0.0, &b.ctl->neg_kappa2, (long)(sizeof(SolverCtl) / sizeof(double))};
     launch_sites_batch(g, bl, OpAccumulate<S>{v64(b.xe, g, fb64(g)), v(b.x_hat, g)}, ba, s);
-    EpiStore<SpinorF64> e0{v64(b.tmp64, g, fb64(g))};
-    launch_dslash_mrhs<double>(g, bl, v64(b.xe, g, fb64(g)), T64::gauge(c), 1, 0, e0, ba, s);
+    ops_f64()->dslash_batch_args(c, bl, b.tmp64, b.xe, 1, ba, s);
     EpiRelupBicg<S, S, FinRelupBicg> e1{v64(b.b_hat, g, fb64(g)), v64(b.xe, g, fb64(g)), v(b.r_hat, g),
                                         v(b.r_tilde, g), nk2, c.red, FinRelupBicg{b.ctl}};
-    launch_dslash_mrhs<double>(g, bl, v64(b.tmp64, g, fb64(g)), T64::gauge(c), 0, 0, e1, ba, s);
+    launch_dslash_mrhs<double>(g, bl, v64(b.tmp64, g, fb64(g)), T64::gauge(c), 0, kPlain, e1, ba, s);
     launch_finalize<4>(bl, ba, mrhs_grid<double>(bl), FinRelupBicg{b.ctl}, b.bc, 3, 0, s);
   }
 };

@@ -1,0 +1,492 @@
+// The FP64 dslash of one site in block fixed point, on the integer pipe.
+//
+// An SM quarter of GB300 takes one FP64 warp instruction every 67 cycles
+// (measured), but a 32 x 32 + 64-bit integer multiply-add every 4.2 and an
+// integer add, logic or shift instruction every 2.4.  The FP64 stencil takes 614
+// FP64 instructions a site and is bound by that pipe alone.  Here every number of
+// a hop is a 64-bit integer, a product of two takes three integer multiply-adds,
+// and nothing is rounded more coarsely than in FP64.  24^3 x 64, temporal gauge,
+// 18 reals: 471 -> 145 us a dslash (its bytes take 81 us); 12-real general links
+// of 20 x 14 x 22 x 38, M_hat: 459 -> 129 us; 8^3 x 16: 27 -> 14 us.  What bounds
+// it now is the issue of 6100 integer instructions per 32 sites: the multiplier
+// is 59 % busy and the other integer pipe 45 %, which add up rather than overlap.
+//
+//  * A link element u, |u| <= 1, is the integer u 2^60 (converted once, when
+//    the links are loaded).  A double of at least 2^-8 is exact in it, a
+//    smaller one is off by at most 2^-61.
+//  * The spinors of a site's neighbours share one exponent E (|x| < 2^(E-1023)
+//    for all of their components): x is the integer x 2^(59-(E-1023)), so a
+//    projected component, a sum of two, is below 2^60.
+//  * Both are kept as two signed 32-bit limbs, a = ah 2^32 + al with al in
+//    [-2^31, 2^31).  Of a product's limbs ah bh, (ah bl + al bh) 2^-32 and
+//    al bl 2^-64, the last is left out: at most a quarter of the unit 2^(E-1078)
+//    in which the sums are kept.
+//  * The 24 sums are 64-bit integers of that unit, 2^-55 of the largest
+//    neighbour component, where FP64 rounds every partial sum at 2^-53 of
+//    itself.  They are rounded once, to the double they become.
+//
+// E is known only when all neighbours are, so it is a running maximum: a hop
+// that raises it shifts the sums down.  Starting one above the first hop's
+// exponent makes that rare.  Sums cannot overflow: with |u| <= 1.125 (the rule
+// by which links take this form, kFixedLinkMax) each of the eight hops adds at
+// most 6 x 1.125 x 2^56, and a middle sum stays below 12 x 1.125 x 2^59.
+//
+// Sites whose neighbours hold an infinity, a NaN, or only numbers outside
+// 2^-830 .. 2^870 are computed by dslash_site in FP64 as before.
+#pragma once
+
+#include "wd_async.cuh"
+#include "wd_device.cuh"
+
+namespace wd {
+
+constexpr int kFixedMinExp = 192, kFixedMaxExp = 1892;  // biased exponents E of the fixed-point path
+
+struct Fx {
+  int h, l;  // h * 2^32 + l
+};
+
+__device__ __forceinline__ Fx fx_split(long long v) {
+  const unsigned lo = (unsigned)v;
+  return Fx{(int)(v >> 32) + (int)(lo >> 31), (int)lo};
+}
+__device__ __forceinline__ long long fx_join(Fx a) { return ((long long)a.h << 32) + a.l; }
+// a b + c.  The product is opaque to the compiler's algebra, which would split
+// one with a negated factor; with the sum left to it, the two become one
+// multiply-add (a mad.wide in its place took 0.7 more instructions)
+__device__ __forceinline__ long long fx_mad(int a, int b, long long c) {
+  long long p;
+  asm("mul.wide.s32 %0, %1, %2;" : "=l"(p) : "r"(a), "r"(b));
+  return c + p;
+}
+
+// shifts that give 0 (or the sign) for any count of 64 and more
+__device__ __forceinline__ unsigned long long fx_shr(unsigned long long v, int s) {
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));
+  return r;
+}
+__device__ __forceinline__ long long fx_sar(long long v, int s) {
+  long long r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));
+  return r;
+}
+
+// v 2^e by the conversion of the FP64 pipe (otherwise idle here) and an
+// addition to its exponent
+__device__ __forceinline__ double fx_sum_value(long long v, int e) {
+  const double d = __ll2double_rn(v);
+  const int hi = __double2hiint(d);
+  return __hiloint2double(hi ? hi + (e << 20) : 0, __double2loint(d));
+}
+
+// The FP64 links in this form: the words of GaugeF64, each double replaced by
+// its two limbs (h first).
+struct GaugeX64 {
+  using real = double;
+  static constexpr bool kScaled = false;
+  const int4* p;
+  int stride;
+  int recon;
+  __device__ __forceinline__ GaugeF64 f64() const { return GaugeF64{(const double2*)p, stride, recon, true}; }
+};
+
+// Staging of one hop per thread, as in wd_async.cuh: the neighbour's spinor and
+// the link, each refilled by cp.async for the next hop as soon as this hop has
+// read it (the spinor while the SU(3) product runs, the link while the next
+// spinor is converted), so the loads hold no registers.
+constexpr int kFixedBlock = 128;
+struct FixedSlots {
+  uint4 sp[12][kFixedBlock];
+  int4 lk[9][kFixedBlock];
+};
+
+// a b + c d - e f - g q of link elements, as a link element
+__device__ __forceinline__ long long fx_minor(Fx a, Fx b, Fx c, Fx d, Fx e, Fx f, Fx g, Fx q) {
+  long long hp = fx_mad(a.h, b.h, 0), mp = fx_mad(a.h, b.l, 1ll << 27);
+  mp = fx_mad(a.l, b.h, mp);
+  hp = fx_mad(c.h, d.h, hp);
+  mp = fx_mad(c.h, d.l, mp);
+  mp = fx_mad(c.l, d.h, mp);
+  long long hq = fx_mad(e.h, f.h, 0), mq = fx_mad(e.h, f.l, 0);
+  mq = fx_mad(e.l, f.h, mq);
+  hq = fx_mad(g.h, q.h, hq);
+  mq = fx_mad(g.h, q.l, mq);
+  mq = fx_mad(g.l, q.h, mq);
+  return ((hp - hq) << 4) + ((mp - mq) >> 28);
+}
+
+// row c = (a x b)^* of a 12-real link, written to its slots
+__device__ __forceinline__ void fx_row3(FixedSlots& sm) {
+  const int tid = threadIdx.x;
+  Fx r[6], i[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const int4 w = sm.lk[c][tid];
+    r[c] = Fx{w.x, w.y};
+    i[c] = Fx{w.z, w.w};
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int j = (c + 1) % 3, k = (c + 2) % 3;
+    const Fx re = fx_split(fx_minor(r[j], r[3 + k], i[k], i[3 + j], i[j], i[3 + k], r[k], r[3 + j]));
+    const Fx im = fx_split(fx_minor(r[k], i[3 + j], i[k], r[3 + j], r[j], i[3 + k], i[j], r[3 + k]));
+    sm.lk[6 + c][tid] = make_int4(re.h, re.l, im.h, im.l);
+  }
+}
+
+// The double (low word x, high word y) in the unit of the
+// common exponent, e4 = E + 4: |x| 2^(59-(E-1023)) cut to an integer, 0 for a
+// denormal or a zero, times the sign of x and of the mask `flip` (0 or -1).  A
+// negative number is the one's complement of its magnitude, one unit (2^-59 of
+// the largest component, a sixteenth of the unit of the sums) too low; a zero
+// stays zero in the sums, which round.
+__device__ __forceinline__ unsigned fx_xor3(unsigned a, unsigned b, unsigned c) {
+  unsigned r;
+  asm("lop3.b32 %0, %1, %2, %3, 0x96;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+  return r;
+}
+__device__ __forceinline__ long long fx_number(unsigned x, unsigned y, int e4, int flip) {
+  const int s = e4 - (int)((y >> 20) & 0x7ffu);
+  const unsigned mh = __funnelshift_l(x, y, 11) | 0x80000000u;
+  unsigned ml;  // x << 11 by the funnel shifter: the compiler's choice is the multiplier, which bounds the kernel
+  asm("shf.l.clamp.b32 %0, 0, %1, 11;" : "=r"(ml) : "r"(x));
+  const unsigned long long a = fx_shr(((unsigned long long)mh << 32) | ml, s);
+  const int m = (int)y >> 31;
+  const unsigned lo = fx_xor3((unsigned)a, m, flip), hi = fx_xor3((unsigned)(a >> 32), m, flip);
+  return (long long)(((unsigned long long)hi << 32) | lo);
+}
+
+// largest of m and |a|, |b| read as floats: the high words of doubles order like
+// floats, and an exponent above 2039 (infinities and NaN among them) reads as a
+// NaN, which stays
+__device__ __forceinline__ float fx_max(float m, unsigned a, unsigned b) {
+  float r;
+  asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(m), "f"(__uint_as_float(a)), "f"(__uint_as_float(b)));
+  return r;
+}
+// the biased exponent of the double whose high word gave m, plus 1
+__device__ __forceinline__ int fx_exponent(float m) { return (int)(__float_as_uint(m) >> 20) + 1; }
+
+__device__ __forceinline__ int fixed_neighbour(const Geom& g, int h, int x, int y, int z, int t, int k) {
+  switch (k) {
+    case 0: return (x == g.X - 1) ? h - (g.Xh - 1) : h + (x & 1);
+    case 1: return (x == 0) ? h + (g.Xh - 1) : h - ((x & 1) ^ 1);
+    case 2: return (y == g.Y - 1) ? h - g.wy : h + g.Xh;
+    case 3: return (y == 0) ? h + g.wy : h - g.Xh;
+    case 4: return (z == g.Z - 1) ? h - g.wz : h + g.XhY;
+    case 5: return (z == 0) ? h + g.wz : h - g.XhY;
+    case 6: return (t == g.T - 1) ? h - g.wt : h + g.XhYZ;
+    default: return (t == 0) ? h + g.wt : h - g.XhYZ;
+  }
+}
+
+// copies of hop k: the neighbour's spinor (the half a temporal hop reads), and
+// the link (none for the unit links of the temporal gauge)
+template <bool DAGGER>
+__device__ __forceinline__ void fixed_issue_spinor(FixedSlots& sm, const SpinorF64& in, int n, int k) {
+  const int tid = threadIdx.x;
+  const bool lower = (k == 6) != DAGGER;  // the temporal hop's projector keeps spins 2, 3
+  const double2* p = in.p + (size_t)((k >= 6 && lower) ? 6 : 0) * in.stride + n;
+#pragma unroll
+  for (int c = 0; c < 6; ++c) cp16_cg(&sm.sp[c][tid], p + (size_t)c * in.stride);
+  if (k < 6) {
+#pragma unroll
+    for (int c = 6; c < 12; ++c) cp16_cg(&sm.sp[c][tid], p + (size_t)c * in.stride);
+  }
+}
+__device__ __forceinline__ void fixed_issue_link(FixedSlots& sm, const GaugeX64& gauge, int parity, int h, int n,
+                                                 int k) {
+  const int tid = threadIdx.x;
+  const int nc = gauge.recon >> 1;
+  const int slot = ((k & 1) ? 1 - parity : parity) * 4 + (k >> 1);
+  const int4* p = gauge.p + (size_t)slot * nc * gauge.stride + ((k & 1) ? n : h);
+  const uint64_t pol = l2_evict_first();
+#pragma unroll
+  for (int c = 0; c < 6; ++c) cp16_cg_ef(&sm.lk[c][tid], p + (size_t)c * gauge.stride, pol);
+  if (nc == 9) {
+#pragma unroll
+    for (int c = 6; c < 9; ++c) cp16_cg_ef(&sm.lk[c][tid], p + (size_t)c * gauge.stride, pol);
+  }
+}
+
+// reconstruct() of row s: the upper row s of a hop, and the lower row that the
+// projector makes of it.  CONJ: the row is that of the conjugate (backward hops,
+// see dslash_site_fixed)
+template <int MU, int S_, bool CONJ, int ROW>
+__device__ __forceinline__ void fixed_add(const long long (&gr)[3], const long long (&gi)[3], long long (&a)[24]) {
+  constexpr int S = (MU == 1) ? -S_ : S_;
+  constexpr int up = (MU == 3 && S_ < 0) ? 12 + 6 * ROW : 6 * ROW;
+  constexpr int lo = (MU == 2) ? 12 + 6 * ROW : 18 - 6 * ROW;
+  // lower row = t g (y) or t i g (x, z): x: -S for both rows, y: -S, S, z: -S, S
+  constexpr int t = (MU == 0 || ROW == 0) ? -S : S;
+  constexpr int ci = CONJ ? -1 : 1;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    a[up + 2 * c] += gr[c];
+    a[up + 2 * c + 1] += ci * gi[c];
+    if constexpr (MU == 1) {
+      a[lo + 2 * c] += t * gr[c];
+      a[lo + 2 * c + 1] += t * ci * gi[c];
+    } else if constexpr (MU != 3) {
+      a[lo + 2 * c] += -t * ci * gi[c];
+      a[lo + 2 * c + 1] += t * gr[c];
+    }
+  }
+}
+
+// A site whose neighbours are zero (false: its sums are right), or hold numbers
+// the fixed-point form does not take (out = (D in)(h) in FP64).  Not inlined:
+// the FP64 arithmetic would be in every kernel that has the fixed-point one.
+template <bool DAGGER, bool TFIX, bool PAIR>
+__device__ __noinline__ bool dslash_site_outside(Geom g, SpinorF64 in, GaugeX64 gauge, int h,
+                                                 int parity, int top, double (&out)[24]) {
+  if (top < kFixedMinExp) {
+    int x, y, z, t;
+    site_coords(g, h, parity, x, y, z, t);
+    int nb[8];
+    neighbours(g, h, x, y, z, t, nb);
+    unsigned long long any = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+#pragma unroll 1
+      for (int c = 0; c < 12; ++c) {
+        const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(in.p + (size_t)c * in.stride + nb[k]));
+        any |= (v.x | v.y) & 0x7fffffffffffffffull;
+      }
+    if (any == 0) return false;
+  }
+  dslash_site<DAGGER, TFIX, false, PAIR>(g, in, gauge.f64(), h, parity, out);
+  return true;
+}
+
+// U h: the limbs of the two rows of h, the link in its slots read by rows (step
+// 3, 1) or columns (1, 3); g in the unit of the sums
+__device__ __forceinline__ void fixed_su3(const FixedSlots& sm, int step_i, int step_j, const long long (&hr)[2][3],
+                                          const long long (&hi)[2][3], long long (&gr)[2][3], long long (&gi)[2][3]) {
+  const int tid = threadIdx.x;
+  Fx r[2][3], i[2][3], ni[2][3];
+#pragma unroll
+  for (int s = 0; s < 2; ++s)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      r[s][j] = fx_split(hr[s][j]);
+      i[s][j] = fx_split(hi[s][j]);
+      ni[s][j] = Fx{-i[s][j].h, ~i[s][j].l};  // -hi, one unit of 2^-59 low
+    }
+  const long long half = 1ll << 31;  // the middle sums are rounded to their high words
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    long long rh[2], ih[2], rm[2], im[2];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int4 w = sm.lk[c * step_i + j * step_j][tid];
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        rh[s] = fx_mad(w.x, r[s][j].h, j ? rh[s] : 0);
+        rm[s] = fx_mad(w.x, r[s][j].l, j ? rm[s] : half);
+        ih[s] = fx_mad(w.x, i[s][j].h, j ? ih[s] : 0);
+        im[s] = fx_mad(w.x, i[s][j].l, j ? im[s] : half);
+      }
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        rm[s] = fx_mad(w.y, r[s][j].h, rm[s]);
+        im[s] = fx_mad(w.y, i[s][j].h, im[s]);
+        rh[s] = fx_mad(w.z, ni[s][j].h, rh[s]);
+        ih[s] = fx_mad(w.z, r[s][j].h, ih[s]);
+      }
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        rm[s] = fx_mad(w.z, ni[s][j].l, rm[s]);
+        im[s] = fx_mad(w.z, r[s][j].l, im[s]);
+        rm[s] = fx_mad(w.w, ni[s][j].h, rm[s]);
+        im[s] = fx_mad(w.w, r[s][j].h, im[s]);
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      gr[s][c] = rh[s] + (int)(rm[s] >> 32);
+      gi[s][c] = ih[s] + (int)(im[s] >> 32);
+    }
+  }
+}
+
+// the sums move to the exponent of a hop that needs a larger one
+__device__ __forceinline__ void fixed_raise(float m, int& E, int& top, long long (&acc)[24]) {
+  const int e = fx_exponent(m);
+  top = max(top, e);
+  if (e > E) {
+#pragma unroll
+    for (int q = 0; q < 24; ++q) acc[q] = fx_sar(acc[q], e - E);
+    E = e;
+  }
+}
+
+// dslash_site in fixed point.  Two loops, over the six spatial and the two
+// temporal hops: unrolled, a site is 7600 instructions that the instruction
+// caches do not hold, and the warps wait for instructions longer than for
+// anything else.  The directions differ in which lower spin row joins which
+// upper one (a choice of slots), in signs (masks of the conversion) and in the
+// rows that the sums go to (a branch that all threads take alike).
+//
+// A backward hop takes U^dag h as the conjugate of U^T h^*: the same product
+// with the link read by columns, the projection's imaginary parts negated as
+// they are converted, and the result's as they are added.
+template <bool DAGGER, bool TFIX, bool PAIR>
+__device__ __forceinline__ void dslash_site_fixed(const Geom& g, const SpinorF64& in, const GaugeX64& gauge, int h,
+                                                  int parity, double (&out)[24]) {
+  __shared__ FixedSlots sm;
+  constexpr int SF = DAGGER ? +1 : -1;  // the projector sign of the forward hops
+  const int tid = threadIdx.x;
+  int x, y, z, t;
+  site_coords(g, h, parity, x, y, z, t);
+  const bool last = (t == g.T - 1), first = (t == 0);
+  long long acc[24];
+#pragma unroll
+  for (int k = 0; k < 24; ++k) acc[k] = 0;
+  int E = kFixedMinExp, top = 0;
+  int n = fixed_neighbour(g, h, x, y, z, t, 0);
+  fixed_issue_spinor<DAGGER>(sm, in, n, 0);
+  cp_commit();
+  fixed_issue_link(sm, gauge, parity, h, n, 0);
+  cp_commit();
+#pragma unroll 1
+  for (int k = 0; k < 6; ++k) {
+    const int mu = k >> 1;
+    const bool fwd = (k & 1) == 0;
+    cp_wait<1>();  // the spinor of hop k
+    {
+      float m = 0.f;
+#pragma unroll
+      for (int c = 0; c < 12; ++c) {
+        const uint4 w = sm.sp[c][tid];
+        m = fx_max(m, w.y, w.w);
+      }
+      if (k == 0) E = max(fx_exponent(m), kFixedMinExp) + 1;
+      fixed_raise(m, E, top, acc);
+    }
+    // rows 0, 1 and their partners: row 0 joins spin 3 (x, y) or 2 (z), row 1
+    // the other; a real part joins a real one (y) or an imaginary one (x, z)
+    const uint2* p = reinterpret_cast<const uint2*>(&sm.sp[0][tid]);
+    const int qr = (mu == 1) ? 0 : 1, qi = 1 - qr;
+    // sign masks.  cj: imaginary parts of a backward hop; sp: the sign S of the
+    // projector; x: h0 = p0 + S i p3, h1 = p1 + S i p2; y: h0 = p0 + S p3,
+    // h1 = p1 - S p2; z: h0 = p0 + S i p2, h1 = p1 - S i p3
+    const int cj = fwd ? 0 : -1;
+    const int sp = (fwd != DAGGER) ? -1 : 0;
+    const int e4 = E + 4;
+    const int step_i = fwd ? 3 : 1, step_j = fwd ? 1 : 3;
+    long long hr[2][3], hi[2][3];
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+      const int q = ((mu == 2) == (s == 1) ? 9 : 6) * (2 * kFixedBlock);
+      const int fr = s ? ((mu == 2) ? sp : ~sp) : ((mu == 1) ? sp : ~sp);
+      const int fi = (s && mu != 0) ? ~sp ^ cj : sp ^ cj;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const uint4 w = sm.sp[3 * s + c][tid];
+        const uint2 vr = p[q + c * 2 * kFixedBlock + qr], vi = p[q + c * 2 * kFixedBlock + qi];
+        hr[s][c] = fx_number(w.x, w.y, e4, 0) + fx_number(vr.x, vr.y, e4, fr);
+        hi[s][c] = fx_number(w.z, w.w, e4, cj) + fx_number(vi.x, vi.y, e4, fi);
+      }
+    }
+    // the next hop's spinor takes the slots just read
+    const int nn = fixed_neighbour(g, h, x, y, z, t, k + 1);
+    fixed_issue_spinor<DAGGER>(sm, in, nn, k + 1);
+    cp_commit();
+    cp_wait<1>();  // the link of hop k
+    if (gauge.recon == 12) fx_row3(sm);
+    long long gr[2][3], gi[2][3];
+    fixed_su3(sm, step_i, step_j, hr, hi, gr, gi);
+    if (!(TFIX && k == 5 && !last)) fixed_issue_link(sm, gauge, parity, h, nn, k + 1);
+    cp_commit();
+#define WD_FIXED_ADD(MU, S, CONJ)                          \
+  fixed_add<MU, S, CONJ, 0>(gr[0], gi[0], acc);            \
+  fixed_add<MU, S, CONJ, 1>(gr[1], gi[1], acc)
+    switch (k) {
+      case 0: WD_FIXED_ADD(0, SF, false); break;
+      case 1: WD_FIXED_ADD(0, -SF, true); break;
+      case 2: WD_FIXED_ADD(1, SF, false); break;
+      case 3: WD_FIXED_ADD(1, -SF, true); break;
+      case 4: WD_FIXED_ADD(2, SF, false); break;
+      default: WD_FIXED_ADD(2, -SF, true); break;
+    }
+  }
+#pragma unroll 1
+  for (int k = 6; k < 8; ++k) {
+    const bool fwd = k == 6;
+    cp_wait<1>();
+    {
+      float m = 0.f;
+#pragma unroll
+      for (int c = 0; c < 6; ++c) {
+        const uint4 w = sm.sp[c][tid];
+        m = fx_max(m, w.y, w.w);
+      }
+      fixed_raise(m, E, top, acc);
+    }
+    const bool unit = TFIX && (fwd ? !last : !first);
+    const int fm = (g.tbc_anti && (fwd ? last : first)) ? -1 : 0;
+    const int cj = (fwd || unit) ? fm : ~fm;
+    long long hr[2][3], hi[2][3];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {  // twice the component: the projector is 2
+      const uint4 w = sm.sp[q][tid];
+      hr[q / 3][q % 3] = fx_number(w.x, w.y, E + 3, fm);
+      hi[q / 3][q % 3] = fx_number(w.z, w.w, E + 3, cj);
+    }
+    int nn = 0;
+    if (fwd) {
+      nn = fixed_neighbour(g, h, x, y, z, t, 7);
+      fixed_issue_spinor<DAGGER>(sm, in, nn, 7);
+    }
+    cp_commit();
+    cp_wait<1>();
+    long long gr[2][3], gi[2][3];
+    if (unit) {
+#pragma unroll
+      for (int q = 0; q < 6; ++q) {
+        gr[q / 3][q % 3] = (hr[q / 3][q % 3] + 8) >> 4;
+        gi[q / 3][q % 3] = (hi[q / 3][q % 3] + 8) >> 4;
+      }
+    } else {
+      if (gauge.recon == 12) fx_row3(sm);
+      fixed_su3(sm, fwd ? 3 : 1, fwd ? 1 : 3, hr, hi, gr, gi);
+      if (!fwd) {
+#pragma unroll
+        for (int q = 0; q < 6; ++q) gi[q / 3][q % 3] = -gi[q / 3][q % 3];
+      }
+    }
+    if (fwd && !(TFIX && !first)) fixed_issue_link(sm, gauge, parity, h, nn, 7);
+    cp_commit();
+    if (fwd) {
+      WD_FIXED_ADD(3, SF, false);
+    } else {
+      WD_FIXED_ADD(3, -SF, false);
+    }
+  }
+#undef WD_FIXED_ADD
+  if (top < kFixedMinExp || top > kFixedMaxExp) {
+    double slow[24];  // its address is taken on this path only
+    if (dslash_site_outside<DAGGER, TFIX, PAIR>(g, in, gauge, h, parity, top, slow)) {
+#pragma unroll
+      for (int k = 0; k < 24; ++k) out[k] = slow[k];
+      return;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 24; ++k) out[k] = fx_sum_value(acc[k], E - 1078);
+}
+
+// epi on (D in)(h) for the sites [h_begin, h_end) of a launch
+template <bool DAGGER, bool TFIX, class Epi>
+__device__ __forceinline__ void dslash_sites_fixed(const Geom& g, const SpinorF64& in, const GaugeX64& gauge,
+                                                   int h_begin, int h_end, int parity, const Epi& epi, double* red) {
+  for (int h = h_begin + blockIdx.x * blockDim.x + threadIdx.x; h < h_end; h += gridDim.x * blockDim.x) {
+    double acc[24];
+    dslash_site_fixed<DAGGER, TFIX, Epi::NRED == 0>(g, in, gauge, h, parity, acc);
+    epi(h, acc, red);
+  }
+}
+
+}  // namespace wd

@@ -45,6 +45,7 @@ struct SolverCtl {
 struct Ctx;
 struct BatchLaunch;
 struct BatchBufs;
+struct BatchArgs;
 
 // Per-precision operations, one table per storage precision.
 struct PrecOps {
@@ -67,6 +68,10 @@ struct PrecOps {
   void (*bicg_update)(const Ctx&, struct SolveBufs&, cudaStream_t);
   // setup from the FP64 even residual src (b_hat, or b_hat - M_hat x0)
   void (*bicg_setup)(const Ctx&, struct SolveBufs&, const void* src, cudaStream_t);
+  // FP64 table only: the reliable updates' residual b_hat - M_hat x from
+  // tmp64 = D_oe x, stored rounded to FP32 (BiCGstab) or in FP64 (CG)
+  void (*resid_f32)(const Ctx&, struct SolveBufs&, cudaStream_t);
+  void (*resid_cg)(const Ctx&, struct SolveBufs&, cudaStream_t);
   // S7 CG on the normal equations, and its reliable update
   void (*cg_iteration)(const Ctx&, struct SolveBufs&, cudaStream_t);
   void (*cg_update)(const Ctx&, struct SolveBufs&, cudaStream_t);
@@ -74,6 +79,8 @@ struct PrecOps {
   // S11: multi-RHS dslash and the batched BiCGstab with this inner precision
   void (*dslash_batch)(const Ctx&, const BatchLaunch&, void* out, const void* in, int parity, int dagger,
                        cudaStream_t);
+  void (*dslash_batch_args)(const Ctx&, const BatchLaunch&, void* out, const void* in, int parity,
+                            const BatchArgs&, cudaStream_t);  // D, the systems named by the BatchArgs
   void (*batch_setup)(const Ctx&, const BatchLaunch&, BatchBufs&, cudaStream_t);
   void (*batch_iteration)(const Ctx&, const BatchLaunch&, BatchBufs&, cudaStream_t);
   void (*batch_update)(const Ctx&, const BatchLaunch&, BatchBufs&, cudaStream_t);
@@ -126,6 +133,7 @@ struct Ctx {
   void* gauge[5];       // by wd_prec: F64 double2; F32 float4; 16-bit: uint4 part
   void* gauge4[5];      // 16-bit: uint2 part
   bool gauge_loaded;
+  bool gauge_fixed;     // the FP64 copy holds fixed-point links (wd_fixed.cuh)
   // temporal gauge (wd_load_gauge_opt): G(x) as [parity][9][stride] double2,
   // or nullptr; c.g.tfix is set with it
   double2* gfix;

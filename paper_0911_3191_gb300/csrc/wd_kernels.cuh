@@ -14,6 +14,7 @@
 #include "wd_internal.h"
 #include "wd_slab.cuh"
 #include "wd_async.cuh"
+#include "wd_fixed.cuh"
 
 namespace wd {
 
@@ -590,6 +591,24 @@ struct UseAsync {
 };
 static_assert(kDslashBlock == kAsyncBlock, "the async slots are sized for the dslash block");
 
+// epi on (D in)(h) for the sites [h_begin, h_end) of a launch, by the routine of
+// the storage: fixed point for FP64 with fixed-point links, cp.async for 16-bit
+// spinors, registers otherwise
+template <bool DAGGER, bool TFIX, bool R8, class In, class G, class Epi>
+__device__ __forceinline__ void dslash_sites(const Geom& g, const In& in, const G& gauge, int h_begin, int h_end,
+                                             int parity, const Epi& epi, double* red) {
+  if constexpr (std::is_same<G, GaugeX64>::value) {
+    dslash_sites_fixed<DAGGER, TFIX>(g, in, gauge, h_begin, h_end, parity, epi, red);
+  } else {
+    for (int h = h_begin + blockIdx.x * blockDim.x + threadIdx.x; h < h_end; h += gridDim.x * blockDim.x) {
+      typename G::real acc[24];
+      if constexpr (UseAsync<In, R8>::value) dslash_site_async<DAGGER, TFIX>(g, in, gauge, h, parity, acc);
+      else dslash_site<DAGGER, TFIX, R8, Epi::NRED == 0>(g, in, gauge, h, parity, acc);
+      epi(h, acc, red);
+    }
+  }
+}
+
 // TFIX: links in the temporal gauge; R8: FP32 / 16-bit links as the 8
 // numbers of App. A.2.  Both are compile-time variants selected at launch.
 template <bool DAGGER, bool TFIX, bool R8, typename R, class In, class G, class Epi>
@@ -600,12 +619,7 @@ __global__ void __launch_bounds__(kDslashBlock, (DslashOccupancy<R, In, Epi::NRE
   double red[NR];
 #pragma unroll
   for (int k = 0; k < NR; ++k) red[k] = 0.0;
-  for (int h = g.h_begin + blockIdx.x * blockDim.x + threadIdx.x; h < g.h_end; h += gridDim.x * blockDim.x) {
-    R acc[24];
-    if constexpr (UseAsync<In, R8>::value) dslash_site_async<DAGGER, TFIX>(g, in, gauge, h, parity, acc);
-    else dslash_site<DAGGER, TFIX, R8, Epi::NRED == 0>(g, in, gauge, h, parity, acc);
-    epi(h, acc, red);
-  }
+  dslash_sites<DAGGER, TFIX, R8>(g, in, gauge, g.h_begin, g.h_end, parity, epi, red);
   if constexpr (Epi::NRED > 0) grid_reduce<Epi::NRED>(red, epi.rs, epi.fin);
 }
 
@@ -984,13 +998,13 @@ struct Tr<WD_F64> {
   using R = double;
   static size_t bytes(int stride) { return align256(192 * (size_t)stride); }
   static S view(const void* p, const Geom& g, size_t rs = 0) { return S{(double2*)p, g.stride, rs}; }
-  static G gauge(const Ctx& c) { return G{(const double2*)c.gauge[WD_F64], c.g.stride, c.recon}; }
+  static G gauge(const Ctx& c) { return G{(const double2*)c.gauge[WD_F64], c.g.stride, c.recon, c.gauge_fixed}; }
   // T-slab faces (wd_slab.cuh)
   using Fc = FaceF64;
   static size_t face_bytes(int fs) { return align256(96 * (size_t)fs); }
   static Fc face(const void* p, int fs) { return Fc{(const double2*)p, fs}; }
   static size_t link_face_bytes(const Ctx& c, int fs) { return align256((size_t)2 * (c.recon / 2) * 16 * fs); }
-  static LinkFace<G> link_face(const Ctx& c, const void* p, int fs) { return {G{(const double2*)p, fs, c.recon}}; }
+  static LinkFace<G> link_face(const Ctx& c, const void* p, int fs) { return {G{(const double2*)p, fs, c.recon, false}}; }
   static void pack_faces(const Ctx& c, void* lo, void* hi, const void* in, int fs, int dagger, int grid,
                          cudaStream_t s) {
     pack_faces_f64_kernel<<<grid, 256, 0, s>>>(c.g, (const double2*)in, c.g.stride, (double2*)lo, (double2*)hi, fs,
@@ -998,7 +1012,7 @@ struct Tr<WD_F64> {
   }
   static void pack_link_face(const Ctx& c, void* out, int fs, int grid, cudaStream_t s) {
     pack_link_face_kernel<double2><<<grid, 256, 0, s>>>(c.g, (const double2*)c.gauge[WD_F64], c.recon / 2,
-                                                        c.g.stride, (double2*)out, fs);
+                                                        c.g.stride, (double2*)out, fs, c.gauge_fixed);
   }
 };
 template <>
@@ -1113,11 +1127,31 @@ inline int wave_grid(int units, int block, int num_sms, int per_sm) {
   return b < w ? b : w;
 }
 
-template <typename R, class In, class G, class Epi>
-void launch_dslash(const Ctx& c, const In& in, const G& gauge, int parity, int dagger, const Epi& epi,
+// D or D^dag: kPlain / kDagger where the call site knows which (only that
+// kernel is compiled), an int where the caller's argument decides
+constexpr std::false_type kPlain{};
+constexpr std::true_type kDagger{};
+template <class Go>
+void pick_dagger(std::false_type, const Go& go) { go(std::false_type{}); }
+template <class Go>
+void pick_dagger(std::true_type, const Go& go) { go(std::true_type{}); }
+template <class Go>
+void pick_dagger(int dagger, const Go& go) {
+  if (dagger) go(std::true_type{});
+  else go(std::false_type{});
+}
+
+template <typename R, class In, class G, class Dag, class Epi>
+void launch_dslash(const Ctx& c, const In& in, const G& gauge, int parity, Dag dagger, const Epi& epi,
                    cudaStream_t s, const Geom* sub = nullptr) {
   // sub: the context's geometry with a narrower output-site range
   const Geom& geo = sub ? *sub : c.g;
+  if constexpr (std::is_same<G, GaugeF64>::value) {
+    if (gauge.fixed) {
+      launch_dslash<R>(c, in, GaugeX64{(const int4*)gauge.p, gauge.stride, gauge.recon}, parity, dagger, epi, s, sub);
+      return;
+    }
+  }
   // FP64 links never use the 8 numbers
   const bool r8 = (sizeof(R) == 4) && c.low_recon == 8;
   auto go = [&](auto dag, auto tfix, auto rec8) {
@@ -1137,17 +1171,19 @@ void launch_dslash(const Ctx& c, const In& in, const G& gauge, int parity, int d
     const int grid = wave_grid(geo.h_end - geo.h_begin, kDslashBlock, c.num_sms, per_sm);
     launch_pdl(k, dim3(grid), dim3(kDslashBlock), 0, s, geo, in, gauge, parity, epi);
   };
-  using T_ = std::true_type;
-  using F_ = std::false_type;
-  if constexpr (sizeof(R) == 4) {
-    if (r8) {
-      if (c.g.tfix) dagger ? go(T_{}, T_{}, T_{}) : go(F_{}, T_{}, T_{});
-      else dagger ? go(T_{}, F_{}, T_{}) : go(F_{}, F_{}, T_{});
-      return;
+  pick_dagger(dagger, [&](auto dag) {
+    using T_ = std::true_type;
+    using F_ = std::false_type;
+    if constexpr (sizeof(R) == 4) {
+      if (r8) {
+        if (c.g.tfix) go(dag, T_{}, T_{});
+        else go(dag, F_{}, T_{});
+        return;
+      }
     }
-  }
-  if (c.g.tfix) dagger ? go(T_{}, T_{}, F_{}) : go(F_{}, T_{}, F_{});
-  else dagger ? go(T_{}, F_{}, F_{}) : go(F_{}, F_{}, F_{});
+    if (c.g.tfix) go(dag, T_{}, F_{});
+    else go(dag, F_{}, F_{});
+  });
 }
 
 template <class Op>
@@ -1226,7 +1262,7 @@ struct Impl {
     {
       EpiXpayDot<S, S, S, FinBicgAlpha> e{T::view(b.v, g), T::view(b.p, g), T::view(b.r_tilde, g), nk2, c.red,
                                           FinBicgAlpha{b.ctl}};
-      launch_dslash<R>(c, T::view(b.tmp, g), T::gauge(c), 0, 0, e, s);
+      launch_dslash<R>(c, T::view(b.tmp, g), T::gauge(c), 0, kPlain, e, s);
     }
     // s = r - alpha v
     launch_sites(c, g.Vh, OpBicgS<S>{T::view(b.r_hat, g), T::view(b.v, g), b.ctl}, s);
@@ -1234,7 +1270,7 @@ struct Impl {
     dslash(c, b.tmp, b.r_hat, 1, 0, s);
     {
       EpiXpayTS<S, S, FinBicgOmega> e{T::view(b.t, g), T::view(b.r_hat, g), nk2, c.red, FinBicgOmega{b.ctl}};
-      launch_dslash<R>(c, T::view(b.tmp, g), T::gauge(c), 0, 0, e, s);
+      launch_dslash<R>(c, T::view(b.tmp, g), T::gauge(c), 0, kPlain, e, s);
     }
     // x_hat += alpha p + omega s, r = s - omega t, |r|^2, rho = <r_tilde, r>
     if (xf32(b))
@@ -1254,13 +1290,11 @@ struct Impl {
   static void bicg_update(const Ctx& c, SolveBufs& b, cudaStream_t s) {
     const Geom& g = c.g;
     accumulate(c, b, s);
-    EpiStore<SpinorF64> e0{T64::view(b.tmp64, g)};
-    launch_dslash<double>(c, T64::view(b.x, g), T64::gauge(c), 1, 0, e0, s);
+    ops_f64()->dslash(c, b.tmp64, b.x, 1, 0, s);
     if constexpr (P != WD_F64) {
       // r in FP32 in the FP64 residual buffer (unused by BiCGstab), then the
       // quantisation and reductions in a pass of their own
-      EpiResidF32 e1{TX::view(b.r, g), T64::view(b.b_hat, g), T64::view(b.x, g), Coef{0.0, &b.ctl->neg_kappa2}};
-      launch_dslash<double>(c, T64::view(b.tmp64, g), T64::gauge(c), 0, 0, e1, s);
+      ops_f64()->resid_f32(c, b, s);
       launch_sites(c, g.Vh,
                    OpRelupQuant<S, S, FinRelupBicg>{TX::view(b.r, g), T::view(b.r_hat, g), T::view(b.r_tilde, g),
                                                     c.red, FinRelupBicg{b.ctl}},
@@ -1269,23 +1303,37 @@ struct Impl {
       EpiRelupBicg<S, S, FinRelupBicg> e1{T64::view(b.b_hat, g), T64::view(b.x, g), T::view(b.r_hat, g),
                                            T::view(b.r_tilde, g), Coef{0.0, &b.ctl->neg_kappa2}, c.red,
                                            FinRelupBicg{b.ctl}};
-      launch_dslash<double>(c, T64::view(b.tmp64, g), T64::gauge(c), 0, 0, e1, s);
+      launch_dslash<double>(c, T64::view(b.tmp64, g), T64::gauge(c), 0, kPlain, e1, s);
     }
     launch_sites(c, g.Vh, OpRestart<S>{T::view(b.r_tilde, g), T::view(b.r_hat, g), T::view(b.p, g), T::view(b.v, g),
                                        b.ctl},
                  s);
   }
 
+  // the FP64 residuals r = b_hat - M_hat x of the reliable updates, from
+  // tmp64 = D_oe x, whatever the inner precision (in the FP64 table only)
+  static void resid_f32(const Ctx& c, SolveBufs& b, cudaStream_t s) {
+    const Geom& g = c.g;
+    EpiResidF32 e{TX::view(b.r, g), T64::view(b.b_hat, g), T64::view(b.x, g), Coef{0.0, &b.ctl->neg_kappa2}};
+    launch_dslash<double>(c, T64::view(b.tmp64, g), T64::gauge(c), 0, kPlain, e, s);
+  }
+  static void resid_cg(const Ctx& c, SolveBufs& b, cudaStream_t s) {
+    const Geom& g = c.g;
+    EpiResid<SpinorF64, SpinorF64, SpinorF64, FinRelupCgR> e{
+        T64::view(b.r, g), true, T64::view(b.b_hat, g), T64::view(b.x, g), Coef{0.0, &b.ctl->neg_kappa2}, c.red,
+        FinRelupCgR{b.ctl}};
+    launch_dslash<double>(c, T64::view(b.tmp64, g), T64::gauge(c), 0, kPlain, e, s);
+  }
+
   // ---- CG on M_hat^dag M_hat (Sec. 5.1), inner precision P
   static void cg_setup(const Ctx& c, SolveBufs& b, cudaStream_t s) {
     const Geom& g = c.g;
     // r_hat = M_hat^dag b_hat  (FP64 dslash, output quantised)
-    EpiStore<SpinorF64> e0{T64::view(b.tmp64, g)};
-    launch_dslash<double>(c, T64::view(b.b_hat, g), T64::gauge(c), 1, 1, e0, s);
+    ops_f64()->dslash(c, b.tmp64, b.b_hat, 1, 1, s);
     EpiXpayNorm<S, SpinorF64, FinCgSetup> e1{T::view(b.r_hat, g), T64::view(b.b_hat, g),
                                              Coef{0.0, &b.ctl->neg_kappa2}, c.red,
                                              FinCgSetup{b.ctl, c.scalars + 2}};
-    launch_dslash<double>(c, T64::view(b.tmp64, g), T64::gauge(c), 0, 1, e1, s);
+    launch_dslash<double>(c, T64::view(b.tmp64, g), T64::gauge(c), 0, kDagger, e1, s);
     zero(c, b.p, s);
     zero_xhat(c, b, s);
   }
@@ -1297,18 +1345,20 @@ struct Impl {
     dslash(c, b.tmp, b.p, 1, 0, s);
     {
       EpiXpayNorm<S, S, FinCgAlpha> e{T::view(b.v, g), T::view(b.p, g), nk2, c.red, FinCgAlpha{b.ctl}};
-      launch_dslash<R>(c, T::view(b.tmp, g), T::gauge(c), 0, 0, e, s);
+      launch_dslash<R>(c, T::view(b.tmp, g), T::gauge(c), 0, kPlain, e, s);
     }
     // q = M_hat^dag w; x_hat += alpha p; r -= alpha q; |r|^2
     dslash(c, b.tmp, b.v, 1, 1, s);
     if (xf32(b)) {
-      EpiCgUpdate<S, FinCgIter, SpinorF32> e{T::view(b.v, g), T::view(b.p, g), TX::view(b.x_hat, g),
-                                             T::view(b.r_hat, g), nk2, b.ctl, c.red, FinCgIter{b.ctl}};
-      launch_dslash<R>(c, T::view(b.tmp, g), T::gauge(c), 0, 1, e, s);
+      if constexpr (T::S::kBytesPerSite < 96) {
+        EpiCgUpdate<S, FinCgIter, SpinorF32> e{T::view(b.v, g), T::view(b.p, g), TX::view(b.x_hat, g),
+                                               T::view(b.r_hat, g), nk2, b.ctl, c.red, FinCgIter{b.ctl}};
+        launch_dslash<R>(c, T::view(b.tmp, g), T::gauge(c), 0, kDagger, e, s);
+      }
     } else {
       EpiCgUpdate<S, FinCgIter> e{T::view(b.v, g), T::view(b.p, g), T::view(b.x_hat, g), T::view(b.r_hat, g),
                                   nk2, b.ctl, c.red, FinCgIter{b.ctl}};
-      launch_dslash<R>(c, T::view(b.tmp, g), T::gauge(c), 0, 1, e, s);
+      launch_dslash<R>(c, T::view(b.tmp, g), T::gauge(c), 0, kDagger, e, s);
     }
   }
   static void cg_update(const Ctx& c, SolveBufs& b, cudaStream_t s) {
@@ -1316,16 +1366,14 @@ struct Impl {
     const Coef nk2{0.0, &b.ctl->neg_kappa2};
     accumulate(c, b, s);
     // r = b_hat - M_hat x  (FP64, stored)
-    EpiStore<SpinorF64> e0{T64::view(b.tmp64, g)};
-    launch_dslash<double>(c, T64::view(b.x, g), T64::gauge(c), 1, 0, e0, s);
-    EpiResid<SpinorF64, SpinorF64, SpinorF64, FinRelupCgR> e1{
-        T64::view(b.r, g), true, T64::view(b.b_hat, g), T64::view(b.x, g), nk2, c.red, FinRelupCgR{b.ctl}};
-    launch_dslash<double>(c, T64::view(b.tmp64, g), T64::gauge(c), 0, 0, e1, s);
+    const PrecOps* o64 = ops_f64();
+    o64->dslash(c, b.tmp64, b.x, 1, 0, s);
+    o64->resid_cg(c, b, s);
     // r_hat = M_hat^dag r (quantised)
-    launch_dslash<double>(c, T64::view(b.r, g), T64::gauge(c), 1, 1, e0, s);
+    o64->dslash(c, b.tmp64, b.r, 1, 1, s);
     EpiXpayNorm<S, SpinorF64, FinRelupCgN> e2{T::view(b.r_hat, g), T64::view(b.r, g), nk2, c.red,
                                               FinRelupCgN{b.ctl}};
-    launch_dslash<double>(c, T64::view(b.tmp64, g), T64::gauge(c), 0, 1, e2, s);
+    launch_dslash<double>(c, T64::view(b.tmp64, g), T64::gauge(c), 0, kDagger, e2, s);
   }
 
   // ---- T-slab decomposition (Sec. 6): faces and the split dslash
@@ -1391,6 +1439,10 @@ struct Impl {
     o.bicg_iteration = &bicg_iteration;
     o.bicg_update = &bicg_update;
     o.bicg_setup = &bicg_setup;
+    if constexpr (P == WD_F64) {
+      o.resid_f32 = &resid_f32;
+      o.resid_cg = &resid_cg;
+    }
     o.cg_iteration = &cg_iteration;
     o.cg_update = &cg_update;
     o.cg_setup = &cg_setup;

@@ -420,10 +420,10 @@ wd_status retire(wd_server* sv, Pool& pl, Request& q, int r, const SolverCtl& hc
   const Coef ck{-q.kappa, nullptr};
   EpiResid<SpinorF64, SpinorF64, SpinorF64, FinStore> ee{T64::view(nullptr, g), false, T64::view(bf, g),
                                                          T64::view(s.x, g), ck, c.red, FinStore{sc + 2, 1}};
-  launch_dslash<double>(c, T64::view(s.tmp64, g), T64::gauge(c), 0, 0, ee, c.stream);
+  launch_dslash<double>(c, T64::view(s.tmp64, g), T64::gauge(c), 0, kPlain, ee, c.stream);
   EpiResid<SpinorF64, SpinorF64, SpinorF64, FinStore> eo{T64::view(nullptr, g), false, T64::view(bf + f64, g),
                                                          T64::view(s.tmp64, g), ck, c.red, FinStore{sc + 3, 1}};
-  launch_dslash<double>(c, T64::view(s.x, g), T64::gauge(c), 1, 0, eo, c.stream);
+  launch_dslash<double>(c, T64::view(s.x, g), T64::gauge(c), 1, kPlain, eo, c.stream);
   WS_CK(sv, cudaGetLastError());
   // the request's four norms into its own pinned entry
   if (!sv->scal_pinned) {

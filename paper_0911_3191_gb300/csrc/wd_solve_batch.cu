@@ -292,7 +292,7 @@ wd_status solve_batch_device(wd_ctx* ctx, int n, void* x, const void* bsrc, cons
   launch_finalize<1>(bl, all, bl.blas_gx, FinStore{b.scal + n, 1}, b.bc, 0, 0, s);
   // b_hat_r = b_e,r + kappa_r D_eo b_o,r ; x accumulators zero
   EpiXpay<SpinorF64, SpinorF64> eb{bhat, be, Coef{0.0, b.kappas, 1}};
-  launch_dslash_mrhs<double>(g, bl, bo, T64::gauge(c), 0, 0, eb, all, s);
+  launch_dslash_mrhs<double>(g, bl, bo, T64::gauge(c), 0, kPlain, eb, all, s);
   launch_sites_batch(g, bl, OpZero<SpinorF64>{xacc}, all, s);
   WB_CK_LAUNCH(ctx);
 
@@ -328,13 +328,13 @@ wd_status solve_batch_device(wd_ctx* ctx, int n, void* x, const void* bsrc, cons
   // FP64 true residuals |b_r - M x_r|^2 (S13)
   launch_sites_batch(g, bl, OpConvert<SpinorF64, SpinorF64>{xe, xacc}, all, s);
   EpiXpay<SpinorF64, SpinorF64> ex{xo, bo, Coef{0.0, b.kappas, 1}};
-  launch_dslash_mrhs<double>(g, bl, xe, T64::gauge(c), 1, 0, ex, all, s);
+  launch_dslash_mrhs<double>(g, bl, xe, T64::gauge(c), 1, kPlain, ex, all, s);
   const Coef nk{0.0, b.kappas + n, 1};
   EpiResid<SpinorF64, SpinorF64, SpinorF64, FinStore> re{xe, false, be, xe, nk, c.red, FinStore{b.scal + 2 * n, 1}};
-  launch_dslash_mrhs<double>(g, bl, xo, T64::gauge(c), 0, 0, re, all, s);
+  launch_dslash_mrhs<double>(g, bl, xo, T64::gauge(c), 0, kPlain, re, all, s);
   launch_finalize<1>(bl, all, mrhs_grid<double>(bl), FinStore{b.scal + 2 * n, 1}, b.bc, 0, 0, s);
   EpiResid<SpinorF64, SpinorF64, SpinorF64, FinStore> ro{xo, false, bo, xo, nk, c.red, FinStore{b.scal + 3 * n, 1}};
-  launch_dslash_mrhs<double>(g, bl, xe, T64::gauge(c), 1, 0, ro, all, s);
+  launch_dslash_mrhs<double>(g, bl, xe, T64::gauge(c), 1, kPlain, ro, all, s);
   launch_finalize<1>(bl, all, mrhs_grid<double>(bl), FinStore{b.scal + 3 * n, 1}, b.bc, 0, 0, s);
   WB_CK_LAUNCH(ctx);
   SolverCtl* hc = (SolverCtl*)c.batch_host;
