@@ -251,24 +251,30 @@ __global__ void gauge_f64_to_16_kernel(Geom g, const double2* in, int nc, bool f
 
 // Batch loop control, last node of the batched WHILE body: continue while a
 // system is unconverged; bounded on its own at max_iter + 16 executions.
+// One warp, a lane per system.
 __global__ void batch_loop_control_kernel(BatchCtl* bc, const SolverCtl* ctl_in, int nrhs) {
   SolverCtl* ctl = const_cast<SolverCtl*>(ctl_in);
-  int all = 1;
-  for (int r = 0; r < nrhs; ++r)
-    if (!ctl[r].done) all = 0;
-  bc->loops += 1;
-  bc->step_loops += 1;
-  if (!all && bc->loops > bc->max_loops) {
-    for (int r = 0; r < nrhs; ++r)
+  const int lane = threadIdx.x;
+  bool mine = true;
+  for (int r = lane; r < nrhs; r += 32) mine = mine && ctl[r].done;
+  int all = __all_sync(0xffffffffu, mine);
+  const int loops = bc->loops + 1, step_loops = bc->step_loops + 1;
+  if (!all && loops > bc->max_loops) {
+    for (int r = lane; r < nrhs; r += 32)
       if (!ctl[r].done) {
         ctl[r].done = 1;
         if (ctl[r].status == WD_OK) ctl[r].status = WD_ERR_NOT_CONVERGED;
       }
     all = 1;
   }
-  bc->all_done = all;
-  const int cont = !all && bc->step_loops < bc->step_limit;
-  if (bc->in_graph) cudaGraphSetConditional((cudaGraphConditionalHandle)bc->h_loop, cont ? 1u : 0u);
+  __syncwarp();  // every lane has read the counters
+  if (lane == 0) {
+    bc->loops = loops;
+    bc->step_loops = step_loops;
+    bc->all_done = all;
+    const int cont = !all && step_loops < bc->step_limit;
+    if (bc->in_graph) cudaGraphSetConditional((cudaGraphConditionalHandle)bc->h_loop, cont ? 1u : 0u);
+  }
 }
 
 __global__ void batch_init_kernel(SolverCtl* ctl, BatchCtl* bc, int nrhs, double tol, double delta, int max_iter,

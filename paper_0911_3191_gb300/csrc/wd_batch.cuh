@@ -491,8 +491,8 @@ __global__ void __launch_bounds__(kDslashBlock, (DslashOccupancy<R, In, Epi::NRE
   for (int k = 0; k < NR; ++k) red[k] = 0.0;
   dslash_sites<DAGGER, TFIX, R8>(g, v, gauge, 0, g.Vh, parity, e, red);
   if constexpr (Epi::NRED > 0) {
-    __shared__ double sm[32][NR];
-    block_sum<NR>(red, sm);
+    __shared__ double sm[NR * kDslashBlock];
+    block_sum<NR, kDslashBlock>(red, sm);
     if (threadIdx.x == 0)
 #pragma unroll
       for (int k = 0; k < NR; ++k) ba.partials[((size_t)r * NR + k) * gridDim.x + blockIdx.x] = red[k];
@@ -513,8 +513,8 @@ __global__ void __launch_bounds__(kBlasBlock) site_batch_kernel(int n, Op op, Ba
     for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < n; h += gridDim.x * blockDim.x) o(h, red);
   }
   if constexpr (Op::NRED > 0) {
-    __shared__ double sm[32][NR];
-    block_sum<NR>(red, sm);
+    __shared__ double sm[NR * kBlasBlock];
+    block_sum<NR, kBlasBlock>(red, sm);
     if (threadIdx.x == 0)
 #pragma unroll
       for (int k = 0; k < NR; ++k) ba.partials[((size_t)r * NR + k) * gridDim.x + blockIdx.x] = red[k];
@@ -525,20 +525,16 @@ __global__ void __launch_bounds__(kBlasBlock) site_batch_kernel(int n, Op op, Ba
 // finaliser; the last block decides for the batch.  `which` selects the
 // ticket counter; set_update != 0 publishes "any update pending" to the IF
 // node of the solver graph.
+constexpr int kFinalizeBlock = 128;
 template <int NR, class Fin>
-__global__ void __launch_bounds__(128) batch_finalize_kernel(BatchArgs ba, int nblk, Fin fin, BatchCtl* bc,
+__global__ void __launch_bounds__(kFinalizeBlock) batch_finalize_kernel(BatchArgs ba, int nblk, Fin fin, BatchCtl* bc,
                                                              int which, int set_update) {
   pdl_wait();
   const int r = blockIdx.x;
   double s[NR];
-#pragma unroll
-  for (int k = 0; k < NR; ++k) s[k] = 0.0;
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x)
-#pragma unroll
-    for (int k = 0; k < NR; ++k) s[k] += __ldcg(ba.partials + ((size_t)r * NR + k) * nblk + b);
-  __shared__ double sm[32][NR];
+  __shared__ double sm[NR * kFinalizeBlock];
   __shared__ bool last;
-  block_sum<NR>(s, sm);
+  partial_sum<NR, kFinalizeBlock>(ba.partials + (size_t)r * NR * nblk, nblk, nblk, 1, s, sm);
   if (threadIdx.x == 0) {
     if (rhs_active(ba, r)) fin.at(r)(s);
     __threadfence();
@@ -546,16 +542,29 @@ __global__ void __launch_bounds__(128) batch_finalize_kernel(BatchArgs ba, int n
     last = (ticket == gridDim.x - 1);
   }
   __syncthreads();
-  if (last && threadIdx.x == 0 && set_update) {
+  if (last && threadIdx.x < 32 && set_update) {
+    // one lane per system: read one after another, the control blocks cost an
+    // L2 latency each (12 systems: 16 -> 8 us for this kernel)
     __threadfence();
+    const int lane = threadIdx.x;
     int any = 0;
-    for (int q = 0; q < ba.nrhs; ++q) {
-      const volatile SolverCtl* c = ba.ctl + q;
-      if (!c->done && c->do_update) bc->upd_list[any++] = q;
+    for (int q0 = 0; q0 < ba.nrhs; q0 += 32) {
+      const int q = q0 + lane;
+      bool due = false;
+      if (q < ba.nrhs) {
+        const volatile SolverCtl* c = ba.ctl + q;
+        const int done = c->done, upd = c->do_update;
+        due = !done && upd;
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, due);
+      if (due) bc->upd_list[any + __popc(m & ((1u << lane) - 1u))] = q;
+      any += __popc(m);
     }
-    bc->nupd = any;
-    bc->any_update = any > 0;
-    if (bc->in_graph) cudaGraphSetConditional((cudaGraphConditionalHandle)bc->h_update, any > 0 ? 1u : 0u);
+    if (lane == 0) {
+      bc->nupd = any;
+      bc->any_update = any > 0;
+      if (bc->in_graph) cudaGraphSetConditional((cudaGraphConditionalHandle)bc->h_update, any > 0 ? 1u : 0u);
+    }
   }
 }
 
@@ -663,7 +672,7 @@ void launch_sites_batch(const Geom& g, const BatchLaunch& bl, const Op& op, cons
 template <int NR, class Fin>
 void launch_finalize(const BatchLaunch& bl, const BatchArgs& ba, int nblk, const Fin& fin, BatchCtl* bc, int which,
                      int set_update, cudaStream_t s) {
-  launch_pdl(batch_finalize_kernel<NR, Fin>, dim3(bl.nrhs), dim3(128), 0, s, ba, nblk, fin, bc, which, set_update);
+  launch_pdl(batch_finalize_kernel<NR, Fin>, dim3(bl.nrhs), dim3(kFinalizeBlock), 0, s, ba, nblk, fin, bc, which, set_update);
 }
 
 // Fields of a batched solve: one allocation per field kind, system r's field

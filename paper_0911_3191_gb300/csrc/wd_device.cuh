@@ -1087,7 +1087,7 @@ __device__ __forceinline__ void dslash_site(const Geom& g, const In& in, const G
 
 // ------------------------------------------------------- FP64 reductions
 // Deterministic single-pass grid reduction (Sec. 5.1: global sums in FP64,
-// tree reduction): fixed-order warp-shuffle tree inside each block, one
+// tree reduction): fixed-order sum inside each block, one
 // partial per block, and the last block to finish (found with an atomic
 // ticket that resets itself) sums the partials in block order and runs the
 // finaliser.  The result depends only on the grid size, never on timing.
@@ -1096,35 +1096,62 @@ struct RedScratch {
   unsigned* counter;   // zero between reductions
 };
 
-template <int N>
-__device__ __forceinline__ void block_sum(double (&v)[N], double (*sm)[N]) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+// Sum over a block of B threads, N quantities: through shared memory, one warp
+// per quantity (32 lanes each add B / 32 values, then a shuffle tree).  Every
+// FP64 add holds its SM quarter's FP64 pipe for 67 cycles whatever its lanes do,
+// so the count of warp-wide adds is what a reduction costs: N (B / 32 + 4) here,
+// against 5 N B / 32 for a shuffle tree in every warp (256 threads, three sums:
+// 36 for 135).  sm holds N * B doubles; the totals come back in v of thread 0.
+template <int N, int B>
+__device__ __forceinline__ void block_sum(double (&v)[N], double* sm) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 #pragma unroll
-  for (int k = 0; k < N; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < N; ++k) sm[warp][k] = v[k];
+  for (int k = 0; k < N; ++k) sm[k * B + tid] = v[k];
   __syncthreads();
-  if (warp == 0) {
 #pragma unroll
-    for (int k = 0; k < N; ++k) {
-      v[k] = (lane < nw) ? sm[lane][k] : 0.0;
+  for (int k0 = 0; k0 < N; k0 += B / 32) {
+    const int k = k0 + warp;
+    if (k < N) {
+      double s = sm[k * B + lane];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+      for (int j = 32; j < B; j += 32) s += sm[k * B + j + lane];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+      if (lane == 0) sm[k * B] = s;
     }
   }
   __syncthreads();
+  if (tid == 0)
+#pragma unroll
+    for (int k = 0; k < N; ++k) v[k] = sm[k * B];
 }
 
-// All threads of the block call this once, after their grid-stride loop.
-// fin(const double* totals) runs on one thread of the last block.
-template <int N, class Fin>
+// Sum of n partials per quantity, quantity k of partial b at p[k * ks + b * bs],
+// by a block of B threads; four loads of each thread are in flight at a time
+// (one after another, the L2 latency of each would follow the other's).
+template <int N, int B>
+__device__ __forceinline__ void partial_sum(const double* p, int n, size_t ks, size_t bs, double (&s)[N], double* sm) {
+#pragma unroll
+  for (int k = 0; k < N; ++k) s[k] = 0.0;
+  for (int b = threadIdx.x; b < n; b += 4 * B) {
+    double t[4][N];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int k = 0; k < N; ++k) t[j][k] = b + j * B < n ? __ldcg(p + k * ks + (size_t)(b + j * B) * bs) : 0.0;
+#pragma unroll
+    for (int k = 0; k < N; ++k) s[k] += (t[0][k] + t[1][k]) + (t[2][k] + t[3][k]);
+  }
+  block_sum<N, B>(s, sm);
+}
+
+// All threads of the block (B of them) call this once, after their grid-stride
+// loop.  fin(const double* totals) runs on one thread of the last block.
+template <int N, int B, class Fin>
 __device__ __forceinline__ void grid_reduce(double (&v)[N], const RedScratch& rs, const Fin& fin) {
-  __shared__ double sm[32][N];
+  __shared__ double sm[N * B];
   __shared__ bool is_last;
-  block_sum<N>(v, sm);
+  block_sum<N, B>(v, sm);
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int k = 0; k < N; ++k) rs.partials[(size_t)blockIdx.x * N + k] = v[k];
@@ -1136,12 +1163,7 @@ __device__ __forceinline__ void grid_reduce(double (&v)[N], const RedScratch& rs
   if (!is_last) return;
   __threadfence();
   double s[N];
-#pragma unroll
-  for (int k = 0; k < N; ++k) s[k] = 0.0;
-  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
-#pragma unroll
-    for (int k = 0; k < N; ++k) s[k] += __ldcg(rs.partials + (size_t)b * N + k);
-  block_sum<N>(s, sm);
+  partial_sum<N, B>(rs.partials, gridDim.x, 1, N, s, sm);
   if (threadIdx.x == 0) fin(s);
 }
 
@@ -1150,8 +1172,8 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
-  double d = b.x * b.x + b.y * b.y;
-  return make_double2((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
+  const double i = 1.0 / (b.x * b.x + b.y * b.y);  // one division: some ten dependent FP64 operations
+  return make_double2((a.x * b.x + a.y * b.y) * i, (a.y * b.x - a.x * b.y) * i);
 }
 __device__ __forceinline__ bool cfinite(double2 a) { return isfinite(a.x) && isfinite(a.y); }
 

@@ -103,7 +103,7 @@ struct FinBicgIter {
     ctl->rr = rr;
     ctl->rho_prev = ctl->rho;
     ctl->rho = rho_new;
-    ctl->beta = cmul(cdiv(rho_new, ctl->rho_prev), cdiv(ctl->alpha, ctl->omega));
+    ctl->beta = cdiv(cmul(rho_new, ctl->alpha), cmul(ctl->rho_prev, ctl->omega));
     decide_update(ctl, (rho_new.x == 0.0 && rho_new.y == 0.0) ? 0.0 : rr, ctl->stop2);
   }
 };
@@ -128,7 +128,7 @@ struct FinRelupBicg {
       ctl->beta = make_double2(0.0, 0.0);
     } else {
       ctl->rho = rho;
-      ctl->beta = cmul(cdiv(rho, ctl->rho_prev), cdiv(ctl->alpha, ctl->omega));
+      ctl->beta = cdiv(cmul(rho, ctl->alpha), cmul(ctl->rho_prev, ctl->omega));
     }
     if (r2 <= ctl->stop2) { ctl->status = WD_OK; ctl->done = 1; }
     else if (ctl->iter >= ctl->max_iter) ctl_fail(ctl, WD_ERR_NOT_CONVERGED);
@@ -620,7 +620,7 @@ __global__ void __launch_bounds__(kDslashBlock, (DslashOccupancy<R, In, Epi::NRE
 #pragma unroll
   for (int k = 0; k < NR; ++k) red[k] = 0.0;
   dslash_sites<DAGGER, TFIX, R8>(g, in, gauge, g.h_begin, g.h_end, parity, epi, red);
-  if constexpr (Epi::NRED > 0) grid_reduce<Epi::NRED>(red, epi.rs, epi.fin);
+  if constexpr (Epi::NRED > 0) grid_reduce<Epi::NRED, kDslashBlock>(red, epi.rs, epi.fin);
 }
 
 template <class Op>
@@ -631,7 +631,7 @@ __global__ void __launch_bounds__(kBlasBlock) site_kernel(int n, Op op) {
 #pragma unroll
   for (int k = 0; k < NR; ++k) red[k] = 0.0;
   for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < n; h += gridDim.x * blockDim.x) op(h, red);
-  if constexpr (Op::NRED > 0) grid_reduce<Op::NRED>(red, op.rs, op.fin);
+  if constexpr (Op::NRED > 0) grid_reduce<Op::NRED, kBlasBlock>(red, op.rs, op.fin);
 }
 
 __global__ void loop_control_kernel(SolverCtl* ctl);

@@ -597,7 +597,7 @@ wd_status pool_progress(wd_server* s, Pool& pl, int& waiting_for_memory, bool& d
       WS_CK(s, cudaMemcpyAsync(&hb, pl.bb.bc, sizeof(hb), cudaMemcpyDeviceToHost, c.stream));
       WS_CK(s, cudaStreamSynchronize(c.stream));
       if (hb.any_update) o->batch_update(c, pl.bl, pl.bb, c.stream);
-      batch_loop_control_kernel<<<1, 1, 0, c.stream>>>(pl.bb.bc, pl.bb.ctl, pl.capacity);
+      batch_loop_control_kernel<<<1, 32, 0, c.stream>>>(pl.bb.bc, pl.bb.ctl, pl.capacity);
       WS_CK(s, cudaMemcpyAsync(&hb, pl.bb.bc, sizeof(hb), cudaMemcpyDeviceToHost, c.stream));
       WS_CK(s, cudaStreamSynchronize(c.stream));
       if (hb.all_done) break;

@@ -318,7 +318,7 @@ wd_status solve_batch_device(wd_ctx* ctx, int n, void* x, const void* bsrc, cons
         o->batch_update(c, bl, b, s);
         WB_CK_LAUNCH(ctx);
       }
-      batch_loop_control_kernel<<<1, 1, 0, s>>>(b.bc, b.ctl, n);
+      batch_loop_control_kernel<<<1, 32, 0, s>>>(b.bc, b.ctl, n);
       WB_CK(ctx, cudaMemcpyAsync(&hb, b.bc, sizeof(hb), cudaMemcpyDeviceToHost, s));
       WB_CK(ctx, cudaStreamSynchronize(s));
       if (hb.all_done) break;
@@ -420,7 +420,7 @@ cudaError_t build_batch_loop_graph(const Ctx& c, int prec, BatchBufs& b, const B
   o->batch_update(c, bl, b, cs);
   WB_RET(cudaStreamEndCapture(cs, &unused));
   WB_RET(cudaStreamBeginCaptureToGraph(cs, body, &inode, nullptr, 1, cudaStreamCaptureModeThreadLocal));
-  batch_loop_control_kernel<<<1, 1, 0, cs>>>(b.bc, b.ctl, bl.nrhs);
+  batch_loop_control_kernel<<<1, 32, 0, cs>>>(b.bc, b.ctl, bl.nrhs);
   WB_RET(cudaStreamEndCapture(cs, &unused));
   WB_RET(cudaStreamDestroy(cs));
   WB_RET(cudaGraphInstantiate(exec, g, 0));
