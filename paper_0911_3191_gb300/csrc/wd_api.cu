@@ -25,18 +25,6 @@
 
 namespace wd {
 
-// Last node of the WHILE body: continue while not done.  The body count is
-// bounded here on its own (max_iter + 16 executions), whatever the
-// finalisers did, so the device loop always terminates.
-__global__ void loop_control_kernel(SolverCtl* ctl) {
-  ctl->loops += 1;
-  if (ctl->loops > ctl->max_iter + 16 && !ctl->done) {
-    ctl->done = 1;
-    if (ctl->status == WD_OK) ctl->status = WD_ERR_NOT_CONVERGED;
-  }
-  if (ctl->in_graph) cudaGraphSetConditional((cudaGraphConditionalHandle)ctl->h_loop, ctl->done ? 0u : 1u);
-}
-
 __global__ void init_ctl_kernel(SolverCtl* ctl, double tol, double delta, int max_iter, double kappa,
                                 const double* bnorm2, int in_graph, unsigned long long h_update,
                                 unsigned long long h_loop, int restart) {
@@ -540,7 +528,7 @@ cudaGraphNodeParams make_conditional_params() {
   return raw.p;
 }
 
-// WHILE(!done) { iteration; IF(update) { reliable update }; loop control }
+// WHILE(!done) { iteration; IF(update) { reliable update } }
 wd_status build_graph(wd_ctx* ctx, int solver, int prec, unsigned long long* h_update, unsigned long long* h_loop) {
   Ctx& c = ctx->c;
   const PrecOps* ops = prec_ops(prec);
@@ -583,10 +571,6 @@ wd_status build_graph(wd_ctx* ctx, int solver, int prec, unsigned long long* h_u
   WD_CK(ctx, cudaStreamBeginCaptureToGraph(cs, ubody, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
   if (solver == WD_BICGSTAB) ops->bicg_update(c, c.sb, cs);
   else ops->cg_update(c, c.sb, cs);
-  WD_CK(ctx, cudaStreamEndCapture(cs, &unused));
-  // loop control
-  WD_CK(ctx, cudaStreamBeginCaptureToGraph(cs, body, &inode, nullptr, 1, cudaStreamCaptureModeThreadLocal));
-  loop_control_kernel<<<1, 1, 0, cs>>>(c.sb.ctl);
   WD_CK(ctx, cudaStreamEndCapture(cs, &unused));
   WD_CK(ctx, cudaStreamDestroy(cs));
   cudaGraphExec_t exec;
@@ -756,15 +740,15 @@ wd_status solve_device(wd_ctx* ctx, void* x_full, const void* b_full, double kap
     info->status = result;
     info->seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     // setup: 3 norms, b_hat, zero x, control init, solver setup (4 kernels,
-    // CG: 2 dslash + 2 zero); per iteration: BiCGstab 7 (CG 5) + loop control;
-    // per reliable update: BiCGstab 4 (5 with a lower inner precision: the
+    // CG: 2 dslash + 2 zero); per iteration: BiCGstab 7 (CG 5);
+    // per reliable update: BiCGstab 3 (4 with a lower inner precision: the
     // quantisation pass), CG 5; end: x_o with the odd residual,
     // and the even residual dslash
     // (an initial guess: its two residual dslashes instead of the zeroing,
     // and the control update when it already meets the tolerance)
     const long long setup = 3 + (odd_zero ? 0 : 1) + (x0 ? 2 : 1) + 1 + 4 + (start_converged ? 1 : 0);
-    const long long per_it = (p.solver == WD_BICGSTAB ? 7 : 5) + (p.use_graph ? 1 : 0);
-    const long long per_up = (p.solver == WD_BICGSTAB) ? (p.inner_precision == WD_F64 ? 4 : 5) : 5;
+    const long long per_it = (p.solver == WD_BICGSTAB ? 7 : 5);
+    const long long per_up = (p.solver == WD_BICGSTAB) ? (p.inner_precision == WD_F64 ? 3 : 4) : 5;
     info->kernel_launches = setup + (long long)hc.iter * per_it + (long long)hc.updates * per_up + 2;
   }
   if (result != WD_OK) {

@@ -40,6 +40,20 @@ __device__ __forceinline__ void ctl_set_update(SolverCtl* ctl, int v) {
   if (ctl->in_graph) cudaGraphSetConditional((cudaGraphConditionalHandle)ctl->h_update, (unsigned)v);
 }
 
+// The solver graph's WHILE condition, set by the finaliser that ends an
+// iteration and again by the one that ends a reliable update (a kernel of its
+// own at the end of the body was one launch in nine of an iteration).  The
+// iteration's finaliser also bounds the body count on its own, at max_iter + 16
+// executions whatever the others do, so the device loop always terminates.
+__device__ __forceinline__ void ctl_set_loop(SolverCtl* ctl) {
+  if (ctl->in_graph) cudaGraphSetConditional((cudaGraphConditionalHandle)ctl->h_loop, ctl->done ? 0u : 1u);
+}
+__device__ __forceinline__ void ctl_end_iteration(SolverCtl* ctl) {
+  ctl->loops += 1;
+  if (ctl->loops > ctl->max_iter + 16 && !ctl->done) ctl_fail(ctl, WD_ERR_NOT_CONVERGED);
+  ctl_set_loop(ctl);
+}
+
 struct FinStore {
   double* out;
   int n;
@@ -113,6 +127,10 @@ struct FinRelupBicg {
   SolverCtl* ctl;
   __device__ __forceinline__ FinRelupBicg at(int r) const { return FinRelupBicg{ctl + r}; }
   __device__ void operator()(const double* t) const {
+    update(t);
+    ctl_set_loop(ctl);
+  }
+  __device__ __forceinline__ void update(const double* t) const {
     ctl->updates += 1;
     const double r2 = t[0];
     const double2 rho = make_double2(t[1], t[2]);
@@ -122,7 +140,7 @@ struct FinRelupBicg {
     ctl->maxr = sqrt(t[3]);
     if (ctl->restart) {
       // Alg. 1: a new inner solve from the new residual (r_tilde = r_hat,
-      // p = v = 0, set by OpRestart in the same update)
+      // p = v = 0, set by OpRelupQuant)
       ctl->rho = make_double2(t[3], 0.0);
       ctl->rho_prev = ctl->alpha = ctl->omega = make_double2(1.0, 0.0);
       ctl->beta = make_double2(0.0, 0.0);
@@ -179,6 +197,10 @@ struct FinRelupCgR {
   SolverCtl* ctl;
   __device__ __forceinline__ FinRelupCgR at(int r) const { return FinRelupCgR{ctl + r}; }
   __device__ void operator()(const double* t) const {
+    update(t);
+    ctl_set_loop(ctl);
+  }
+  __device__ __forceinline__ void update(const double* t) const {
     ctl->updates += 1;
     const double r2 = t[0];
     if (!isfinite(r2)) { ctl_fail(ctl, WD_ERR_NUMERIC); return; }
@@ -198,7 +220,7 @@ struct FinRelupCgN {
   __device__ __forceinline__ FinRelupCgN at(int r) const { return FinRelupCgN{ctl + r}; }
   __device__ void operator()(const double* t) const {
     const double rr = t[0];
-    if (!isfinite(rr)) { ctl_fail(ctl, WD_ERR_NUMERIC); return; }
+    if (!isfinite(rr)) { ctl_fail(ctl, WD_ERR_NUMERIC); ctl_set_loop(ctl); return; }
     ctl->rr = rr;
     ctl->maxr = sqrt(rr);
     // defect correction restarts CG from the new residual: p = r_hat
@@ -524,13 +546,16 @@ struct EpiResidF32 {
 };
 
 // r_hat = quantised r; reduce |r|^2 (from the FP32 values, one FP64 add per
-// site), <r_tilde, r_hat> and |r_hat|^2: the reductions of EpiRelupBicg
+// site), <r_tilde, r_hat> and |r_hat|^2: the reductions of EpiRelupBicg.
+// Defect correction (ctl->restart) also starts the next inner solve here:
+// r_tilde = r_hat, p = v = 0 (its <r_tilde, r_hat> is not used)
 template <class RH, class RT, class Fin>
 struct OpRelupQuant {
   static constexpr int NRED = 4;
   SpinorF32 r;
   RH rh;
-  RT rt;
+  RT rt, p, v;
+  const SolverCtl* ctl;
   RedScratch rs;
   Fin fin;
   __device__ __forceinline__ void operator()(int h, double* red) const {
@@ -556,6 +581,13 @@ struct OpRelupQuant {
     red[1] += (double)re;
     red[2] += (double)im;
     red[3] += (double)m;
+    if (ctl->restart) {
+      rt.store(h, q);
+#pragma unroll
+      for (int k = 0; k < 24; ++k) q[k] = 0.f;
+      p.store(h, q);
+      v.store(h, q);
+    }
   }
 };
 
@@ -633,8 +665,6 @@ __global__ void __launch_bounds__(kBlasBlock) site_kernel(int n, Op op) {
   for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < n; h += gridDim.x * blockDim.x) op(h, red);
   if constexpr (Op::NRED > 0) grid_reduce<Op::NRED, kBlasBlock>(red, op.rs, op.fin);
 }
-
-__global__ void loop_control_kernel(SolverCtl* ctl);
 
 // ------------------------------------------------------------ BLAS ops
 template <class S, typename R>
@@ -771,28 +801,6 @@ struct OpAccumulate {
     }
     x.store(h, xv);
     xh.store(h, hv);
-  }
-};
-
-// defect correction only (ctl->restart): r_tilde = r_hat, p = v = 0
-template <class S>
-struct OpRestart {
-  static constexpr int NRED = 0;
-  S rt, rh, p, v;
-  const SolverCtl* ctl;
-  __device__ __forceinline__ OpRestart at(int q) const {
-    return OpRestart{rt.at(q), rh.at(q), p.at(q), v.at(q), ctl + q};
-  }
-  __device__ __forceinline__ void operator()(int h, double*) const {
-    using R = typename S::real;
-    if (!ctl->restart) return;
-    R a[24];
-    rh.load(h, a);
-    rt.store(h, a);
-#pragma unroll
-    for (int k = 0; k < 24; ++k) a[k] = 0;
-    p.store(h, a);
-    v.store(h, a);
   }
 };
 
@@ -1297,7 +1305,8 @@ struct Impl {
       ops_f64()->resid_f32(c, b, s);
       launch_sites(c, g.Vh,
                    OpRelupQuant<S, S, FinRelupBicg>{TX::view(b.r, g), T::view(b.r_hat, g), T::view(b.r_tilde, g),
-                                                    c.red, FinRelupBicg{b.ctl}},
+                                                    T::view(b.p, g), T::view(b.v, g), b.ctl, c.red,
+                                                    FinRelupBicg{b.ctl}},
                    s);
     } else {
       EpiRelupBicg<S, S, FinRelupBicg> e1{T64::view(b.b_hat, g), T64::view(b.x, g), T::view(b.r_hat, g),
@@ -1305,9 +1314,6 @@ struct Impl {
                                            FinRelupBicg{b.ctl}};
       launch_dslash<double>(c, T64::view(b.tmp64, g), T64::gauge(c), 0, kPlain, e1, s);
     }
-    launch_sites(c, g.Vh, OpRestart<S>{T::view(b.r_tilde, g), T::view(b.r_hat, g), T::view(b.p, g), T::view(b.v, g),
-                                       b.ctl},
-                 s);
   }
 
   // the FP64 residuals r = b_hat - M_hat x of the reliable updates, from
