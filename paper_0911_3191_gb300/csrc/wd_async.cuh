@@ -349,26 +349,29 @@ __device__ __forceinline__ void async_step(AsyncSlots& sm, const Geom& g, const 
   async_hop<K, DAGGER, TFIX, In, G>(sm, g, top, bot, acc);
 }
 
+// spin pairs of the accumulator -> spinor order
+__device__ __forceinline__ void from_pairs(const float2 (&a2)[12], float (&acc)[24]) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+#pragma unroll
+    for (int ri = 0; ri < 2; ++ri) {
+      acc[(0 + c) * 2 + ri] = a2[2 * c + ri].x;
+      acc[(3 + c) * 2 + ri] = a2[2 * c + ri].y;
+      acc[(9 + c) * 2 + ri] = a2[6 + 2 * c + ri].x;
+      acc[(6 + c) * 2 + ri] = a2[6 + 2 * c + ri].y;
+    }
+  }
+}
+
 // acc = (D in)(h) (or D^dag), 16-bit spinors and 12-real 16-bit links; the
 // caller's block has kAsyncBlock threads.
 template <bool DAGGER, bool TFIX, class In, class G>
-__device__ __forceinline__ void dslash_site_async(const Geom& g, const In& in, const G& gauge, int h, int parity,
-                                                  float (&acc)[24]) {
-  __shared__ AsyncSlots sm;
+__device__ __forceinline__ void dslash_site_async(const Geom& g, const In& in, const G& gauge, AsyncSlots& sm, int h,
+                                                  int parity, float (&acc)[24]) {
   int x, y, z, t;
   site_coords(g, h, parity, x, y, z, t);
   int nb[8];
-  {
-    const int xo = x & 1;
-    nb[0] = (x == g.X - 1) ? h - (g.Xh - 1) : h + xo;
-    nb[1] = (x == 0) ? h + (g.Xh - 1) : h - (xo ^ 1);
-    nb[2] = (y == g.Y - 1) ? h - g.wy : h + g.Xh;
-    nb[3] = (y == 0) ? h + g.wy : h - g.Xh;
-    nb[4] = (z == g.Z - 1) ? h - g.wz : h + g.XhY;
-    nb[5] = (z == 0) ? h + g.wz : h - g.XhY;
-    nb[6] = (t == g.T - 1) ? h - g.wt : h + g.XhYZ;
-    nb[7] = (t == 0) ? h + g.wt : h - g.XhYZ;
-  }
+  neighbours(g, h, x, y, z, t, nb);
   const bool top = (t == g.T - 1), bot = (t == 0);
   async_issue<0, DAGGER, TFIX>(sm, in, gauge, parity, h, nb, top, bot);
   cp_commit();
@@ -386,16 +389,7 @@ __device__ __forceinline__ void dslash_site_async(const Geom& g, const In& in, c
     async_step_pairs<5, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a2);
     async_step_pairs<6, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a2);
     async_step_pairs<7, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a2);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-#pragma unroll
-      for (int ri = 0; ri < 2; ++ri) {
-        acc[(0 + c) * 2 + ri] = a2[2 * c + ri].x;
-        acc[(3 + c) * 2 + ri] = a2[2 * c + ri].y;
-        acc[(9 + c) * 2 + ri] = a2[6 + 2 * c + ri].x;
-        acc[(6 + c) * 2 + ri] = a2[6 + 2 * c + ri].y;
-      }
-    }
+    from_pairs(a2, acc);
     return;
   }
 #pragma unroll
@@ -408,6 +402,34 @@ __device__ __forceinline__ void dslash_site_async(const Geom& g, const In& in, c
   async_step<5, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, acc);
   async_step<6, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, acc);
   async_step<7, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, acc);
+}
+
+// the two hops of direction MU alone: acc = their sum (dslash_sites_split)
+template <int MU, bool DAGGER, bool TFIX, class In, class G>
+__device__ __forceinline__ void direction_async(const Geom& g, const In& in, const G& gauge, AsyncSlots& sm, int h,
+                                                int parity, const int (&nb)[8], bool top, bool bot,
+                                                float (&acc)[24]) {
+  async_issue<2 * MU, DAGGER, TFIX>(sm, in, gauge, parity, h, nb, top, bot);
+  cp_commit();
+  async_issue<2 * MU + 1, DAGGER, TFIX>(sm, in, gauge, parity, h, nb, top, bot);
+  cp_commit();
+  if constexpr (kSpinPairs && In::kPairedHops) {
+    float2 a2[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) a2[k] = make_float2(0.f, 0.f);
+    cp_wait<1>();
+    async_hop_pairs<2 * MU, DAGGER, TFIX, In, G>(sm, g, top, bot, a2);
+    cp_wait<0>();
+    async_hop_pairs<2 * MU + 1, DAGGER, TFIX, In, G>(sm, g, top, bot, a2);
+    from_pairs(a2, acc);
+  } else {
+#pragma unroll
+    for (int k = 0; k < 24; ++k) acc[k] = 0.f;
+    cp_wait<1>();
+    async_hop<2 * MU, DAGGER, TFIX, In, G>(sm, g, top, bot, acc);
+    cp_wait<0>();
+    async_hop<2 * MU + 1, DAGGER, TFIX, In, G>(sm, g, top, bot, acc);
+  }
 }
 
 }  // namespace wd

@@ -489,7 +489,7 @@ __global__ void __launch_bounds__(kDslashBlock, (DslashOccupancy<R, In, Epi::NRE
   double red[NR];
 #pragma unroll
   for (int k = 0; k < NR; ++k) red[k] = 0.0;
-  dslash_sites<DAGGER, TFIX, R8>(g, v, gauge, 0, g.Vh, parity, e, red);
+  dslash_sites<DAGGER, TFIX, R8, false>(g, v, gauge, 0, g.Vh, parity, e, red);
   if constexpr (Epi::NRED > 0) {
     __shared__ double sm[NR * kDslashBlock];
     block_sum<NR, kDslashBlock>(red, sm);

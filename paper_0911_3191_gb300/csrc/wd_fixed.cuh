@@ -332,26 +332,29 @@ __device__ __forceinline__ void fixed_raise(float m, int& E, int& top, long long
 // A backward hop takes U^dag h as the conjugate of U^T h^*: the same product
 // with the link read by columns, the projection's imaginary parts negated as
 // they are converted, and the result's as they are added.
-template <bool DAGGER, bool TFIX, bool PAIR>
-__device__ __forceinline__ void dslash_site_fixed(const Geom& g, const SpinorF64& in, const GaugeX64& gauge, int h,
-                                                  int parity, double (&out)[24]) {
-  __shared__ FixedSlots sm;
+//
+// The hops k0 .. k1 - 1 of a site (0, 8: all), in the unit of E; top: the largest
+// exponent met.
+template <bool DAGGER, bool TFIX>
+__device__ __forceinline__ void fixed_hops(const Geom& g, const SpinorF64& in, const GaugeX64& gauge, FixedSlots& sm,
+                                           int h, int parity, int k0, int k1, int& E, int& top,
+                                           long long (&acc)[24]) {
   constexpr int SF = DAGGER ? +1 : -1;  // the projector sign of the forward hops
   const int tid = threadIdx.x;
   int x, y, z, t;
   site_coords(g, h, parity, x, y, z, t);
   const bool last = (t == g.T - 1), first = (t == 0);
-  long long acc[24];
 #pragma unroll
   for (int k = 0; k < 24; ++k) acc[k] = 0;
-  int E = kFixedMinExp, top = 0;
-  int n = fixed_neighbour(g, h, x, y, z, t, 0);
-  fixed_issue_spinor<DAGGER>(sm, in, n, 0);
+  E = kFixedMinExp;
+  top = 0;
+  const int n = fixed_neighbour(g, h, x, y, z, t, k0);
+  fixed_issue_spinor<DAGGER>(sm, in, n, k0);
   cp_commit();
-  fixed_issue_link(sm, gauge, parity, h, n, 0);
+  if (!(TFIX && k0 == 6 && !last)) fixed_issue_link(sm, gauge, parity, h, n, k0);
   cp_commit();
 #pragma unroll 1
-  for (int k = 0; k < 6; ++k) {
+  for (int k = k0; k < min(k1, 6); ++k) {
     const int mu = k >> 1;
     const bool fwd = (k & 1) == 0;
     cp_wait<1>();  // the spinor of hop k
@@ -362,7 +365,7 @@ __device__ __forceinline__ void dslash_site_fixed(const Geom& g, const SpinorF64
         const uint4 w = sm.sp[c][tid];
         m = fx_max(m, w.y, w.w);
       }
-      if (k == 0) E = max(fx_exponent(m), kFixedMinExp) + 1;
+      if (k == k0) E = max(fx_exponent(m), kFixedMinExp) + 1;
       fixed_raise(m, E, top, acc);
     }
     // rows 0, 1 and their partners: row 0 joins spin 3 (x, y) or 2 (z), row 1
@@ -391,14 +394,17 @@ __device__ __forceinline__ void dslash_site_fixed(const Geom& g, const SpinorF64
       }
     }
     // the next hop's spinor takes the slots just read
-    const int nn = fixed_neighbour(g, h, x, y, z, t, k + 1);
-    fixed_issue_spinor<DAGGER>(sm, in, nn, k + 1);
+    int nn = 0;
+    if (k + 1 < k1) {
+      nn = fixed_neighbour(g, h, x, y, z, t, k + 1);
+      fixed_issue_spinor<DAGGER>(sm, in, nn, k + 1);
+    }
     cp_commit();
     cp_wait<1>();  // the link of hop k
     if (gauge.recon == 12) fx_row3(sm);
     long long gr[2][3], gi[2][3];
     fixed_su3(sm, step_i, step_j, hr, hi, gr, gi);
-    if (!(TFIX && k == 5 && !last)) fixed_issue_link(sm, gauge, parity, h, nn, k + 1);
+    if (k + 1 < k1 && !(TFIX && k == 5 && !last)) fixed_issue_link(sm, gauge, parity, h, nn, k + 1);
     cp_commit();
 #define WD_FIXED_ADD(MU, S, CONJ)                          \
   fixed_add<MU, S, CONJ, 0>(gr[0], gi[0], acc);            \
@@ -413,7 +419,7 @@ __device__ __forceinline__ void dslash_site_fixed(const Geom& g, const SpinorF64
     }
   }
 #pragma unroll 1
-  for (int k = 6; k < 8; ++k) {
+  for (int k = max(k0, 6); k < k1; ++k) {
     const bool fwd = k == 6;
     cp_wait<1>();
     {
@@ -423,6 +429,7 @@ __device__ __forceinline__ void dslash_site_fixed(const Geom& g, const SpinorF64
         const uint4 w = sm.sp[c][tid];
         m = fx_max(m, w.y, w.w);
       }
+      if (k == k0) E = max(fx_exponent(m), kFixedMinExp) + 1;
       fixed_raise(m, E, top, acc);
     }
     const bool unit = TFIX && (fwd ? !last : !first);
@@ -466,6 +473,15 @@ __device__ __forceinline__ void dslash_site_fixed(const Geom& g, const SpinorF64
     }
   }
 #undef WD_FIXED_ADD
+}
+
+// out = (D in)(h) for this thread's site
+template <bool DAGGER, bool TFIX, bool PAIR>
+__device__ __forceinline__ void dslash_site_fixed(const Geom& g, const SpinorF64& in, const GaugeX64& gauge,
+                                                  FixedSlots& sm, int h, int parity, double (&out)[24]) {
+  int E, top;
+  long long acc[24];
+  fixed_hops<DAGGER, TFIX>(g, in, gauge, sm, h, parity, 0, 8, E, top, acc);
   if (top < kFixedMinExp || top > kFixedMaxExp) {
     double slow[24];  // its address is taken on this path only
     if (dslash_site_outside<DAGGER, TFIX, PAIR>(g, in, gauge, h, parity, top, slow)) {
@@ -478,14 +494,84 @@ __device__ __forceinline__ void dslash_site_fixed(const Geom& g, const SpinorF64
   for (int k = 0; k < 24; ++k) out[k] = fx_sum_value(acc[k], E - 1078);
 }
 
+// The same with four warps for 32 sites, warp w taking the two hops of direction
+// w: a lattice that gives an SM no more than a warp or two per quarter is bound
+// by the latency of one thread's eight hops.  The partial sums pass through the
+// slots; warp w adds and converts spin w, and the threads of warp 0 get the
+// result (true) of sites below h_end.
+template <bool DAGGER, bool TFIX, bool PAIR>
+__device__ __forceinline__ bool dslash_site_fixed_split(const Geom& g, const SpinorF64& in, const GaugeX64& gauge,
+                                                        FixedSlots& sm, int h0, int h_end, int parity,
+                                                        double (&out)[24]) {
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, h = h0 + lane;
+  const bool ok = h < h_end;
+  if (ok) {
+    int E, top;
+    long long acc[24];
+    fixed_hops<DAGGER, TFIX>(g, in, gauge, sm, h, parity, 2 * w, 2 * w + 2, E, top, acc);
+#pragma unroll
+    for (int c = 0; c < 12; ++c)
+      *reinterpret_cast<longlong2*>(&sm.sp[c][tid]) = make_longlong2(acc[2 * c], acc[2 * c + 1]);
+    sm.lk[0][tid] = make_int4(E, top, 0, 0);
+  }
+  __syncthreads();
+  double* fin = reinterpret_cast<double*>(&sm.lk[1][0]);  // [24][32]
+  int top = 0;
+  if (ok) {
+    int e[4], E = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int4 v = sm.lk[0][lane + 32 * q];
+      e[q] = v.x;
+      E = max(E, v.x);
+      top = max(top, v.y);
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      long long r = 0, i = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const longlong2 v = *reinterpret_cast<const longlong2*>(&sm.sp[3 * w + c][lane + 32 * q]);
+        r += fx_sar(v.x, E - e[q]);
+        i += fx_sar(v.y, E - e[q]);
+      }
+      fin[(6 * w + 2 * c) * 32 + lane] = fx_sum_value(r, E - 1078);
+      fin[(6 * w + 2 * c + 1) * 32 + lane] = fx_sum_value(i, E - 1078);
+    }
+  }
+  __syncthreads();
+  if (!ok || w != 0) return false;
+  if (top < kFixedMinExp || top > kFixedMaxExp) {
+    double slow[24];
+    if (dslash_site_outside<DAGGER, TFIX, PAIR>(g, in, gauge, h, parity, top, slow)) {
+#pragma unroll
+      for (int k = 0; k < 24; ++k) out[k] = slow[k];
+      return true;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 24; ++k) out[k] = fin[k * 32 + lane];
+  return true;
+}
+
 // epi on (D in)(h) for the sites [h_begin, h_end) of a launch
-template <bool DAGGER, bool TFIX, class Epi>
+template <bool DAGGER, bool TFIX, bool SPLIT, class Epi>
 __device__ __forceinline__ void dslash_sites_fixed(const Geom& g, const SpinorF64& in, const GaugeX64& gauge,
                                                    int h_begin, int h_end, int parity, const Epi& epi, double* red) {
-  for (int h = h_begin + blockIdx.x * blockDim.x + threadIdx.x; h < h_end; h += gridDim.x * blockDim.x) {
-    double acc[24];
-    dslash_site_fixed<DAGGER, TFIX, Epi::NRED == 0>(g, in, gauge, h, parity, acc);
-    epi(h, acc, red);
+  __shared__ FixedSlots sm;
+  constexpr bool kPair = Epi::NRED == 0;
+  double acc[24];
+  if constexpr (SPLIT) {
+    for (int h0 = h_begin + blockIdx.x * 32; h0 < h_end; h0 += gridDim.x * 32) {
+      if (dslash_site_fixed_split<DAGGER, TFIX, kPair>(g, in, gauge, sm, h0, h_end, parity, acc))
+        epi(h0 + (int)threadIdx.x, acc, red);
+      __syncthreads();  // the slots are read: the next tile's copies may start
+    }
+  } else {
+    for (int h = h_begin + blockIdx.x * blockDim.x + threadIdx.x; h < h_end; h += gridDim.x * blockDim.x) {
+      dslash_site_fixed<DAGGER, TFIX, kPair>(g, in, gauge, sm, h, parity, acc);
+      epi(h, acc, red);
+    }
   }
 }
 

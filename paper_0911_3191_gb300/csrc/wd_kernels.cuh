@@ -623,19 +623,97 @@ struct UseAsync {
 };
 static_assert(kDslashBlock == kAsyncBlock, "the async slots are sized for the dslash block");
 
+// Exchange of the split kernels (SPLIT): four warps take 32 sites, warp w
+// the two hops of direction w, and warp 0 adds the four partial sums and runs the
+// epilogue.  A lattice that gives an SM quarter no more than a warp or so is
+// bound by the latency of one thread's eight hops, a few hundred instructions
+// each waiting for the last.
+struct SplitSums {
+  float v[24][kDslashBlock];
+};
+
+template <bool DAGGER, bool TFIX, bool R8, class In, class G, class Epi>
+__device__ __forceinline__ void dslash_sites_split(const Geom& g, const In& in, const G& gauge, AsyncSlots* slots,
+                                                   SplitSums& sums, int h_begin, int h_end, int parity,
+                                                   const Epi& epi, double* red) {
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  for (int h0 = h_begin + blockIdx.x * 32; h0 < h_end; h0 += gridDim.x * 32) {
+    const int h = h0 + lane;
+    const bool ok = h < h_end;
+    float acc[24];
+    if (ok) {
+      int x, y, z, t;
+      site_coords(g, h, parity, x, y, z, t);
+      int nb[8];
+      neighbours(g, h, x, y, z, t, nb);
+      const bool top = (t == g.T - 1), bot = (t == 0);
+      if constexpr (UseAsync<In, R8>::value) {
+        if (w == 0) direction_async<0, DAGGER, TFIX>(g, in, gauge, *slots, h, parity, nb, top, bot, acc);
+        else if (w == 1) direction_async<1, DAGGER, TFIX>(g, in, gauge, *slots, h, parity, nb, top, bot, acc);
+        else if (w == 2) direction_async<2, DAGGER, TFIX>(g, in, gauge, *slots, h, parity, nb, top, bot, acc);
+        else direction_async<3, DAGGER, TFIX>(g, in, gauge, *slots, h, parity, nb, top, bot, acc);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 24; ++k) acc[k] = 0.f;
+        if (w == 0) {
+          hop<0, true, DAGGER, R8>(in, gauge, parity, h, nb[0], false, acc);
+          hop<0, false, DAGGER, R8>(in, gauge, parity, nb[1], nb[1], false, acc);
+        } else if (w == 1) {
+          hop<1, true, DAGGER, R8>(in, gauge, parity, h, nb[2], false, acc);
+          hop<1, false, DAGGER, R8>(in, gauge, parity, nb[3], nb[3], false, acc);
+        } else if (w == 2) {
+          hop<2, true, DAGGER, R8>(in, gauge, parity, h, nb[4], false, acc);
+          hop<2, false, DAGGER, R8>(in, gauge, parity, nb[5], nb[5], false, acc);
+        } else {
+          hop_t<true, DAGGER, TFIX, R8>(in, gauge, parity, h, nb[6], top && g.tbc_anti, !top, acc);
+          hop_t<false, DAGGER, TFIX, R8>(in, gauge, parity, nb[7], nb[7], bot && g.tbc_anti, !bot, acc);
+        }
+      }
+    }
+    __syncthreads();  // the slots (which the sums may share) are read
+    if (ok)
+#pragma unroll
+      for (int k = 0; k < 24; ++k) sums.v[k][tid] = acc[k];
+    __syncthreads();
+    if (ok && w == 0) {
+#pragma unroll
+      for (int k = 0; k < 24; ++k)
+        acc[k] = (sums.v[k][lane] + sums.v[k][lane + 32]) + (sums.v[k][lane + 64] + sums.v[k][lane + 96]);
+      epi(h, acc, red);
+    }
+    __syncthreads();  // the sums are read: the next tile may start
+  }
+}
+
 // epi on (D in)(h) for the sites [h_begin, h_end) of a launch, by the routine of
 // the storage: fixed point for FP64 with fixed-point links, cp.async for 16-bit
 // spinors, registers otherwise
-template <bool DAGGER, bool TFIX, bool R8, class In, class G, class Epi>
+template <bool DAGGER, bool TFIX, bool R8, bool SPLIT, class In, class G, class Epi>
 __device__ __forceinline__ void dslash_sites(const Geom& g, const In& in, const G& gauge, int h_begin, int h_end,
                                              int parity, const Epi& epi, double* red) {
+  using R = typename G::real;
   if constexpr (std::is_same<G, GaugeX64>::value) {
-    dslash_sites_fixed<DAGGER, TFIX>(g, in, gauge, h_begin, h_end, parity, epi, red);
+    dslash_sites_fixed<DAGGER, TFIX, SPLIT>(g, in, gauge, h_begin, h_end, parity, epi, red);
+  } else if constexpr (UseAsync<In, R8>::value) {
+    __shared__ AsyncSlots sm;
+    static_assert(sizeof(SplitSums) <= sizeof(AsyncSlots), "the sums fit the slots");
+    if constexpr (SPLIT) {
+      dslash_sites_split<DAGGER, TFIX, R8>(g, in, gauge, &sm, reinterpret_cast<SplitSums&>(sm), h_begin, h_end,
+                                           parity, epi, red);
+    } else {
+      for (int h = h_begin + blockIdx.x * blockDim.x + threadIdx.x; h < h_end; h += gridDim.x * blockDim.x) {
+        R acc[24];
+        dslash_site_async<DAGGER, TFIX>(g, in, gauge, sm, h, parity, acc);
+        epi(h, acc, red);
+      }
+    }
+  } else if constexpr (SPLIT) {
+    __shared__ SplitSums sums;
+    dslash_sites_split<DAGGER, TFIX, R8>(g, in, gauge, nullptr, sums, h_begin, h_end, parity, epi, red);
   } else {
     for (int h = h_begin + blockIdx.x * blockDim.x + threadIdx.x; h < h_end; h += gridDim.x * blockDim.x) {
-      typename G::real acc[24];
-      if constexpr (UseAsync<In, R8>::value) dslash_site_async<DAGGER, TFIX>(g, in, gauge, h, parity, acc);
-      else dslash_site<DAGGER, TFIX, R8, Epi::NRED == 0>(g, in, gauge, h, parity, acc);
+      R acc[24];
+      dslash_site<DAGGER, TFIX, R8, Epi::NRED == 0>(g, in, gauge, h, parity, acc);
       epi(h, acc, red);
     }
   }
@@ -643,7 +721,7 @@ __device__ __forceinline__ void dslash_sites(const Geom& g, const In& in, const 
 
 // TFIX: links in the temporal gauge; R8: FP32 / 16-bit links as the 8
 // numbers of App. A.2.  Both are compile-time variants selected at launch.
-template <bool DAGGER, bool TFIX, bool R8, typename R, class In, class G, class Epi>
+template <bool DAGGER, bool TFIX, bool R8, bool SPLIT, typename R, class In, class G, class Epi>
 __global__ void __launch_bounds__(kDslashBlock, (DslashOccupancy<R, In, Epi::NRED, TFIX, R8>::kMinBlocks))
     dslash_kernel(Geom g, In in, G gauge, int parity, Epi epi) {
   pdl_wait();
@@ -651,7 +729,7 @@ __global__ void __launch_bounds__(kDslashBlock, (DslashOccupancy<R, In, Epi::NRE
   double red[NR];
 #pragma unroll
   for (int k = 0; k < NR; ++k) red[k] = 0.0;
-  dslash_sites<DAGGER, TFIX, R8>(g, in, gauge, g.h_begin, g.h_end, parity, epi, red);
+  dslash_sites<DAGGER, TFIX, R8, SPLIT>(g, in, gauge, g.h_begin, g.h_end, parity, epi, red);
   if constexpr (Epi::NRED > 0) grid_reduce<Epi::NRED, kDslashBlock>(red, epi.rs, epi.fin);
 }
 
@@ -1164,7 +1242,8 @@ void launch_dslash(const Ctx& c, const In& in, const G& gauge, int parity, Dag d
   const bool r8 = (sizeof(R) == 4) && c.low_recon == 8;
   auto go = [&](auto dag, auto tfix, auto rec8) {
     constexpr bool kTfix = decltype(tfix)::value;
-    auto* k = dslash_kernel<decltype(dag)::value, kTfix, decltype(rec8)::value, R, In, G, Epi>;
+    constexpr bool kR8 = decltype(rec8)::value;
+    auto* k = dslash_kernel<decltype(dag)::value, kTfix, kR8, false, R, In, G, Epi>;
     // One wave of resident blocks, measured per kernel class against 16
     // blocks per SM (several waves, the last one partly filled) at 64^3x128:
     // FP32 15 % faster, 16-bit temporal-gauge and 8-number kernels 5-8 %,
@@ -1176,7 +1255,20 @@ void launch_dslash(const Ctx& c, const In& in, const G& gauge, int parity, Dag d
     // 64^3x128) keep 16 blocks per SM.
     constexpr bool kWave = !(sizeof(R) == 8 || (In::kIntCodes && !kTfix));
     static const int per_sm = kWave ? resident_blocks(k, kDslashBlock) : 16;
-    const int grid = wave_grid(geo.h_end - geo.h_begin, kDslashBlock, c.num_sms, per_sm);
+    const int n = geo.h_end - geo.h_begin;
+    // Split kernels (a site over four warps) up to one block of 128 sites per
+    // SM.  FP64 in fixed point, 152 SMs: 2048 and 4096 sites 16.5 -> 8.4 us,
+    // 8192 16.6 -> 10.4, 16384 16.6 -> 14.6, 32768 20.7 either way, 65536 33.1
+    // against 34.8.  Compiled where small lattices spend their time: not for
+    // general FP64 links, 8-number links and FP64 with fused reductions.
+    if constexpr (!std::is_same<G, GaugeF64>::value && !kR8 && (sizeof(R) == 4 || Epi::NRED == 0)) {
+      if ((n + kDslashBlock - 1) / kDslashBlock <= c.num_sms) {
+        launch_pdl(dslash_kernel<decltype(dag)::value, kTfix, kR8, true, R, In, G, Epi>, dim3((n + 31) / 32),
+                   dim3(kDslashBlock), 0, s, geo, in, gauge, parity, epi);
+        return;
+      }
+    }
+    const int grid = wave_grid(n, kDslashBlock, c.num_sms, per_sm);
     launch_pdl(k, dim3(grid), dim3(kDslashBlock), 0, s, geo, in, gauge, parity, epi);
   };
   pick_dagger(dagger, [&](auto dag) {
