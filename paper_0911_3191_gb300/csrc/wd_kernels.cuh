@@ -1244,17 +1244,18 @@ void launch_dslash(const Ctx& c, const In& in, const G& gauge, int parity, Dag d
     constexpr bool kTfix = decltype(tfix)::value;
     constexpr bool kR8 = decltype(rec8)::value;
     auto* k = dslash_kernel<decltype(dag)::value, kTfix, kR8, false, R, In, G, Epi>;
-    // One wave of resident blocks, measured per kernel class against 16
-    // blocks per SM (several waves, the last one partly filled) at 64^3x128:
-    // FP32 15 % faster, 16-bit temporal-gauge and 8-number kernels 5-8 %,
-    // H16N/B16N general links 2-3 %; at 24^3x64 the plain Q16 dslash is 2 %
-    // slower on one wave but its reduction epilogues (fewer block partials)
-    // gain more: the benchmark solve is 3.4 % faster than with 16 blocks per
-    // SM for the small lattices.  The FP64 kernel (FP64-pipe bound; 6 %
-    // slower at 24^3x64) and the general-link Q16 kernel (6 % slower at
-    // 64^3x128) keep 16 blocks per SM.
-    constexpr bool kWave = !(sizeof(R) == 8 || (In::kIntCodes && !kTfix));
-    static const int per_sm = kWave ? resident_blocks(k, kDslashBlock) : 16;
+    // Blocks per SM at most, measured per kernel class.  FP32: one wave of
+    // resident blocks (64^3 x 128: 15 % faster than 16 per SM).  16 bit in the
+    // temporal gauge: two waves (24^3 x 64, L2-resident: Q16 30.9 -> 28.7 us,
+    // bf16 28.5 -> 26.1, fp16 30.8 -> 29.5; 64^3 x 128: Q16 929 -> 918, fp16 955
+    // -> 928, bf16 844 -> 850), and one with fused reductions, whose partial
+    // sums grow with the blocks (two: the 24^3 x 64 solve 0.1 % slower).  16 bit
+    // with general links: 16 (24^3 x 64 bf16 30.9 -> 28.0 us; 64^3 x 128 Q16
+    // 1045 -> 991, bf16 960-985 either way).  FP64: 16.
+    constexpr bool k16 = In::kBytesPerSite == 52;
+    constexpr int kWaves = k16 && Epi::NRED == 0 && kTfix && !kR8 ? 2 : 1;
+    constexpr bool kMany = sizeof(R) == 8 || (k16 && !kTfix && (In::kIntCodes || (Epi::NRED == 0 && !kR8)));
+    static const int per_sm = kMany ? 16 : kWaves * resident_blocks(k, kDslashBlock);
     const int n = geo.h_end - geo.h_begin;
     // Split kernels (a site over four warps) up to one block of 128 sites per
     // SM.  FP64 in fixed point, 152 SMs: 2048 and 4096 sites 16.5 -> 8.4 us,
