@@ -56,12 +56,16 @@ constexpr int kAsyncBlock = 128;  // threads per block of the kernels that use t
 constexpr bool kSpinPairs = true;  // packed FP32 pairs over spin rows (async_hop_pairs)
 constexpr int kAsyncStages = 3;
 
-struct AsyncSlots {
-  uint4 sp[kAsyncStages][3][kAsyncBlock];  // spinor words (temporal: 24 B in chunks 0, 1)
-  float sn[kAsyncStages][kAsyncBlock];     // site norm
-  uint4 l4[kAsyncStages][kAsyncBlock];     // link words 0..3
-  uint2 l2[kAsyncStages][kAsyncBlock];     // link words 4, 5
+// N: right-hand sides per thread (two in batches: they share the link, its
+// decoding and rebuilding, and the addresses)
+template <int N>
+struct AsyncSlotsN {
+  uint4 sp[kAsyncStages][N][3][kAsyncBlock];  // spinor words (temporal: 24 B in chunks 0, 1)
+  float sn[kAsyncStages][N][kAsyncBlock];     // site norm
+  uint4 l4[kAsyncStages][kAsyncBlock];        // link words 0..3
+  uint2 l2[kAsyncStages][kAsyncBlock];        // link words 4, 5
 };
+using AsyncSlots = AsyncSlotsN<1>;
 
 // hops in the order of dslash_site: x+, x-, y+, y-, z+, z-, t+, t-
 template <int K>
@@ -71,27 +75,32 @@ struct HopK {
   static constexpr int ST = K % kAsyncStages;
 };
 
-template <int K, bool DAGGER, bool TFIX, class In, class G>
-__device__ __forceinline__ void async_issue(AsyncSlots& sm, const In& in, const G& gauge, int parity, int h,
+template <int K, bool DAGGER, bool TFIX, int N, class In, class G>
+__device__ __forceinline__ void async_issue(AsyncSlotsN<N>& sm, const In (&ins)[N], const G& gauge, int parity, int h,
                                             const int (&nb)[8], bool top, bool bot) {
   using H = HopK<K>;
   const int tid = threadIdx.x;
   const int n = nb[K];
-  const size_t st = (size_t)in.stride;
-  if constexpr (H::MU < 3) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) cp16_cg(&sm.sp[H::ST][c][tid], in.p + c * st + n);
-  } else {
-    constexpr int S = (H::FWD != DAGGER) ? -1 : +1;
-    if constexpr (S == +1) {  // spins 0, 1: chunk 0 and the first half of chunk 1
-      cp16_cg(&sm.sp[H::ST][0][tid], in.p + n);
-      cp8_ca(&sm.sp[H::ST][1][tid], reinterpret_cast<const uint2*>(in.p + st + n));
-    } else {  // spins 2, 3: the second half of chunk 1 and chunk 2
-      cp8_ca(&sm.sp[H::ST][0][tid], reinterpret_cast<const uint2*>(in.p + st + n) + 1);
-      cp16_cg(&sm.sp[H::ST][1][tid], in.p + 2 * st + n);
+  for (int q = 0; q < N; ++q) {
+    const In& in = ins[q];
+    const size_t st = (size_t)in.stride;
+    auto& sp = sm.sp[H::ST][q];
+    if constexpr (H::MU < 3) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) cp16_cg(&sp[c][tid], in.p + c * st + n);
+    } else {
+      constexpr int S = (H::FWD != DAGGER) ? -1 : +1;
+      if constexpr (S == +1) {  // spins 0, 1: chunk 0 and the first half of chunk 1
+        cp16_cg(&sp[0][tid], in.p + n);
+        cp8_ca(&sp[1][tid], reinterpret_cast<const uint2*>(in.p + st + n));
+      } else {  // spins 2, 3: the second half of chunk 1 and chunk 2
+        cp8_ca(&sp[0][tid], reinterpret_cast<const uint2*>(in.p + st + n) + 1);
+        cp16_cg(&sp[1][tid], in.p + 2 * st + n);
+      }
     }
+    cp4_ca(&sm.sn[H::ST][q][tid], in.norm + n);
   }
-  cp4_ca(&sm.sn[H::ST][tid], in.norm + n);
   // the temporal links of the temporal gauge are 1 off the last slice
   const bool unit = TFIX && H::MU == 3 && (H::FWD ? !top : !bot);
   if (!unit) {
@@ -103,14 +112,25 @@ __device__ __forceinline__ void async_issue(AsyncSlots& sm, const In& in, const 
   }
 }
 
-template <int K, bool DAGGER, bool TFIX, class In, class G>
-__device__ __forceinline__ void async_hop(const AsyncSlots& sm, const Geom& g, bool top, bool bot, float (&acc)[24]) {
+// the six words of a temporal half spinor from its slots (24 B: a 16-byte and an
+// 8-byte copy, in the order of the two chunks they come from)
+template <bool UPPER>
+__device__ __forceinline__ void half_words(const uint4& a, const uint4& b, uint32_t (&w)[6]) {
+  if constexpr (UPPER) {
+    w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w; w[4] = b.x; w[5] = b.y;
+  } else {
+    w[0] = a.x; w[1] = a.y; w[2] = b.x; w[3] = b.y; w[4] = b.z; w[5] = b.w;
+  }
+}
+
+template <int K, bool DAGGER, bool TFIX, class In, class G, int N>
+__device__ __forceinline__ void async_hop(const AsyncSlotsN<N>& sm, const Geom& g, bool top, bool bot,
+                                          float (&accs)[N][24]) {
   using H = HopK<K>;
   constexpr int MU = H::MU;
   constexpr bool FWD = H::FWD;
   constexpr int S = (FWD != DAGGER) ? -1 : +1;
   const int tid = threadIdx.x;
-  float w = In::scale_of(sm.sn[H::ST][tid]);
   const bool unit = TFIX && MU == 3 && (FWD ? !top : !bot);
   float u[18];
   if (!unit) {
@@ -118,42 +138,42 @@ __device__ __forceinline__ void async_hop(const AsyncSlots& sm, const Geom& g, b
     const uint2 b = sm.l2[H::ST][tid];
     const uint32_t lw[6] = {a.x, a.y, a.z, a.w, b.x, b.y};
     G::from_words(lw, u);
-    if constexpr (G::kScaled) w *= G::kScale;  // Q16 links come back as raw codes
   }
-  if constexpr (MU < 3) {
-    uint32_t sw[12];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const uint4 d = sm.sp[H::ST][c][tid];
-      sw[4 * c] = d.x; sw[4 * c + 1] = d.y; sw[4 * c + 2] = d.z; sw[4 * c + 3] = d.w;
+  for (int q = 0; q < N; ++q) {
+    auto& sp = sm.sp[H::ST][q];
+    float (&acc)[24] = accs[q];
+    float w = In::scale_of(sm.sn[H::ST][q][tid]);
+    if constexpr (G::kScaled) {
+      if (!unit) w *= G::kScale;  // Q16 links come back as raw codes
     }
-    float psi[24], hs[12];
-    In::words(sw, psi);
-    project<MU, S>(psi, hs);
-    float gs[12];
-    su3_mul<!FWD>(u, hs, gs);
-    reconstruct_scaled<MU, S>(gs, acc, w);
-  } else {
-    constexpr bool upper = (S == +1);
-    uint32_t hw[6];
-    if constexpr (upper) {
-      const uint4 a = sm.sp[H::ST][0][tid];
-      const uint2 b = *reinterpret_cast<const uint2*>(&sm.sp[H::ST][1][tid]);
-      hw[0] = a.x; hw[1] = a.y; hw[2] = a.z; hw[3] = a.w; hw[4] = b.x; hw[5] = b.y;
-    } else {
-      const uint2 a = *reinterpret_cast<const uint2*>(&sm.sp[H::ST][0][tid]);
-      const uint4 b = sm.sp[H::ST][1][tid];
-      hw[0] = a.x; hw[1] = a.y; hw[2] = b.x; hw[3] = b.y; hw[4] = b.z; hw[5] = b.w;
-    }
-    float hs[12];
-    In::words_half(hw, hs);
-    const bool flip = g.tbc_anti && (FWD ? top : bot);
-    if (unit) {
-      accumulate_temporal<FWD, upper>(hs, acc, flip ? -2.f * w : 2.f * w);
-    } else {
+    if constexpr (MU < 3) {
+      uint32_t sw[12];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const uint4 d = sp[c][tid];
+        sw[4 * c] = d.x; sw[4 * c + 1] = d.y; sw[4 * c + 2] = d.z; sw[4 * c + 3] = d.w;
+      }
+      float psi[24], hs[12];
+      In::words(sw, psi);
+      project<MU, S>(psi, hs);
       float gs[12];
       su3_mul<!FWD>(u, hs, gs);
-      accumulate_temporal<FWD, upper>(gs, acc, flip ? -2.f * w : 2.f * w);
+      reconstruct_scaled<MU, S>(gs, acc, w);
+    } else {
+      constexpr bool upper = (S == +1);
+      uint32_t hw[6];
+      half_words<upper>(sp[0][tid], sp[1][tid], hw);
+      float hs[12];
+      In::words_half(hw, hs);
+      const bool flip = g.tbc_anti && (FWD ? top : bot);
+      if (unit) {
+        accumulate_temporal<FWD, upper>(hs, acc, flip ? -2.f * w : 2.f * w);
+      } else {
+        float gs[12];
+        su3_mul<!FWD>(u, hs, gs);
+        accumulate_temporal<FWD, upper>(gs, acc, flip ? -2.f * w : 2.f * w);
+      }
     }
   }
 }
@@ -231,15 +251,14 @@ __device__ __forceinline__ void reconstruct_pairs(const float2 (&gr)[3], const f
   }
 }
 
-template <int K, bool DAGGER, bool TFIX, class In, class G>
-__device__ __forceinline__ void async_hop_pairs(const AsyncSlots& sm, const Geom& g, bool top, bool bot,
-                                                float2 (&acc)[12]) {
+template <int K, bool DAGGER, bool TFIX, class In, class G, int N>
+__device__ __forceinline__ void async_hop_pairs(const AsyncSlotsN<N>& sm, const Geom& g, bool top, bool bot,
+                                                float2 (&accs)[N][12]) {
   using H = HopK<K>;
   constexpr int MU = H::MU;
   constexpr bool FWD = H::FWD;
   constexpr int S = (FWD != DAGGER) ? -1 : +1;
   const int tid = threadIdx.x;
-  float w = In::scale_of(sm.sn[H::ST][tid]);
   const bool unit = TFIX && MU == 3 && (FWD ? !top : !bot);
   float u[18];
   if (!unit) {
@@ -247,128 +266,120 @@ __device__ __forceinline__ void async_hop_pairs(const AsyncSlots& sm, const Geom
     const uint2 b = sm.l2[H::ST][tid];
     const uint32_t lw[6] = {a.x, a.y, a.z, a.w, b.x, b.y};
     G::from_words(lw, u);
-    if constexpr (G::kScaled) w *= G::kScale;  // Q16 links come back as raw codes
   }
-  float2 hr[3], hi[3];
-  if constexpr (MU < 3) {
-    uint32_t sw[12];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const uint4 d = sm.sp[H::ST][c][tid];
-      sw[4 * c] = d.x; sw[4 * c + 1] = d.y; sw[4 * c + 2] = d.z; sw[4 * c + 3] = d.w;
+  for (int q = 0; q < N; ++q) {
+    auto& sp = sm.sp[H::ST][q];
+    float2 (&acc)[12] = accs[q];
+    float w = In::scale_of(sm.sn[H::ST][q][tid]);
+    if constexpr (G::kScaled) {
+      if (!unit) w *= G::kScale;  // Q16 links come back as raw codes
     }
-    // project() on pairs: p = (spin 0, spin 1) and q = (spin 3, spin 2), or
-    // (spin 2, spin 3) for z; word s * 3 + c holds (re, im) of spin s, colour c
-    // (each word decoded whole, as the scalar path does: fp16 pairs convert
-    // in one instruction)
-    constexpr int qa = (MU == 2) ? 2 : 3, qb = (MU == 2) ? 3 : 2;
-    constexpr float s = (float)((MU == 1) ? -S : S);
-    if constexpr (In::kIntCodes) {
-      // integer codes are projected as integers, two dot products of a word (the
-      // codes (re, im)) with (+-1, 0) or (0, +-1) per value, and converted once:
-      // 24 + 12 instructions instead of 48 to decode 24 codes and 6 packed sums;
-      // all of it is exact either way
-      constexpr int si = (MU == 1) ? -S : S;
-      constexpr int re = 1, im = 1 << 8, nre = 0xff, nim = 0xff00;  // byte 0: the real code, byte 1: the imaginary
-      constexpr int pre = si > 0 ? re : nre, pim = si > 0 ? im : nim;    // + s
-      constexpr int mre = si > 0 ? nre : re, mim = si > 0 ? nim : im;    // - s
+    float2 hr[3], hi[3];
+    if constexpr (MU < 3) {
+      uint32_t sw[12];
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const int p0 = (int)sw[c], p1 = (int)sw[3 + c], a = (int)sw[qa * 3 + c], b = (int)sw[qb * 3 + c];
-        // row 0 with spin qa, row 1 with spin qb (the terms written out below)
-        constexpr int r0 = (MU == 1) ? mre : mim, i0 = (MU == 1) ? mim : pre;
-        constexpr int r1 = (MU == 0) ? mim : (MU == 1) ? pre : pim, i1 = (MU == 0) ? pre : (MU == 1) ? pim : mre;
-        hr[c] = make_float2(__int2float_rn(__dp2a_lo(a, r0, __dp2a_lo(p0, re, 0))),
-                            __int2float_rn(__dp2a_lo(b, r1, __dp2a_lo(p1, re, 0))));
-        hi[c] = make_float2(__int2float_rn(__dp2a_lo(a, i0, __dp2a_lo(p0, im, 0))),
-                            __int2float_rn(__dp2a_lo(b, i1, __dp2a_lo(p1, im, 0))));
+        const uint4 d = sp[c][tid];
+        sw[4 * c] = d.x; sw[4 * c + 1] = d.y; sw[4 * c + 2] = d.z; sw[4 * c + 3] = d.w;
       }
-    } else {
-      float2 pw[12];
+      // project() on pairs: p = (spin 0, spin 1) and q = (spin 3, spin 2), or
+      // (spin 2, spin 3) for z; word s * 3 + c holds (re, im) of spin s, colour c
+      // (each word decoded whole, as the scalar path does: fp16 pairs convert
+      // in one instruction)
+      constexpr int qa = (MU == 2) ? 2 : 3, qb = (MU == 2) ? 3 : 2;
+      constexpr float s = (float)((MU == 1) ? -S : S);
+      if constexpr (In::kIntCodes) {
+        // integer codes are projected as integers, two dot products of a word (the
+        // codes (re, im)) with (+-1, 0) or (0, +-1) per value, and converted once:
+        // 24 + 12 instructions instead of 48 to decode 24 codes and 6 packed sums;
+        // all of it is exact either way
+        constexpr int si = (MU == 1) ? -S : S;
+        constexpr int re = 1, im = 1 << 8, nre = 0xff, nim = 0xff00;  // byte 0: the real code, byte 1: the imaginary
+        constexpr int pre = si > 0 ? re : nre, pim = si > 0 ? im : nim;    // + s
+        constexpr int mre = si > 0 ? nre : re, mim = si > 0 ? nim : im;    // - s
 #pragma unroll
-      for (int j = 0; j < 12; ++j) pw[j] = In::pair(sw[j]);
+        for (int c = 0; c < 3; ++c) {
+          const int p0 = (int)sw[c], p1 = (int)sw[3 + c], a = (int)sw[qa * 3 + c], b = (int)sw[qb * 3 + c];
+          // row 0 with spin qa, row 1 with spin qb (the terms written out below)
+          constexpr int r0 = (MU == 1) ? mre : mim, i0 = (MU == 1) ? mim : pre;
+          constexpr int r1 = (MU == 0) ? mim : (MU == 1) ? pre : pim, i1 = (MU == 0) ? pre : (MU == 1) ? pim : mre;
+          hr[c] = make_float2(__int2float_rn(__dp2a_lo(a, r0, __dp2a_lo(p0, re, 0))),
+                              __int2float_rn(__dp2a_lo(b, r1, __dp2a_lo(p1, re, 0))));
+          hi[c] = make_float2(__int2float_rn(__dp2a_lo(a, i0, __dp2a_lo(p0, im, 0))),
+                              __int2float_rn(__dp2a_lo(b, i1, __dp2a_lo(p1, im, 0))));
+        }
+      } else {
+        float2 pw[12];
+#pragma unroll
+        for (int j = 0; j < 12; ++j) pw[j] = In::pair(sw[j]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const float2 pr = make_float2(pw[c].x, pw[3 + c].x);
+          const float2 pi = make_float2(pw[c].y, pw[3 + c].y);
+          const float2 qr = make_float2(pw[qa * 3 + c].x, pw[qb * 3 + c].x);
+          const float2 qi = make_float2(pw[qa * 3 + c].y, pw[qb * 3 + c].y);
+          if constexpr (MU == 0) {  // h0 = p0 + s i p3, h1 = p1 + s i p2
+            hr[c] = __ffma2_rn(dup2(-s), qi, pr);
+            hi[c] = __ffma2_rn(dup2(s), qr, pi);
+          } else if constexpr (MU == 1) {  // h0 = p0 - s p3, h1 = p1 + s p2
+            hr[c] = __ffma2_rn(make_float2(-s, s), qr, pr);
+            hi[c] = __ffma2_rn(make_float2(-s, s), qi, pi);
+          } else {  // h0 = p0 + s i p2, h1 = p1 - s i p3
+            hr[c] = __ffma2_rn(make_float2(-s, s), qi, pr);
+            hi[c] = __ffma2_rn(make_float2(s, -s), qr, pi);
+          }
+        }
+      }
+      float2 gr[3], gi[3];
+      su3_mul_pairs<!FWD>(u, hr, hi, gr, gi);
+      reconstruct_pairs<MU, S>(gr, gi, acc, w);
+    } else {
+      constexpr bool upper = (S == +1);
+      uint32_t hw[6];
+      half_words<upper>(sp[0][tid], sp[1][tid], hw);
+      // rows of the half spinor: (spin 0, spin 1) upper; (spin 3, spin 2) lower,
+      // the order of the accumulator pairs
+      constexpr int ra = upper ? 0 : 3, rb = upper ? 3 : 0;
+      float2 pw[6];
+#pragma unroll
+      for (int j = 0; j < 6; ++j) pw[j] = In::pair(hw[j]);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const float2 pr = make_float2(pw[c].x, pw[3 + c].x);
-        const float2 pi = make_float2(pw[c].y, pw[3 + c].y);
-        const float2 qr = make_float2(pw[qa * 3 + c].x, pw[qb * 3 + c].x);
-        const float2 qi = make_float2(pw[qa * 3 + c].y, pw[qb * 3 + c].y);
-        if constexpr (MU == 0) {  // h0 = p0 + s i p3, h1 = p1 + s i p2
-          hr[c] = __ffma2_rn(dup2(-s), qi, pr);
-          hi[c] = __ffma2_rn(dup2(s), qr, pi);
-        } else if constexpr (MU == 1) {  // h0 = p0 - s p3, h1 = p1 + s p2
-          hr[c] = __ffma2_rn(make_float2(-s, s), qr, pr);
-          hi[c] = __ffma2_rn(make_float2(-s, s), qi, pi);
-        } else {  // h0 = p0 + s i p2, h1 = p1 - s i p3
-          hr[c] = __ffma2_rn(make_float2(-s, s), qi, pr);
-          hi[c] = __ffma2_rn(make_float2(s, -s), qr, pi);
+        hr[c] = make_float2(pw[ra + c].x, pw[rb + c].x);
+        hi[c] = make_float2(pw[ra + c].y, pw[rb + c].y);
+      }
+      const bool flip = g.tbc_anti && (FWD ? top : bot);
+      const float2 t2 = dup2(flip ? -2.f * w : 2.f * w);
+      constexpr int o = upper ? 0 : 6;
+      if (unit) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          acc[o + 2 * c] = __ffma2_rn(t2, hr[c], acc[o + 2 * c]);
+          acc[o + 2 * c + 1] = __ffma2_rn(t2, hi[c], acc[o + 2 * c + 1]);
+        }
+      } else {
+        float2 gr[3], gi[3];
+        su3_mul_pairs<!FWD>(u, hr, hi, gr, gi);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          acc[o + 2 * c] = __ffma2_rn(t2, gr[c], acc[o + 2 * c]);
+          acc[o + 2 * c + 1] = __ffma2_rn(t2, gi[c], acc[o + 2 * c + 1]);
         }
       }
     }
-    float2 gr[3], gi[3];
-    su3_mul_pairs<!FWD>(u, hr, hi, gr, gi);
-    reconstruct_pairs<MU, S>(gr, gi, acc, w);
-  } else {
-    constexpr bool upper = (S == +1);
-    uint32_t hw[6];
-    if constexpr (upper) {
-      const uint4 a = sm.sp[H::ST][0][tid];
-      const uint2 b = *reinterpret_cast<const uint2*>(&sm.sp[H::ST][1][tid]);
-      hw[0] = a.x; hw[1] = a.y; hw[2] = a.z; hw[3] = a.w; hw[4] = b.x; hw[5] = b.y;
-    } else {
-      const uint2 a = *reinterpret_cast<const uint2*>(&sm.sp[H::ST][0][tid]);
-      const uint4 b = sm.sp[H::ST][1][tid];
-      hw[0] = a.x; hw[1] = a.y; hw[2] = b.x; hw[3] = b.y; hw[4] = b.z; hw[5] = b.w;
-    }
-    // rows of the half spinor: (spin 0, spin 1) upper; (spin 3, spin 2) lower,
-    // the order of the accumulator pairs
-    constexpr int ra = upper ? 0 : 3, rb = upper ? 3 : 0;
-    float2 pw[6];
-#pragma unroll
-    for (int j = 0; j < 6; ++j) pw[j] = In::pair(hw[j]);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      hr[c] = make_float2(pw[ra + c].x, pw[rb + c].x);
-      hi[c] = make_float2(pw[ra + c].y, pw[rb + c].y);
-    }
-    const bool flip = g.tbc_anti && (FWD ? top : bot);
-    const float2 t2 = dup2(flip ? -2.f * w : 2.f * w);
-    constexpr int o = upper ? 0 : 6;
-    if (unit) {
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        acc[o + 2 * c] = __ffma2_rn(t2, hr[c], acc[o + 2 * c]);
-        acc[o + 2 * c + 1] = __ffma2_rn(t2, hi[c], acc[o + 2 * c + 1]);
-      }
-    } else {
-      float2 gr[3], gi[3];
-      su3_mul_pairs<!FWD>(u, hr, hi, gr, gi);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        acc[o + 2 * c] = __ffma2_rn(t2, gr[c], acc[o + 2 * c]);
-        acc[o + 2 * c + 1] = __ffma2_rn(t2, gi[c], acc[o + 2 * c + 1]);
-      }
-    }
   }
 }
 
-template <int K, bool DAGGER, bool TFIX, class In, class G>
-__device__ __forceinline__ void async_step_pairs(AsyncSlots& sm, const Geom& g, const In& in, const G& gauge,
-                                                 int parity, int h, const int (&nb)[8], bool top, bool bot,
-                                                 float2 (&acc)[12]) {
+// hop K of a thread's site; A: the accumulators, spin pairs or plain
+template <int K, bool DAGGER, bool TFIX, int N, class In, class G, class A>
+__device__ __forceinline__ void async_step(AsyncSlotsN<N>& sm, const Geom& g, const In (&in)[N], const G& gauge,
+                                           int parity, int h, const int (&nb)[8], bool top, bool bot, A& acc) {
   if constexpr (K + 2 < 8) async_issue<K + 2, DAGGER, TFIX>(sm, in, gauge, parity, h, nb, top, bot);
   cp_commit();
   cp_wait<2>();  // the copies of hop K have landed
-  async_hop_pairs<K, DAGGER, TFIX, In, G>(sm, g, top, bot, acc);
-}
-
-template <int K, bool DAGGER, bool TFIX, class In, class G>
-__device__ __forceinline__ void async_step(AsyncSlots& sm, const Geom& g, const In& in, const G& gauge, int parity,
-                                           int h, const int (&nb)[8], bool top, bool bot, float (&acc)[24]) {
-  if constexpr (K + 2 < 8) async_issue<K + 2, DAGGER, TFIX>(sm, in, gauge, parity, h, nb, top, bot);
-  cp_commit();
-  cp_wait<2>();  // the copies of hop K have landed
-  async_hop<K, DAGGER, TFIX, In, G>(sm, g, top, bot, acc);
+  if constexpr (kSpinPairs && In::kPairedHops) async_hop_pairs<K, DAGGER, TFIX, In, G>(sm, g, top, bot, acc);
+  else async_hop<K, DAGGER, TFIX, In, G>(sm, g, top, bot, acc);
 }
 
 // spin pairs of the accumulator -> spinor order
@@ -385,11 +396,11 @@ __device__ __forceinline__ void from_pairs(const float2 (&a2)[12], float (&acc)[
   }
 }
 
-// acc = (D in)(h) (or D^dag), 16-bit spinors and 12-real 16-bit links; the
-// caller's block has kAsyncBlock threads.
-template <bool DAGGER, bool TFIX, class In, class G>
-__device__ __forceinline__ void dslash_site_async(const Geom& g, const In& in, const G& gauge, AsyncSlots& sm, int h,
-                                                  int parity, float (&acc)[24]) {
+// acc = (D in)(h) (or D^dag) for N right-hand sides, 16-bit spinors and 12-real
+// 16-bit links; the caller's block has kAsyncBlock threads.
+template <bool DAGGER, bool TFIX, int N, class In, class G>
+__device__ __forceinline__ void dslash_site_async(const Geom& g, const In (&in)[N], const G& gauge,
+                                                  AsyncSlotsN<N>& sm, int h, int parity, float (&acc)[N][24]) {
   int x, y, z, t;
   site_coords(g, h, parity, x, y, z, t);
   int nb[8];
@@ -399,58 +410,61 @@ __device__ __forceinline__ void dslash_site_async(const Geom& g, const In& in, c
   cp_commit();
   async_issue<1, DAGGER, TFIX>(sm, in, gauge, parity, h, nb, top, bot);
   cp_commit();
+  auto hops = [&](auto& a) {
+    async_step<0, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a);
+    async_step<1, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a);
+    async_step<2, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a);
+    async_step<3, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a);
+    async_step<4, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a);
+    async_step<5, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a);
+    async_step<6, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a);
+    async_step<7, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a);
+  };
   if constexpr (kSpinPairs && In::kPairedHops) {
-    float2 a2[12];
+    float2 a2[N][12];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) a2[k] = make_float2(0.f, 0.f);
-    async_step_pairs<0, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a2);
-    async_step_pairs<1, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a2);
-    async_step_pairs<2, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a2);
-    async_step_pairs<3, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a2);
-    async_step_pairs<4, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a2);
-    async_step_pairs<5, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a2);
-    async_step_pairs<6, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a2);
-    async_step_pairs<7, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, a2);
-    from_pairs(a2, acc);
-    return;
+    for (int q = 0; q < N; ++q)
+#pragma unroll
+      for (int k = 0; k < 12; ++k) a2[q][k] = make_float2(0.f, 0.f);
+    hops(a2);
+#pragma unroll
+    for (int q = 0; q < N; ++q) from_pairs(a2[q], acc[q]);
+  } else {
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+#pragma unroll
+      for (int k = 0; k < 24; ++k) acc[q][k] = 0.f;
+    hops(acc);
   }
-#pragma unroll
-  for (int k = 0; k < 24; ++k) acc[k] = 0.f;
-  async_step<0, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, acc);
-  async_step<1, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, acc);
-  async_step<2, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, acc);
-  async_step<3, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, acc);
-  async_step<4, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, acc);
-  async_step<5, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, acc);
-  async_step<6, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, acc);
-  async_step<7, DAGGER, TFIX>(sm, g, in, gauge, parity, h, nb, top, bot, acc);
 }
 
 // the two hops of direction MU alone: acc = their sum (dslash_sites_split)
 template <int MU, bool DAGGER, bool TFIX, class In, class G>
-__device__ __forceinline__ void direction_async(const Geom& g, const In& in, const G& gauge, AsyncSlots& sm, int h,
+__device__ __forceinline__ void direction_async(const Geom& g, const In (&in)[1], const G& gauge, AsyncSlots& sm, int h,
                                                 int parity, const int (&nb)[8], bool top, bool bot,
-                                                float (&acc)[24]) {
+                                                float (&acc)[1][24]) {
   async_issue<2 * MU, DAGGER, TFIX>(sm, in, gauge, parity, h, nb, top, bot);
   cp_commit();
   async_issue<2 * MU + 1, DAGGER, TFIX>(sm, in, gauge, parity, h, nb, top, bot);
   cp_commit();
-  if constexpr (kSpinPairs && In::kPairedHops) {
-    float2 a2[12];
-#pragma unroll
-    for (int k = 0; k < 12; ++k) a2[k] = make_float2(0.f, 0.f);
+  auto hops = [&](auto& a) {
     cp_wait<1>();
-    async_hop_pairs<2 * MU, DAGGER, TFIX, In, G>(sm, g, top, bot, a2);
+    if constexpr (kSpinPairs && In::kPairedHops) async_hop_pairs<2 * MU, DAGGER, TFIX, In, G>(sm, g, top, bot, a);
+    else async_hop<2 * MU, DAGGER, TFIX, In, G>(sm, g, top, bot, a);
     cp_wait<0>();
-    async_hop_pairs<2 * MU + 1, DAGGER, TFIX, In, G>(sm, g, top, bot, a2);
-    from_pairs(a2, acc);
+    if constexpr (kSpinPairs && In::kPairedHops) async_hop_pairs<2 * MU + 1, DAGGER, TFIX, In, G>(sm, g, top, bot, a);
+    else async_hop<2 * MU + 1, DAGGER, TFIX, In, G>(sm, g, top, bot, a);
+  };
+  if constexpr (kSpinPairs && In::kPairedHops) {
+    float2 a2[1][12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) a2[0][k] = make_float2(0.f, 0.f);
+    hops(a2);
+    from_pairs(a2[0], acc[0]);
   } else {
 #pragma unroll
-    for (int k = 0; k < 24; ++k) acc[k] = 0.f;
-    cp_wait<1>();
-    async_hop<2 * MU, DAGGER, TFIX, In, G>(sm, g, top, bot, acc);
-    cp_wait<0>();
-    async_hop<2 * MU + 1, DAGGER, TFIX, In, G>(sm, g, top, bot, acc);
+    for (int k = 0; k < 24; ++k) acc[0][k] = 0.f;
+    hops(acc);
   }
 }
 

@@ -499,6 +499,61 @@ __global__ void __launch_bounds__(kDslashBlock, (DslashOccupancy<R, In, Epi::NRE
   }
 }
 
+// The same for 16-bit storage with two systems per thread (blockIdx.y names a
+// pair): they share the link with its decoding and rebuilding, the addresses and
+// the loop, a third of a hop's instructions, and a thread has twice the
+// independent work to cover its latencies with.  A system without an active
+// partner is computed alone.
+// 128 x 4 threads of the 48 KB ring fit an SM; the fp16 temporal-gauge hops
+// spill there and are 1-2 % faster at 3 blocks, the others 2-5 % at 4.
+template <class In, int NRED, bool TFIX>
+struct PairOccupancy {
+  static constexpr int kMinBlocks = (TFIX && !In::kPairedHops) ? 3 : 4;
+};
+template <bool DAGGER, bool TFIX, class In, class G, class Epi>
+__global__ void __launch_bounds__(kDslashBlock, (PairOccupancy<In, Epi::NRED, TFIX>::kMinBlocks))
+    dslash_rhs_pair_kernel(Geom g, In in, G gauge, int parity, Epi epi, BatchArgs ba) {
+  pdl_wait();
+  constexpr int NR = Epi::NRED > 0 ? Epi::NRED : 1;
+  // the ring takes all 48 KB of static shared memory: the sums go over it
+  __shared__ __align__(16) unsigned char smem[sizeof(AsyncSlotsN<2>)];
+  static_assert(NR * kDslashBlock * sizeof(double) <= sizeof(smem), "the sums lie over the ring");
+  const int r0 = 2 * blockIdx.y;
+  const bool a0 = rhs_active(ba, r0), a1 = rhs_active(ba, r0 + 1);  // uniform over the block
+  auto sites = [&](auto nt, int r) {
+    constexpr int N = decltype(nt)::value;
+    AsyncSlotsN<N>& sm = *reinterpret_cast<AsyncSlotsN<N>*>(smem);
+    In ins[N];
+    double red[N][NR];
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      ins[q] = in.at(r + q);
+#pragma unroll
+      for (int k = 0; k < NR; ++k) red[q][k] = 0.0;
+    }
+    const In(&cins)[N] = ins;
+    for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < g.Vh; h += gridDim.x * blockDim.x) {
+      float acc[N][24];
+      dslash_site_async<DAGGER, TFIX>(g, cins, gauge, sm, h, parity, acc);
+#pragma unroll
+      for (int q = 0; q < N; ++q) epi.at(r + q)(h, acc[q], red[q]);
+    }
+    if constexpr (Epi::NRED > 0) {
+      double* const rsm = reinterpret_cast<double*>(smem);
+#pragma unroll
+      for (int q = 0; q < N; ++q) {
+        __syncthreads();  // every copy into the ring has been waited for and read
+        block_sum<NR, kDslashBlock>(red[q], rsm);
+        if (threadIdx.x == 0)
+#pragma unroll
+          for (int k = 0; k < NR; ++k) ba.partials[((size_t)(r + q) * NR + k) * gridDim.x + blockIdx.x] = red[q][k];
+      }
+    }
+  };
+  if (a0 && a1) sites(std::integral_constant<int, 2>{}, r0);
+  else if (a0 || a1) sites(std::integral_constant<int, 1>{}, a0 ? r0 : r0 + 1);
+}
+
 // Site kernel over a batch: blockIdx.y is the right-hand side.
 template <class Op>
 __global__ void __launch_bounds__(kBlasBlock) site_batch_kernel(int n, Op op, BatchArgs ba) {
@@ -586,8 +641,9 @@ struct BatchLaunch {
   int grid;     // multi-RHS dslash blocks (tr = 0: blocks per system), inner precision
   int blas_gx;  // site-kernel blocks per right-hand side
   int grid64 = 0;    // FP64 dslash (dslash_rhs_kernel): blocks per system; 0 = grid
-  int pack = 0;      // 1: two systems per thread in FP32x2 registers (tr = 2, 4, 8
-                     // systems per chunk: tr / 2 thread rows), FP32 / 16-bit storage
+  int pack = 0;      // 1: two systems per thread, in FP32x2 registers (tr = 2, 4, 8
+                     // systems per chunk: tr / 2 thread rows; FP32 / 16-bit storage)
+                     // or a pair per block row (tr = 0; 16-bit storage, not with 8-real links)
 };
 
 // blocks per system of the FP64 per-system dslash: the single-system grid
@@ -612,6 +668,19 @@ void launch_dslash_mrhs(const Geom& g, const BatchLaunch& bl, const In& in, cons
     }
   }
   const int grid = mrhs_grid<R>(bl);
+  if constexpr (UseAsync<In, false>::value) {
+    if (bl.tr == 0 && bl.pack && gauge.recon != 8) {
+      auto pair = [&](auto dag, auto tfix) {
+        launch_pdl(dslash_rhs_pair_kernel<decltype(dag)::value, decltype(tfix)::value, In, G, Epi>,
+                   dim3(grid, (bl.nrhs + 1) / 2), dim3(kDslashBlock), 0, s, g, in, gauge, parity, epi, ba);
+      };
+      pick_dagger(dagger, [&](auto dag) {
+        if (g.tfix) pair(dag, std::true_type{});
+        else pair(dag, std::false_type{});
+      });
+      return;
+    }
+  }
   if (sizeof(R) == 8 || bl.tr == 0) {
     const dim3 gr(grid, bl.nrhs);
     auto go = [&](auto dag, auto tfix, auto rec8) {

@@ -648,10 +648,12 @@ __device__ __forceinline__ void dslash_sites_split(const Geom& g, const In& in, 
       neighbours(g, h, x, y, z, t, nb);
       const bool top = (t == g.T - 1), bot = (t == 0);
       if constexpr (UseAsync<In, R8>::value) {
-        if (w == 0) direction_async<0, DAGGER, TFIX>(g, in, gauge, *slots, h, parity, nb, top, bot, acc);
-        else if (w == 1) direction_async<1, DAGGER, TFIX>(g, in, gauge, *slots, h, parity, nb, top, bot, acc);
-        else if (w == 2) direction_async<2, DAGGER, TFIX>(g, in, gauge, *slots, h, parity, nb, top, bot, acc);
-        else direction_async<3, DAGGER, TFIX>(g, in, gauge, *slots, h, parity, nb, top, bot, acc);
+        const In ins[1] = {in};
+        float (&a)[1][24] = reinterpret_cast<float (&)[1][24]>(acc);
+        if (w == 0) direction_async<0, DAGGER, TFIX>(g, ins, gauge, *slots, h, parity, nb, top, bot, a);
+        else if (w == 1) direction_async<1, DAGGER, TFIX>(g, ins, gauge, *slots, h, parity, nb, top, bot, a);
+        else if (w == 2) direction_async<2, DAGGER, TFIX>(g, ins, gauge, *slots, h, parity, nb, top, bot, a);
+        else direction_async<3, DAGGER, TFIX>(g, ins, gauge, *slots, h, parity, nb, top, bot, a);
       } else {
 #pragma unroll
         for (int k = 0; k < 24; ++k) acc[k] = 0.f;
@@ -702,9 +704,10 @@ __device__ __forceinline__ void dslash_sites(const Geom& g, const In& in, const 
                                            parity, epi, red);
     } else {
       for (int h = h_begin + blockIdx.x * blockDim.x + threadIdx.x; h < h_end; h += gridDim.x * blockDim.x) {
-        R acc[24];
-        dslash_site_async<DAGGER, TFIX>(g, in, gauge, sm, h, parity, acc);
-        epi(h, acc, red);
+        const In ins[1] = {in};
+        R acc[1][24];
+        dslash_site_async<DAGGER, TFIX>(g, ins, gauge, sm, h, parity, acc);
+        epi(h, acc[0], red);
       }
     }
   } else if constexpr (SPLIT) {

@@ -139,6 +139,9 @@ std::string tune_key(const Ctx& c, int n, int prec) {
   return k.str();
 }
 
+// dslash_rhs_pair_kernel takes this precision and link format
+bool has_pairs(const Ctx& c, int prec) { return prec >= WD_Q16 && c.low_recon != 8; }
+
 // Autotuner: time the multi-RHS inner-precision dslash for every (RHS tile,
 // grid) candidate on the batch's own fields and keep the fastest.
 wd_status tune_batch(wd_ctx* ctx, int n, int prec, BatchBufs& b) {
@@ -157,7 +160,7 @@ wd_status tune_batch(wd_ctx* ctx, int n, int prec, BatchBufs& b) {
         const bool shape = static_cast<bool>(v >> tr >> grid);
         if (shape && !(v >> pack)) pack = 0;  // entries without the layout field: one system per thread
         if (shape && (tr == 0 || tr == 1 || tr == 2 || tr == 4 || tr == 8) && grid > 0 &&
-            (pack == 0 || (pack == 1 && tr >= 2 && prec != WD_F64))) {
+            (pack == 0 || (pack == 1 && tr >= 2 && prec != WD_F64) || (pack == 1 && tr == 0 && has_pairs(c, prec)))) {
           c.batch_tr = tr ? tr : -1;
           c.batch_grid = grid;
           c.batch_pack = pack;
@@ -177,12 +180,12 @@ wd_status tune_batch(wd_ctx* ctx, int n, int prec, BatchBufs& b) {
   float best = 1e30f;
   int best_tr = 4, best_grid = c.num_sms * 4, best_pack = 0;
   // block shapes and register layouts: tr 0 is one system per block row (128
-  // sites per block); tr 1..8 systems per 32-site link tile, one system per
-  // thread, or (pack) two systems per thread in FP32x2 registers, tr / 2
-  // thread rows
-  const int trs[8] = {0, 1, 2, 4, 8, 2, 4, 8};
-  const int packs[8] = {0, 0, 0, 0, 0, 1, 1, 1};
-  const int ncand = prec == WD_F64 ? 5 : 8;
+  // sites per block), or (pack) a pair of them; tr 1..8 systems per 32-site
+  // link tile, one system per thread, or (pack) two systems per thread in
+  // FP32x2 registers, tr / 2 thread rows
+  const int trs[9] = {0, 1, 2, 4, 8, 2, 4, 8, 0};
+  const int packs[9] = {0, 0, 0, 0, 0, 1, 1, 1, 1};
+  const int ncand = prec == WD_F64 ? 5 : (n > 1 && has_pairs(c, prec)) ? 9 : 8;
   const int mults[4] = {2, 4, 8, 16};
   const int nblk128 = (c.g.Vh + kDslashBlock - 1) / kDslashBlock;
   for (int ti = 0; ti < ncand; ++ti) {
@@ -227,7 +230,32 @@ BatchLaunch launch_shape(const Ctx& c, int n) {
                  blas_gx(c, n)};
   if (bl.tr && bl.grid > ntiles) bl.grid = ntiles;
   bl.grid64 = rhs_grid64(c.g, c.num_sms);
-  bl.pack = (c.batch_tr > 0) ? c.batch_pack : 0;
+  bl.pack = c.batch_tr ? c.batch_pack : 0;
+  return bl;
+}
+
+// Shape of wd_dslash_batch when no batched solve has tuned one.  Measured cold on
+// 24^3x64 and 16^3x32, 2, 3, 5 and 12 systems, both link gauges, against four
+// systems per tile and four blocks per SM for every case (in brackets):
+// 16-bit storage takes pairs, 12 systems of 24^3x64 in 267 us fp16 (285),
+// 247 Q16 (300), 227 bf16 (288), two in 51, 49 and 45 (113, 117, 113), and one
+// system per block row where the pairs would be under two waves of four blocks
+// per SM (8^3x16, 12 systems: 9 us for 10; 16^3x32, three: equal).  FP32 takes
+// two systems per tile, which read a link once for two, where eight such blocks
+// per SM find work: 12 systems 285 us (486), five 155 (320); with fewer systems or
+// tiles one per block row: two 74 us (202).
+BatchLaunch dslash_shape(const Ctx& c, int n, int prec) {
+  const int ntiles = (c.g.Vh + 31) / 32, nblk = (c.g.Vh + kDslashBlock - 1) / kDslashBlock;
+  BatchLaunch bl{n, 4, std::min(c.num_sms * 4, ntiles), blas_gx(c, n)};
+  if (prec == WD_F64 || c.low_recon == 8) return bl;
+  if (prec == WD_F32 && n >= 4 && ntiles >= 8 * c.num_sms) {
+    bl.tr = 2;
+    bl.grid = 8 * c.num_sms;
+    return bl;
+  }
+  bl.tr = 0;
+  bl.grid = std::min(nblk, 16 * c.num_sms);
+  bl.pack = has_pairs(c, prec) && n > 1 && (long)nblk * ((n + 1) / 2) >= 8 * c.num_sms;
   return bl;
 }
 
@@ -456,14 +484,13 @@ wd_status wd_dslash_batch(wd_ctx* ctx, void* out, const void* in, int nrhs, wd_p
   WB_CK(ctx, cudaSetDevice(c.device));
   wd_status st = wd_internal_ensure_gauge(ctx, prec);
   if (st != WD_OK) return st;
-  BatchLaunch bl{nrhs, 4, c.num_sms * 4, blas_gx(c, nrhs)};
+  BatchLaunch bl = dslash_shape(c, nrhs, prec);
   if (c.batch_tr && c.batch_n == nrhs && c.batch_prec == prec) {
+    const int ntiles = (c.g.Vh + 31) / 32;
     bl.tr = std::max(c.batch_tr, 0);
-    bl.grid = c.batch_grid;
-    bl.pack = c.batch_tr > 0 ? c.batch_pack : 0;
+    bl.grid = bl.tr ? std::min(c.batch_grid, ntiles) : c.batch_grid;
+    bl.pack = c.batch_pack;
   }
-  const int ntiles = (c.g.Vh + 31) / 32;
-  if (bl.tr && bl.grid > ntiles) bl.grid = ntiles;
   prec_ops(prec)->dslash_batch(c, bl, out, in, out_parity, dagger ? 1 : 0, c.stream);
   WB_CK_LAUNCH(ctx);
   return WD_OK;
