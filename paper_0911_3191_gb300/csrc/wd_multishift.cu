@@ -60,6 +60,21 @@ wd_status merr(wd_ctx* ctx, wd_status st, const std::string& m) {
 
 // (<a, b>, |a|^2) with <a, b> = sum_sites conj(a) . b: per-site partials in
 // FP32, the sites summed in FP64
+__device__ __forceinline__ void dot_norm(const float (&av)[24], const float (&bv)[24], double* red) {
+  float re = 0.f, im = 0.f, nn = 0.f;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    re += av[2 * k] * bv[2 * k];
+    re += av[2 * k + 1] * bv[2 * k + 1];
+    im += av[2 * k] * bv[2 * k + 1];
+    im -= av[2 * k + 1] * bv[2 * k];
+    nn += av[2 * k] * av[2 * k];
+    nn += av[2 * k + 1] * av[2 * k + 1];
+  }
+  red[0] += (double)re;
+  red[1] += (double)im;
+  red[2] += (double)nn;
+}
 struct OpDotNormF32 {
   static constexpr int NRED = 3;
   SpinorF32 a, b;
@@ -69,40 +84,7 @@ struct OpDotNormF32 {
     float av[24], bv[24];
     a.load(h, av);
     b.load(h, bv);
-    float re = 0.f, im = 0.f, nn = 0.f;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      re += av[2 * k] * bv[2 * k];
-      re += av[2 * k + 1] * bv[2 * k + 1];
-      im += av[2 * k] * bv[2 * k + 1];
-      im -= av[2 * k + 1] * bv[2 * k];
-      nn += av[2 * k] * av[2 * k];
-      nn += av[2 * k + 1] * av[2 * k + 1];
-    }
-    red[0] += (double)re;
-    red[1] += (double)im;
-    red[2] += (double)nn;
-  }
-};
-
-// out = a - c b (complex c)
-struct OpSubScaledF32 {
-  static constexpr int NRED = 0;
-  SpinorF32 out, a, b;
-  float cr, ci;
-  __device__ __forceinline__ void operator()(int h, double*) const {
-    float av[24], bv[24];
-    a.load(h, av);
-    b.load(h, bv);
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      const float br = bv[2 * k], bi = bv[2 * k + 1];
-      av[2 * k] -= cr * br;
-      av[2 * k] += ci * bi;
-      av[2 * k + 1] -= cr * bi;
-      av[2 * k + 1] -= ci * br;
-    }
-    out.store_f(h, av);
+    dot_norm(av, bv, red);
   }
 };
 
@@ -181,12 +163,12 @@ struct FinMsSetup {
   }
 };
 
-// alpha = rho / <r_tilde, v>  (t = {<v, r_tilde>, |v|^2})
+// alpha = rho / <r_tilde, v>  (t = {<r_tilde, v>})
 struct FinMsAlpha {
   MsCtl* m;
   __device__ void operator()(const double* t) const {
     if (m->failed) return;
-    const double2 rtv = c_conj(make_double2(t[0], t[1]));
+    const double2 rtv = make_double2(t[0], t[1]);
     if (!cfinite(rtv)) { ms_fail(m, WD_ERR_NUMERIC); return; }
     if (c_abs(rtv) == 0.0 || c_abs(m->rho) == 0.0) { ms_fail(m, WD_ERR_BREAKDOWN); return; }
     m->alpha = cdiv(m->rho, rtv);
@@ -209,11 +191,18 @@ struct FinMsOmega {
 
 // end of iteration (t = {<r_new, r_tilde>, |r_new|^2}): beta, the shifted
 // recurrences and update coefficients of every active shift, retirement of
-// converged shifts, the stop test of the seed
+// converged shifts, the stop test of the seed; then the loop condition (the
+// shift update still runs), with the body count bounded on its own
+// (max_iter + 16 executions)
 struct FinMsIter {
   MsCtl* m;
   __device__ void operator()(const double* t) const {
-    if (m->failed) return;
+    if (!m->failed) step(t);
+    m->loops += 1;
+    if (m->loops > m->max_iter + 16 && !m->done) ms_fail(m, WD_ERR_NOT_CONVERGED);
+    if (m->in_graph) cudaGraphSetConditional((cudaGraphConditionalHandle)m->h_loop, m->done ? 0u : 1u);
+  }
+  __device__ void step(const double* t) const {
     m->iters += 1;
     const double2 rho_new = c_conj(make_double2(t[0], t[1]));
     const double rn = sqrt(t[2]);
@@ -272,8 +261,39 @@ struct OpSubScaledMs {
   const double2* c;
   const MsCtl* m;
   __device__ __forceinline__ void operator()(int h, double*) const {
-    if (m->failed) return;
-    OpSubScaledF32{out, a, b, (float)c->x, (float)c->y}(h, nullptr);
+    float av[24];
+    if (!m->failed) sub(h, av);
+  }
+  __device__ __forceinline__ void sub(int h, float (&av)[24]) const {
+    float bv[24];
+    const float cr = (float)c->x, ci = (float)c->y;
+    a.load(h, av);
+    b.load(h, bv);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const float br = bv[2 * k], bi = bv[2 * k + 1];
+      av[2 * k] -= cr * br;
+      av[2 * k] += ci * bi;
+      av[2 * k + 1] -= cr * bi;
+      av[2 * k + 1] -= ci * br;
+    }
+    out.store_f(h, av);
+  }
+};
+
+// r_new = s - omega t with (<r_new, r_tilde>, |r_new|^2) of what it stores
+struct OpSubDotMs {
+  static constexpr int NRED = 3;
+  OpSubScaledMs u;
+  SpinorF32 rt;
+  FinMsIter fin;
+  RedScratch rs;
+  __device__ __forceinline__ void operator()(int h, double* red) const {
+    if (u.m->failed) return;
+    float av[24], bv[24];
+    u.sub(h, av);
+    rt.load(h, bv);
+    dot_norm(av, bv, red);
   }
 };
 
@@ -283,6 +303,7 @@ struct OpSubScaledMs {
 // finaliser wrote; then r <- r_new for the next iteration.
 __global__ void __launch_bounds__(kBlasBlock) shift_update_kernel(int n, SpinorF32 xs, SpinorF32 ps, SpinorF32 r,
                                                                   SpinorF32 r_new, SpinorF32 s, const MsCtl* m) {
+  pdl_wait();
   if (m->failed) return;
   const int nshift = m->n;
   const int stride = r.stride;
@@ -311,14 +332,6 @@ __global__ void __launch_bounds__(kBlasBlock) shift_update_kernel(int n, SpinorF
       r.p[o] = nv;
     }
   }
-}
-
-// last node of the WHILE body: continue while not done; the body count is
-// bounded here on its own (max_iter + 16 executions)
-__global__ void ms_loop_control_kernel(MsCtl* m) {
-  m->loops += 1;
-  if (m->loops > m->max_iter + 16 && !m->done) ms_fail(m, WD_ERR_NOT_CONVERGED);
-  if (m->in_graph) cudaGraphSetConditional((cudaGraphConditionalHandle)m->h_loop, m->done ? 0u : 1u);
 }
 
 // one block: the control block is zeroed word by word in place (a local
@@ -428,25 +441,26 @@ wd_status family_solve(wd_ctx* ctx, const void* src, double kappa_s, const std::
   MS_CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
   {
     const int gx = std::min((g.Vh + kBlasBlock - 1) / kBlasBlock, c.num_sms * 8);
-    auto apply_B = [&](void* out, const void* in) {  // out = M_hat(kappa_s) in
-      o32->dslash(c, f.todd, in, 1, 0, cs);
-      o32->dslash_xpay(c, out, f.todd, in, -kappa_s * kappa_s, nullptr, 0, 0, cs);
-    };
-    apply_B(f.v, f.ps);  // v = B p_0
-    launch_sites(c, g.Vh, OpDotNormMs<FinMsAlpha>{OpDotNormF32{V(f.v), V(f.rt), c.red, FinStore{nullptr, 0}},
-                                                  FinMsAlpha{m}, c.red},
-                 cs);
+    // out = M_hat(kappa_s) in, the second half-step with the reduction that
+    // follows in its epilogue.  With a launch of its own per reduction, for the
+    // loop condition and for r_new's products an iteration had eleven launches
+    // and read four fields more.
+    using S32 = SpinorF32;
+    const auto G32 = Tr<WD_F32>::gauge(c);
+    const Coef nk2{-kappa_s * kappa_s, nullptr};
+    auto hop = [&](const void* in) { o32->dslash(c, f.todd, in, 1, 0, cs); };
+    hop(f.ps);  // v = B p_0
+    launch_dslash<float>(c, V(f.todd), G32, 0, kPlain,
+                         EpiXpayDot<S32, S32, S32, FinMsAlpha>{V(f.v), V(f.ps), V(f.rt), nk2, c.red, FinMsAlpha{m}},
+                         cs);
     launch_sites(c, g.Vh, OpSubScaledMs{V(f.s), V(f.r), V(f.v), &m->alpha, m}, cs);  // s = r - alpha v
-    apply_B(f.t, f.s);                                                              // t = B s
-    launch_sites(c, g.Vh, OpDotNormMs<FinMsOmega>{OpDotNormF32{V(f.t), V(f.s), c.red, FinStore{nullptr, 0}},
-                                                  FinMsOmega{m}, c.red},
-                 cs);
-    launch_sites(c, g.Vh, OpSubScaledMs{V(f.rn), V(f.s), V(f.t), &m->omega, m}, cs);  // r_new = s - omega t
-    launch_sites(c, g.Vh, OpDotNormMs<FinMsIter>{OpDotNormF32{V(f.rn), V(f.rt), c.red, FinStore{nullptr, 0}},
-                                                 FinMsIter{m}, c.red},
-                 cs);
-    shift_update_kernel<<<gx, kBlasBlock, 0, cs>>>(g.Vh, V(f.xs, fb), V(f.ps, fb), V(f.r), V(f.rn), V(f.s), m);
-    ms_loop_control_kernel<<<1, 1, 0, cs>>>(m);
+    hop(f.s);                                                                       // t = B s
+    launch_dslash<float>(c, V(f.todd), G32, 0, kPlain,
+                         EpiXpayTS<S32, S32, FinMsOmega>{V(f.t), V(f.s), nk2, c.red, FinMsOmega{m}}, cs);
+    launch_sites(c, g.Vh,
+                 OpSubDotMs{OpSubScaledMs{V(f.rn), V(f.s), V(f.t), &m->omega, m}, V(f.rt), FinMsIter{m}, c.red}, cs);
+    launch_pdl(shift_update_kernel, dim3(gx), dim3(kBlasBlock), 0, cs, g.Vh, V(f.xs, fb), V(f.ps, fb), V(f.r),
+               V(f.rn), V(f.s), (const MsCtl*)m);
   }
   const cudaError_t ce = cudaStreamEndCapture(cs, &unused);
   cudaStreamDestroy(cs);
@@ -457,7 +471,7 @@ wd_status family_solve(wd_ctx* ctx, const void* src, double kappa_s, const std::
   MS_CK(cudaMemcpyAsync(&hm, m, sizeof(MsCtl), cudaMemcpyDeviceToHost, st));
   MS_CK(cudaStreamSynchronize(st));
   iters = hm.iters;
-  launches += (long long)hm.loops * 11;
+  launches += (long long)hm.loops * 7;
   if (hm.failed) {
     const char* what = hm.status == WD_ERR_BREAKDOWN ? "multi-shift: breakdown" : "multi-shift: NaN/Inf";
     return merr(ctx, (wd_status)(hm.status ? hm.status : WD_ERR_NUMERIC), what);
