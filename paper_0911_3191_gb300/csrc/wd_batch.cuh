@@ -556,7 +556,7 @@ __global__ void __launch_bounds__(kDslashBlock, (PairOccupancy<In, Epi::NRED, TF
 
 // Site kernel over a batch: blockIdx.y is the right-hand side.
 template <class Op>
-__global__ void __launch_bounds__(kBlasBlock) site_batch_kernel(int n, Op op, BatchArgs ba) {
+__global__ void __launch_bounds__(kBlasBlock, SiteOccupancy<Op>::kMinBlocks) site_batch_kernel(int n, Op op, BatchArgs ba) {
   pdl_wait();
   constexpr int NR = Op::NRED > 0 ? Op::NRED : 1;
   const int r = blockIdx.y;

@@ -168,6 +168,74 @@ __device__ __forceinline__ float fx_max(float m, unsigned a, unsigned b) {
 // the biased exponent of the double whose high word gave m, plus 1
 __device__ __forceinline__ int fx_exponent(float m) { return (int)(__float_as_uint(m) >> 20) + 1; }
 
+// ------------------------------------------------------ products of two sites
+// Inner products of a site's 24 doubles in integers, for kernels that the FP64
+// pipe bounds.  A vector becomes integers of 58 bits in the unit of its largest
+// exponent, each split into two signed halves; a product is three 32-bit
+// multiply-adds (12 cycles or so of an SM quarter, an FP64 one 67), the product of
+// the low halves (2^-58 of the two largest components' product) dropped, and a
+// site's 24 products are added exactly.  Cutting, dropping and rounding leave less
+// than FP64 products and sums do.
+constexpr int kFxSiteMinExp = 600, kFxSiteMaxExp = 1500;  // (biased) squares and scales stay normal doubles
+// biased exponent of the largest of 24 doubles; 24 zeros, as most sites of a point
+// source are, count as in range
+__device__ __forceinline__ int fx_site_exp(const double (&x)[24]) {
+  float m = 0.f;
+#pragma unroll
+  for (int k = 0; k < 24; k += 2) m = fx_max(m, (unsigned)__double2hiint(x[k]), (unsigned)__double2hiint(x[k + 1]));
+  if (__float_as_uint(m) == 0u) {
+    unsigned lo = 0u;
+#pragma unroll
+    for (int k = 0; k < 24; ++k) lo |= (unsigned)__double2loint(x[k]);
+    return lo ? 0 : kFxSiteMinExp;
+  }
+  return (int)(__float_as_uint(m) >> 20);
+}
+__device__ __forceinline__ bool fx_site_ok(int e) { return e >= kFxSiteMinExp && e <= kFxSiteMaxExp; }
+struct FxSite {
+  int h[24], l[24];  // x 2^(1080-e) = h 2^29 + l
+  int e;
+  __device__ __forceinline__ FxSite(const double (&x)[24], int e) : e(e) {
+#pragma unroll
+    for (int k = 0; k < 24; ++k) {
+      const long long v =
+          fx_number((unsigned)__double2loint(x[k]), (unsigned)__double2hiint(x[k]), e + 6, 0) + (1 << 28);
+      h[k] = (int)(v >> 29);
+      l[k] = ((int)v & ((1 << 29) - 1)) - (1 << 28);
+    }
+  }
+};
+struct FxSum {
+  long long hh = 0, hl = 0;
+  __device__ __forceinline__ void add(int ah, int al, int bh, int bl) {
+    hh = fx_mad(ah, bh, hh);
+    hl = fx_mad(ah, bl, hl);
+    hl = fx_mad(al, bh, hl);
+  }
+  __device__ __forceinline__ double value(int ea, int eb) const {
+    const long long t = hh + ((hl + (1 << 28)) >> 29);
+    return (double)t * __hiloint2double((ea + eb - 1079) << 20, 0);  // 2^(ea+eb-2102)
+  }
+};
+// |a|^2 and <w, a> = sum conj(w) a
+__device__ __forceinline__ double fx_norm2(const FxSite& a) {
+  FxSum n;
+#pragma unroll
+  for (int k = 0; k < 24; ++k) n.add(a.h[k], a.l[k], a.h[k], a.l[k]);
+  return n.value(a.e, a.e);
+}
+__device__ __forceinline__ double2 fx_dot(const FxSite& w, const FxSite& a) {
+  FxSum re, im;
+#pragma unroll
+  for (int k = 0; k < 24; k += 2) {
+    re.add(w.h[k], w.l[k], a.h[k], a.l[k]);
+    re.add(w.h[k + 1], w.l[k + 1], a.h[k + 1], a.l[k + 1]);
+    im.add(w.h[k], w.l[k], a.h[k + 1], a.l[k + 1]);
+    im.add(-w.h[k + 1], -w.l[k + 1], a.h[k], a.l[k]);
+  }
+  return make_double2(re.value(w.e, a.e), im.value(w.e, a.e));
+}
+
 __device__ __forceinline__ int fixed_neighbour(const Geom& g, int h, int x, int y, int z, int t, int k) {
   switch (k) {
     case 0: return (x == g.X - 1) ? h - (g.Xh - 1) : h + (x & 1);

@@ -110,3 +110,42 @@ def test_not_finite(bad):
         assert (test(out[0]) == test(out[1])).all()
     fine = np.isfinite(out[1])
     assert rel_err(out[0][fine], out[1][fine]) <= TOL_REL
+
+
+@pytest.mark.parametrize("exp2", [-100, 100])
+@pytest.mark.parametrize("point", [False, True])
+def test_solver_products_keep_every_digit_under_scaling(exp2, point):
+    """The FP64 BiCGstab takes the norm of r and its product with r_tilde from integers
+    in the unit of each site's largest component; sites without an exponent (zero) and
+    outside the range are told apart.  Scaled by a power of two every digit stays."""
+    wdp = _wd()
+    U = li.gauge(DIMS, 0.4, 1020)
+    b = li.point_source(DIMS, (1, 2, 3, 4), 1, 2) if point else li.gaussian_spinor(DIMS, 1021)
+    wd = wdp.WilsonDirac(DIMS)
+    wd.load_gauge(U)
+    xs, iters = [], []
+    for k in (0, exp2):
+        x = np.zeros_like(b)
+        info = wd.solve(x, b * 2.0 ** k, 0.12, tol=1e-10, solver=wdp.BICGSTAB, inner_precision=wdp.F64)
+        xs.append(x * 2.0 ** -k)
+        iters.append(info.iters)
+        rel = oracle.true_residual(xs[-1], b, U, DIMS, 0.12)
+        assert info.status == 0 and rel <= 1e-10, (k, info, rel)
+    assert iters[0] == iters[1] and np.array_equal(xs[0], xs[1])
+    wd.close()
+
+
+def test_solver_products_of_uneven_sites():
+    """Sites 2^-500 of the rest are outside the integers' range and take the FP64
+    products; the solve is that of the source without them to its rounding."""
+    wdp = _wd()
+    U = li.gauge(DIMS, 0.4, 1022)
+    b = li.gaussian_spinor(DIMS, 1023)
+    b[::3] *= 2.0 ** -500
+    wd = wdp.WilsonDirac(DIMS)
+    wd.load_gauge(U)
+    x = np.zeros_like(b)
+    info = wd.solve(x, b, 0.12, tol=1e-10, solver=wdp.BICGSTAB, inner_precision=wdp.F64)
+    rel = oracle.true_residual(x, b, U, DIMS, 0.12)
+    assert info.status == 0 and rel <= 1e-10, (info, rel)
+    wd.close()
