@@ -1146,7 +1146,10 @@ __device__ __forceinline__ void partial_sum(const double* p, int n, size_t ks, s
 }
 
 // All threads of the block (B of them) call this once, after their grid-stride
-// loop.  fin(const double* totals) runs on one thread of the last block.
+// loop.  The ticket is the release of this block's partials and, for the last
+// block, the acquire of the others' (the barrier hands it to its threads): two
+// fences round a relaxed one took 0.4 us more on the reductions of 8^3 x 16, 6.0 us
+// back to back.  fin(const double* totals) runs on one thread of the last block.
 template <int N, int B, class Fin>
 __device__ __forceinline__ void grid_reduce(double (&v)[N], const RedScratch& rs, const Fin& fin) {
   __shared__ double sm[N * B];
@@ -1155,13 +1158,13 @@ __device__ __forceinline__ void grid_reduce(double (&v)[N], const RedScratch& rs
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int k = 0; k < N; ++k) rs.partials[(size_t)blockIdx.x * N + k] = v[k];
-    __threadfence();
-    unsigned ticket = atomicInc(rs.counter, gridDim.x - 1);
+    unsigned ticket;
+    asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;"
+                 : "=r"(ticket) : "l"(rs.counter), "r"(gridDim.x - 1) : "memory");
     is_last = (ticket == gridDim.x - 1);
   }
   __syncthreads();
   if (!is_last) return;
-  __threadfence();
   double s[N];
   partial_sum<N, B>(rs.partials, gridDim.x, 1, N, s, sm);
   if (threadIdx.x == 0) fin(s);

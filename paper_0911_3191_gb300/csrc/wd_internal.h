@@ -20,7 +20,7 @@ struct SolverCtl {
   double cg_alpha;   // CG step
   double rr;         // |r_hat|^2, the iterated residual (CG: normal residual)
   double rr_prev;    // CG: |r_hat|^2 of the previous iteration
-  double maxr;       // M(r_hat) of Alg. 2: max |r_hat| since the last update
+  double maxr2;      // M(r_hat)^2 of Alg. 2: max |r_hat|^2 since the last update
   double stop2;      // (tol |b|)^2, b the full source
   double delta;      // reliable-update threshold of Alg. 2
   double r2_true;    // |b_hat - M_hat x|^2 at the last reliable update

@@ -1,6 +1,7 @@
 """The dslash on both sides of the line between the two thread layouts: four warps
 per 32 sites up to one block of 128 sites per SM (152 SMs: 19456 sites of a
 parity), one thread per site above; neither lattice fills its last block."""
+import numpy as np
 import pytest
 
 import lattice_inputs as li
@@ -35,4 +36,22 @@ def test_both_sides_of_the_line(dims, prec, temporal, anti, dagger, parity):
     assert rel_err(wd.download(o, prec, parity=parity), d) <= tol
     want = psi * parity_mask(dims, parity) - 0.37 * d
     assert rel_err(wd.download(o2, prec, parity=parity), want) <= tol
+    wd.close()
+
+
+@pytest.mark.parametrize("dims", [(4, 16, 16, 38), (4, 16, 16, 40), (2, 6, 10, 14)])
+@pytest.mark.parametrize("prec", [0, 1, 2])
+def test_site_kernels_on_both_sides_of_the_small_block(dims, prec):
+    """Up to 128 sites per SM (19456 with 152 SMs, the first lattice) the site kernels run
+    in blocks of 128, beyond in blocks of 256; 840 sites fill neither."""
+    import paper_0911_3191_gb300 as m
+    U = li.gauge(dims, 0.4, 1030)
+    b = li.gaussian_spinor(dims, 1031)
+    wd = m.WilsonDirac(dims)
+    wd.load_gauge(U)
+    for solver in (m.BICGSTAB, m.CGNR):
+        x = np.zeros_like(b)
+        info = wd.solve(x, b, 0.115, tol=1e-10, solver=solver, inner_precision=prec)
+        rel = oracle.true_residual(x, b, U, dims, 0.115)
+        assert info.status == 0 and rel <= 1e-10, (solver, info, rel)
     wd.close()
