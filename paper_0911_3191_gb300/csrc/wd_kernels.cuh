@@ -1295,10 +1295,13 @@ void launch_dslash(const Ctx& c, const In& in, const G& gauge, int parity, Dag d
     // Split kernels (a site over four warps) up to one block of 128 sites per
     // SM.  FP64 in fixed point, 152 SMs: 2048 and 4096 sites 16.5 -> 8.4 us,
     // 8192 16.6 -> 10.4, 16384 16.6 -> 14.6, 32768 20.7 either way, 65536 33.1
-    // against 34.8.  Compiled where small lattices spend their time: not for
-    // general FP64 links, 8-number links and FP64 with fused reductions.
-    if constexpr (!std::is_same<G, GaugeF64>::value && !kR8 && (sizeof(R) == 4 || Epi::NRED == 0)) {
-      if ((n + kDslashBlock - 1) / kDslashBlock <= c.num_sms) {
+    // against 34.8.  With fused reductions, whose FP64 arithmetic one warp of the
+    // four does, half as far: <r_tilde, v> at 4096 sites 19.9 -> 11.5 us, 8192
+    // 20.4 -> 13.1, 16384 20.3 against 22.5.  Not compiled for general FP64 links
+    // and 8-number links.
+    if constexpr (!std::is_same<G, GaugeF64>::value && !kR8) {
+      constexpr int kSites = (sizeof(R) == 8 && Epi::NRED > 0) ? kDslashBlock / 2 : kDslashBlock;
+      if (n <= kSites * c.num_sms) {
         launch_pdl(dslash_kernel<decltype(dag)::value, kTfix, kR8, true, R, In, G, Epi>, dim3((n + 31) / 32),
                    dim3(kDslashBlock), 0, s, geo, in, gauge, parity, epi);
         return;

@@ -39,11 +39,13 @@ def test_both_sides_of_the_line(dims, prec, temporal, anti, dagger, parity):
     wd.close()
 
 
-@pytest.mark.parametrize("dims", [(4, 16, 16, 38), (4, 16, 16, 40), (2, 6, 10, 14)])
+@pytest.mark.parametrize("dims", [(4, 16, 16, 38), (4, 16, 16, 40), (2, 6, 10, 14), (8, 8, 8, 38), (8, 8, 8, 40)])
 @pytest.mark.parametrize("prec", [0, 1, 2])
-def test_site_kernels_on_both_sides_of_the_small_block(dims, prec):
+def test_solvers_on_both_sides_of_the_small_shapes(dims, prec):
     """Up to 128 sites per SM (19456 with 152 SMs, the first lattice) the site kernels run
-    in blocks of 128, beyond in blocks of 256; 840 sites fill neither."""
+    in blocks of 128, beyond in blocks of 256; 840 sites fill neither.  The last two
+    lattices lie on the two sides of 64 sites per SM (9728), up to which the FP64
+    dslash with a fused reduction is the one of four warps per 32 sites."""
     import paper_0911_3191_gb300 as m
     U = li.gauge(dims, 0.4, 1030)
     b = li.gaussian_spinor(dims, 1031)
