@@ -1279,18 +1279,22 @@ void launch_dslash(const Ctx& c, const In& in, const G& gauge, int parity, Dag d
     constexpr bool kTfix = decltype(tfix)::value;
     constexpr bool kR8 = decltype(rec8)::value;
     auto* k = dslash_kernel<decltype(dag)::value, kTfix, kR8, false, R, In, G, Epi>;
-    // Blocks per SM at most, measured per kernel class.  FP32: one wave of
-    // resident blocks (64^3 x 128: 15 % faster than 16 per SM).  16 bit in the
-    // temporal gauge: two waves (24^3 x 64, L2-resident: Q16 30.9 -> 28.7 us,
-    // bf16 28.5 -> 26.1, fp16 30.8 -> 29.5; 64^3 x 128: Q16 929 -> 918, fp16 955
-    // -> 928, bf16 844 -> 850), and one with fused reductions, whose partial
-    // sums grow with the blocks (two: the 24^3 x 64 solve 0.1 % slower).  16 bit
-    // with general links: 16 (24^3 x 64 bf16 30.9 -> 28.0 us; 64^3 x 128 Q16
-    // 1045 -> 991, bf16 960-985 either way).  FP64: 16.
+    // Blocks, measured per kernel class (152 SMs, cold; 64^3 x 128 unless said).
+    // Without reductions 16-bit and FP64 storage take a block per 128 sites, no
+    // loop: the hardware hands out blocks in order, so the sites in work stay one
+    // window of the lattice and find their neighbours in L2, where looping blocks
+    // drift apart.  Against 2 waves (temporal gauge) and 16 per SM (general links):
+    // Q16 948 -> 878 and 1021 -> 965 us, bf16 880 -> 835 and 978 -> 875, fp16 977 ->
+    // 901 and 1022 -> 980; 48^3 x 96 bf16 general 307 -> 273; FP64 32^3 x 64 389 ->
+    // 378; nothing on 24^3 x 64, which L2 holds.  FP32: one wave of resident blocks
+    // (48^3 x 96 401 us against 410 without a loop and 491 at 16 per SM; general
+    // links 461, 463, 547).  Fused reductions, whose partial sums grow with the
+    // blocks: one wave in 16 bit (two: the 24^3 x 64 solve 0.1 % slower), 16 per SM
+    // in FP64 and in Q16 with general links.
     constexpr bool k16 = In::kBytesPerSite == 52;
-    constexpr int kWaves = k16 && Epi::NRED == 0 && kTfix && !kR8 ? 2 : 1;
-    constexpr bool kMany = sizeof(R) == 8 || (k16 && !kTfix && (In::kIntCodes || (Epi::NRED == 0 && !kR8)));
-    static const int per_sm = kMany ? 16 : kWaves * resident_blocks(k, kDslashBlock);
+    constexpr bool kMany = sizeof(R) == 8 || (k16 && !kTfix && In::kIntCodes);
+    constexpr bool kNoLoop = Epi::NRED == 0 && (sizeof(R) == 8 || (k16 && !kR8));
+    static const int per_sm = kMany ? 16 : resident_blocks(k, kDslashBlock);
     const int n = geo.h_end - geo.h_begin;
     // Split kernels (a site over four warps) up to one block of 128 sites per
     // SM.  FP64 in fixed point, 152 SMs: 2048 and 4096 sites 16.5 -> 8.4 us,
@@ -1307,7 +1311,7 @@ void launch_dslash(const Ctx& c, const In& in, const G& gauge, int parity, Dag d
         return;
       }
     }
-    const int grid = wave_grid(n, kDslashBlock, c.num_sms, per_sm);
+    const int grid = kNoLoop ? (n + kDslashBlock - 1) / kDslashBlock : wave_grid(n, kDslashBlock, c.num_sms, per_sm);
     launch_pdl(k, dim3(grid), dim3(kDslashBlock), 0, s, geo, in, gauge, parity, epi);
   };
   pick_dagger(dagger, [&](auto dag) {

@@ -254,7 +254,7 @@ BatchLaunch dslash_shape(const Ctx& c, int n, int prec) {
     return bl;
   }
   bl.tr = 0;
-  bl.grid = std::min(nblk, 16 * c.num_sms);
+  bl.grid = prec == WD_F32 ? std::min(nblk, 16 * c.num_sms) : nblk;
   bl.pack = has_pairs(c, prec) && n > 1 && (long)nblk * ((n + 1) / 2) >= 8 * c.num_sms;
   return bl;
 }
