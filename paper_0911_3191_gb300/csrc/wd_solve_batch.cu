@@ -247,6 +247,7 @@ BatchLaunch launch_shape(const Ctx& c, int n) {
 BatchLaunch dslash_shape(const Ctx& c, int n, int prec) {
   const int ntiles = (c.g.Vh + 31) / 32, nblk = (c.g.Vh + kDslashBlock - 1) / kDslashBlock;
   BatchLaunch bl{n, 4, std::min(c.num_sms * 4, ntiles), blas_gx(c, n)};
+  if (prec == WD_F64) bl.grid64 = nblk;  // as the single dslash: no loop, no partial sums
   if (prec == WD_F64 || c.low_recon == 8) return bl;
   if (prec == WD_F32 && n >= 4 && ntiles >= 8 * c.num_sms) {
     bl.tr = 2;
