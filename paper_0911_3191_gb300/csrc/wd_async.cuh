@@ -1,5 +1,6 @@
 // The dslash of one site for 16-bit storage (Sec. 4.6) with its neighbour
-// data staged through shared memory by asynchronous copies (cp.async).
+// data staged through shared memory by asynchronous copies (cp.async), for one
+// spinor field or for N that share the links (N = 2: batches).
 //
 // Each thread owns three stages of shared-memory slots (structure of arrays
 // by thread, so a warp's accesses are conflict-free).  A stage holds one

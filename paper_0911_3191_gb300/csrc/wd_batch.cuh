@@ -6,7 +6,9 @@
 // into shared memory (decoded, third row rebuilt once) and every chunk of TR
 // right-hand sides reuses them, so a launch reads each link from DRAM once
 // however many right-hand sides it serves.  Each right-hand side has its own
-// coefficient (kappa), its own fused epilogue and its own FP64 reductions.
+// coefficient (kappa), its own fused epilogue and its own FP64 reductions.  16-bit
+// storage is mostly faster without the tile, with two right-hand sides per thread
+// (dslash_rhs_pair_kernel).
 //
 // Reductions of a batch are two-stage: the producing kernel writes one FP64
 // partial per (right-hand side, quantity, block); a finalise kernel with one
@@ -467,11 +469,11 @@ __global__ void __launch_bounds__(32 * TP) dslash_mrhs2_kernel(Geom g, In in, G 
 // Per-system dslash over a batch: the single-system site kernel with
 // blockIdx.y naming the system (in mode 1, the y-th entry of the list of
 // systems due for an update; blocks past the list's end return at once).
-// Always used for FP64, where the FP64 pipe, not the link bytes, sets the
+// Always used for FP64, where the arithmetic, not the link bytes, sets the
 // time, so sharing a link tile between systems gains nothing, while a tile
 // whose systems are mostly idle (one reliable update due among several)
 // leaves the SM a few computing warps; used for the inner precision when the
-// launch shape says so (tr = 0: few systems).
+// launch shape says so (tr = 0).
 template <bool DAGGER, bool TFIX, bool R8, typename R, class In, class G, class Epi>
 __global__ void __launch_bounds__(kDslashBlock, (DslashOccupancy<R, In, Epi::NRED, TFIX, R8>::kMinBlocks))
     dslash_rhs_kernel(Geom g, In in, G gauge, int parity, Epi epi, BatchArgs ba) {

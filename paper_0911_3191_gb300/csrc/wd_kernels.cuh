@@ -530,8 +530,8 @@ struct EpiRelupBicg {
 // The FP64 part of the BiCGstab reliable update for an FP32 or 16-bit inner
 // precision: r = b_hat - (x + c acc) in FP64, stored rounded to FP32 (the
 // values EpiRelupBicg rounds before quantising); OpRelupQuant then finishes
-// the update in a bandwidth-bound pass, so the FP64-pipe-bound dslash carries
-// no FP32 epilogue work and no reductions.
+// the update in a bandwidth-bound pass, so the FP64 dslash carries no FP32
+// epilogue work and no reductions.
 struct EpiResidF32 {
   static constexpr int NRED = 0;
   SpinorF32 out;
@@ -606,7 +606,8 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // Resident blocks per SM the register allocation is held to (chosen from
 // ptxas register and spill counts): the FP32 and 16-bit kernels are
 // memory-latency bound and want warps, the fused-reduction epilogues need a
-// few more registers, and the FP64 kernel is bound by the FP64 pipe.
+// few more registers, and the FP64 kernels (fixed point: bound by the integer
+// units; general links: by the FP64 pipe) need 168.
 template <typename R, class In, int NRED, bool TFIX, bool R8>
 struct DslashOccupancy {
   // (the 16-bit temporal-gauge kernels with spin-paired hops spill at 5

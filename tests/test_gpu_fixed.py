@@ -149,3 +149,24 @@ def test_solver_products_of_uneven_sites():
     rel = oracle.true_residual(x, b, U, DIMS, 0.12)
     assert info.status == 0 and rel <= 1e-10, (info, rel)
     wd.close()
+
+
+@pytest.mark.parametrize("prec", [1, 2, 3, 4])
+@pytest.mark.parametrize("angle", [0.0, 1e-12, 3e-10, 1e-5])
+def test_derived_links_with_small_numbers(prec, angle):
+    """The FP32 and 16-bit links are derived from the limbs of the fixed-point ones: zeros,
+    numbers below 2^-28 (one limb) and ordinary ones, of both signs."""
+    from tests.wd_testutil import TOL
+    wdp = _wd()
+    U = np.zeros((int(np.prod(DIMS)), 4, 3, 3), dtype=np.complex128)
+    s = angle * np.where(np.arange(U.shape[0]) % 2, 1.0, -1.0)[:, None]
+    for a, f in ((0, 1.0), (1, -2.0), (2, 1.0)):
+        U[:, :, a, a] = np.exp(1j * f * s)
+    psi = li.gaussian_spinor(DIMS, 1024)
+    wd = wdp.WilsonDirac(DIMS)
+    wd.load_gauge(U)
+    f, o = wd.upload(psi, prec, parity=0), wd.new_field(prec)
+    wd.dslash(o, f, 1, False, prec)
+    want = oracle.dslash(psi * parity_mask(DIMS, 0), U, DIMS, dagger=False, out_parity=1, tbc_anti=False)
+    assert rel_err(wd.download(o, prec, parity=1), want) <= TOL[prec]
+    wd.close()
