@@ -740,7 +740,8 @@ wd_status solve_device(wd_ctx* ctx, void* x_full, const void* b_full, double kap
     info->status = result;
     info->seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     // setup: 3 norms, b_hat, zero x, control init, solver setup (4 kernels,
-    // CG: 2 dslash + 2 zero); per iteration: BiCGstab 7 (CG 5);
+    // CG: 2 dslash + 2 zero); per iteration (hc.loops counts those that ran, one
+    // that failed before its end included): BiCGstab 7 (CG 5);
     // per reliable update: BiCGstab 3 (4 with a lower inner precision: the
     // quantisation pass), CG 5; end: x_o with the odd residual,
     // and the even residual dslash
@@ -749,7 +750,7 @@ wd_status solve_device(wd_ctx* ctx, void* x_full, const void* b_full, double kap
     const long long setup = 3 + (odd_zero ? 0 : 1) + (x0 ? 2 : 1) + 1 + 4 + (start_converged ? 1 : 0);
     const long long per_it = (p.solver == WD_BICGSTAB ? 7 : 5);
     const long long per_up = (p.solver == WD_BICGSTAB) ? (p.inner_precision == WD_F64 ? 3 : 4) : 5;
-    info->kernel_launches = setup + (long long)hc.iter * per_it + (long long)hc.updates * per_up + 2;
+    info->kernel_launches = setup + (long long)hc.loops * per_it + (long long)hc.updates * per_up + 2;
   }
   if (result != WD_OK) {
     char m[160];

@@ -36,7 +36,7 @@ struct SolverCtl {
   int forced;        // the update was forced by apparent convergence or max_iter
   int in_graph;      // 1: running inside the solver graph (set the conditionals)
   int restart;       // 1: defect correction (Alg. 1): every update restarts the Krylov space
-  int loops;         // WHILE-body executions, counted by the iteration's finaliser
+  int loops;         // iterations run (graph: WHILE-body executions), counted by the finaliser that ends one
   int pad;
   unsigned long long h_update;  // graph conditional handles (used when in_graph)
   unsigned long long h_loop;

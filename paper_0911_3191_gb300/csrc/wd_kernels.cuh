@@ -45,11 +45,12 @@ __device__ __forceinline__ void ctl_set_update(SolverCtl* ctl, int v) {
   if (ctl->in_graph) cudaGraphSetConditional((cudaGraphConditionalHandle)ctl->h_update, (unsigned)v);
 }
 
-// The solver graph's WHILE condition, set by the finaliser that ends an
-// iteration and again by the one that ends a reliable update (a kernel of its
-// own at the end of the body was one launch in nine of an iteration).  The
-// iteration's finaliser also bounds the body count on its own, at max_iter + 16
-// executions whatever the others do, so the device loop always terminates.
+// The solver graph's WHILE condition, set on every path through the finaliser
+// that ends an iteration (ctl_end_iteration: a failure of that or an earlier
+// finaliser of the same body runs no reliable update) and again by the one that
+// ends a reliable update.  The iteration's finaliser also bounds the body count
+// on its own, at max_iter + 16 executions whatever the others do, so the device
+// loop always terminates.
 __device__ __forceinline__ void ctl_set_loop(SolverCtl* ctl) {
   if (ctl->in_graph) cudaGraphSetConditional((cudaGraphConditionalHandle)ctl->h_loop, ctl->done ? 0u : 1u);
 }
@@ -113,6 +114,10 @@ struct FinBicgIter {
   SolverCtl* ctl;
   __device__ __forceinline__ FinBicgIter at(int r) const { return FinBicgIter{ctl + r}; }
   __device__ void operator()(const double* t) const {
+    step(t);
+    ctl_end_iteration(ctl);
+  }
+  __device__ __forceinline__ void step(const double* t) const {
     if (ctl->done) { ctl_set_update(ctl, 0); return; }
     const double rr = t[0];
     const double2 rho_new = make_double2(t[1], t[2]);
@@ -185,6 +190,10 @@ struct FinCgIter {
   SolverCtl* ctl;
   __device__ __forceinline__ FinCgIter at(int r) const { return FinCgIter{ctl + r}; }
   __device__ void operator()(const double* t) const {
+    step(t);
+    ctl_end_iteration(ctl);
+  }
+  __device__ __forceinline__ void step(const double* t) const {
     if (ctl->done) { ctl_set_update(ctl, 0); return; }
     const double rr = t[0];
     ctl->iter += 1;
