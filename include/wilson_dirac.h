@@ -100,6 +100,10 @@ size_t wd_field_bytes(const wd_ctx *ctx, wd_prec prec);
  * c = (a x b)^* (App. A.1; exact for SU(3) links); recon = 18 stores all
  * nine entries (FP64 only).  Lower-precision copies (FP32; Q16 codes
  * rint(u*32767); fp16; bf16) are derived from the FP64 copy on first use.
+ * Links of modulus 1.125 at most per real are also kept as 64-bit integers
+ * u 2^60 for the FP64 dslash on the integer units, as many bytes again as the
+ * FP64 copy, unless that is more than a quarter of the free device memory;
+ * without them the FP64 dslash takes about three times as long.
  * Replaces any previous gauge field. */
 wd_status wd_load_gauge(wd_ctx *ctx, const double *U, int is_device, int recon);
 
@@ -328,7 +332,9 @@ wd_status wd_solve_multishift_device(wd_ctx *ctx, int n, void *x, const void *b,
  * slots of batched, lockstep reliable-update BiCGstab solves (Sec. 5 and the
  * batched solver above).  Requests that arrive while others are running are
  * admitted at the next step as slots and memory free up; every device
- * allocation is charged against budget_bytes.  Each gauge field has its own
+ * allocation is charged against budget_bytes, the integer copy of the FP64
+ * links (wd_load_gauge) among a field's solver slots: it is made with them when
+ * it takes at most a quarter of their memory.  Each gauge field has its own
  * CUDA stream, so solves on different volumes overlap on the device.  A
  * request's iterates follow the same kernel sequence alone and in a mix. */
 typedef struct wd_server wd_server;

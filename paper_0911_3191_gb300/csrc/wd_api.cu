@@ -52,10 +52,9 @@ __global__ void mark_done_kernel(SolverCtl* ctl) {
   ctl->done = 1;
 }
 
-// ---- gauge field: host layout -> even-odd structure of arrays (S1), the
-// elements as fixed-point numbers (nbad counts the links with an element the
-// fixed-point form does not take, row c of 12-real storage included) or, with
-// nbad null, as the doubles they are
+// ---- gauge field: host layout -> even-odd structure of arrays (S1); nbad
+// counts the links with an element the fixed-point form does not take, row c of
+// 12-real storage included
 __global__ void gauge_pack_f64_kernel(Geom g, const double* lex, double2* out, int nc, unsigned* nbad) {
   const int n = 2 * g.Vh;
   unsigned bad = 0;
@@ -63,44 +62,38 @@ __global__ void gauge_pack_f64_kernel(Geom g, const double* lex, double2* out, i
     const int parity = i / g.Vh, h = i - parity * g.Vh;
     int x, y, z, t;
     site_coords(g, h, parity, x, y, z, t);
-    const size_t s = (size_t)x + (size_t)g.X * (y + (size_t)g.Y * (z + (size_t)g.Z * t));
+    const size_t s = ((size_t)x + (size_t)g.X * (y + (size_t)g.Y * (z + (size_t)g.Z * t)));
     for (int mu = 0; mu < 4; ++mu) {
       const double2* src = reinterpret_cast<const double2*>(lex + (s * 4 + mu) * 18);
       double2* dst = out + (size_t)(parity * 4 + mu) * nc * g.stride + h;
-      if (!nbad) {
-        for (int c = 0; c < nc; ++c) dst[(size_t)c * g.stride] = src[c];
-        continue;
-      }
-      double2 u[9];
-#pragma unroll
-      for (int c = 0; c < 6; ++c) u[c] = src[c];
-      if (nc == 9) {
-#pragma unroll
-        for (int c = 6; c < 9; ++c) u[c] = src[c];
-      } else {
-        double r[18];
-#pragma unroll
-        for (int c = 0; c < 6; ++c) {
-          r[2 * c] = u[c].x;
-          r[2 * c + 1] = u[c].y;
-        }
-        reconstruct_row3(r);
-#pragma unroll
-        for (int c = 6; c < 9; ++c) u[c] = make_double2(r[2 * c], r[2 * c + 1]);
-      }
-      bool ok = true;
+      double r[18];
 #pragma unroll
       for (int c = 0; c < 9; ++c) {
-        ok = ok && fabs(u[c].x) <= kFixedLinkMax && fabs(u[c].y) <= kFixedLinkMax;  // false for a NaN
-        if (c < nc) {
-          const int2 re = fx_link(u[c].x), im = fx_link(u[c].y);
-          reinterpret_cast<int4*>(dst)[(size_t)c * g.stride] = make_int4(re.x, re.y, im.x, im.y);
-        }
+        if (c >= nc) break;
+        const double2 u = src[c];
+        dst[(size_t)c * g.stride] = u;
+        r[2 * c] = u.x;
+        r[2 * c + 1] = u.y;
       }
+      if (nc == 6) reconstruct_row3(r);
+      bool ok = true;
+#pragma unroll
+      for (int k = 0; k < 18; ++k) ok = ok && fabs(r[k]) <= kFixedLinkMax;  // false for a NaN
       bad += !ok;
     }
   }
   if (bad) atomicAdd(nbad, bad);
+}
+
+// the fixed-point copy of n complex numbers per parity, direction and element
+__global__ void gauge_f64_to_fixed_kernel(Geom g, const double2* in, int nc, int4* out) {
+  const int n = g.Vh;
+  for (int q = blockIdx.y; q < 8 * nc; q += gridDim.y)
+    for (int h = blockIdx.x * blockDim.x + threadIdx.x; h < n; h += gridDim.x * blockDim.x) {
+      const double2 u = in[(size_t)q * g.stride + h];
+      const int2 re = fx_link(u.x), im = fx_link(u.y);
+      out[(size_t)q * g.stride + h] = make_int4(re.x, re.y, im.x, im.y);
+    }
 }
 
 // ---- temporal gauge (Sec. 4.3), FP64 on the host-layout links in place.
@@ -197,13 +190,13 @@ __global__ void temporal_gauge_pack_kernel(Geom g, const double2* G, double2* ou
 }
 
 // FP64 copy (first two rows) -> FP32 / 16-bit copies
-__global__ void gauge_f64_to_f32_kernel(Geom g, const double2* in, int nc, bool fixed, float4* out) {
+__global__ void gauge_f64_to_f32_kernel(Geom g, const double2* in, int nc, float4* out) {
   const int n = 8 * g.Vh;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int pm = i / g.Vh, h = i - pm * g.Vh;
     double r[12];
     for (int c = 0; c < 6; ++c) {
-      double2 d = link_value(in[((size_t)pm * nc + c) * g.stride + h], fixed);
+      double2 d = in[((size_t)pm * nc + c) * g.stride + h];
       r[2 * c] = d.x;
       r[2 * c + 1] = d.y;
     }
@@ -223,17 +216,47 @@ __device__ __forceinline__ uint32_t link16(double u) {
 }
 
 template <Fmt16 F>
-__global__ void gauge_f64_to_16_kernel(Geom g, const double2* in, int nc, bool fixed, uint4* out8, uint2* out4) {
+__global__ void gauge_f64_to_16_kernel(Geom g, const double2* in, int nc, uint4* out8, uint2* out4) {
   const int n = 8 * g.Vh;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int pm = i / g.Vh, h = i - pm * g.Vh;
     uint32_t w[6];
     for (int c = 0; c < 6; ++c) {
-      double2 d = link_value(in[((size_t)pm * nc + c) * g.stride + h], fixed);
+      double2 d = in[((size_t)pm * nc + c) * g.stride + h];
       w[c] = link16<F>(d.x) | (link16<F>(d.y) << 16);
     }
     out8[(size_t)pm * g.stride + h] = make_uint4(w[0], w[1], w[2], w[3]);
     out4[(size_t)pm * g.stride + h] = make_uint2(w[4], w[5]);
+  }
+}
+
+size_t fixed_link_bytes(const Ctx& c) { return (size_t)8 * (c.recon / 2) * c.g.stride * sizeof(int4); }
+
+void drop_fixed_links(Ctx& c) {
+  if (c.gauge_fx) cudaFree(c.gauge_fx);
+  c.gauge_fx = nullptr;
+}
+
+// Without it the dslash works on the doubles: slower, with the same calls taken.
+// A quarter of the free memory at most, so that a lattice that fills the device
+// keeps the room that its solver fields had.
+void make_fixed_links(Ctx& c) {
+  if (c.gauge_fx || !c.fixed_ok) return;
+  const size_t bytes = fixed_link_bytes(c);
+  size_t free_bytes = 0, total = 0;
+  if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess || bytes > free_bytes / 4 ||
+      cudaMalloc(&c.gauge_fx, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    c.gauge_fx = nullptr;
+    return;
+  }
+  const int nc = c.recon / 2;
+  const int gx = (c.g.Vh + 255) / 256 < c.num_sms * 2 ? (c.g.Vh + 255) / 256 : c.num_sms * 2;
+  gauge_f64_to_fixed_kernel<<<dim3(gx, 8 * nc), 256, 0, c.stream>>>(c.g, (const double2*)c.gauge[WD_F64], nc,
+                                                                    (int4*)c.gauge_fx);
+  if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(c.stream) != cudaSuccess) {
+    cudaGetLastError();
+    drop_fixed_links(c);
   }
 }
 
@@ -373,16 +396,16 @@ int grid_for(const Ctx& c, int n, int block) {
 // singularity |a1| = 1 (N = sqrt(|a2|^2 + |a3|^2) below 1e-6); temporal links
 // of the temporal gauge off the last slice are never read.
 template <int P>
-__global__ void gauge_f64_to_8_kernel(Geom g, const double2* in, int nc, bool fixed, void* out, unsigned* nsing) {
+__global__ void gauge_f64_to_8_kernel(Geom g, const double2* in, int nc, void* out, unsigned* nsing) {
   const int n = 8 * g.Vh;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int pm = i / g.Vh, h = i - pm * g.Vh;
     const int parity = pm >> 2, mu = pm & 3;
     double2 r[6];
-    for (int c = 0; c < 6; ++c) r[c] = link_value(in[((size_t)pm * nc + c) * g.stride + h], fixed);
+    for (int c = 0; c < 6; ++c) r[c] = in[((size_t)pm * nc + c) * g.stride + h];
     double2 c1;
     if (nc == 9) {
-      c1 = link_value(in[((size_t)pm * nc + 6) * g.stride + h], fixed);
+      c1 = in[((size_t)pm * nc + 6) * g.stride + h];
     } else {  // c1 = conj(a2 b3 - a3 b2)
       const double re = r[1].x * r[5].x - r[1].y * r[5].y - (r[2].x * r[4].x - r[2].y * r[4].y);
       const double im = r[1].x * r[5].y + r[1].y * r[5].x - (r[2].x * r[4].y + r[2].y * r[4].x);
@@ -417,7 +440,6 @@ wd_status ensure_gauge(wd_ctx* ctx, int prec) {
   const size_t links = (size_t)8 * c.g.stride;
   const int nc = c.recon / 2;
   const double2* src = (const double2*)c.gauge[WD_F64];
-  const bool fx = c.gauge_fixed;
   const int grid = grid_for(c, 8 * c.g.Vh, 256);
   wd_status st;
   if (c.low_recon == 8 && prec != WD_F64) {
@@ -425,10 +447,10 @@ wd_status ensure_gauge(wd_ctx* ctx, int prec) {
     if ((st = dev_alloc(ctx, &c.gauge[prec], bytes)) != WD_OK) return st;
     unsigned* nsing = reinterpret_cast<unsigned*>(c.scalars);
     WD_CK(ctx, cudaMemsetAsync(nsing, 0, sizeof(unsigned), c.stream));
-    if (prec == WD_F32) gauge_f64_to_8_kernel<WD_F32><<<grid, 256, 0, c.stream>>>(c.g, src, nc, fx, c.gauge[prec], nsing);
-    else if (prec == WD_Q16) gauge_f64_to_8_kernel<WD_Q16><<<grid, 256, 0, c.stream>>>(c.g, src, nc, fx, c.gauge[prec], nsing);
-    else if (prec == WD_H16N) gauge_f64_to_8_kernel<WD_H16N><<<grid, 256, 0, c.stream>>>(c.g, src, nc, fx, c.gauge[prec], nsing);
-    else gauge_f64_to_8_kernel<WD_B16N><<<grid, 256, 0, c.stream>>>(c.g, src, nc, fx, c.gauge[prec], nsing);
+    if (prec == WD_F32) gauge_f64_to_8_kernel<WD_F32><<<grid, 256, 0, c.stream>>>(c.g, src, nc, c.gauge[prec], nsing);
+    else if (prec == WD_Q16) gauge_f64_to_8_kernel<WD_Q16><<<grid, 256, 0, c.stream>>>(c.g, src, nc, c.gauge[prec], nsing);
+    else if (prec == WD_H16N) gauge_f64_to_8_kernel<WD_H16N><<<grid, 256, 0, c.stream>>>(c.g, src, nc, c.gauge[prec], nsing);
+    else gauge_f64_to_8_kernel<WD_B16N><<<grid, 256, 0, c.stream>>>(c.g, src, nc, c.gauge[prec], nsing);
     WD_CK_LAUNCH(ctx, "gauge conversion (8 numbers)");
     unsigned h_nsing = 0;
     WD_CK(ctx, cudaMemcpyAsync(&h_nsing, nsing, sizeof(unsigned), cudaMemcpyDeviceToHost, c.stream));
@@ -443,15 +465,15 @@ wd_status ensure_gauge(wd_ctx* ctx, int prec) {
   }
   if (prec == WD_F32) {
     if ((st = dev_alloc(ctx, &c.gauge[prec], links * 3 * sizeof(float4))) != WD_OK) return st;
-    gauge_f64_to_f32_kernel<<<grid, 256, 0, c.stream>>>(c.g, src, nc, fx, (float4*)c.gauge[prec]);
+    gauge_f64_to_f32_kernel<<<grid, 256, 0, c.stream>>>(c.g, src, nc, (float4*)c.gauge[prec]);
   } else {
     if ((st = dev_alloc(ctx, &c.gauge[prec], links * sizeof(uint4))) != WD_OK) return st;
     if ((st = dev_alloc(ctx, &c.gauge4[prec], links * sizeof(uint2))) != WD_OK) return st;
     uint4* o8 = (uint4*)c.gauge[prec];
     uint2* o4 = (uint2*)c.gauge4[prec];
-    if (prec == WD_Q16) gauge_f64_to_16_kernel<Fmt16::Q16><<<grid, 256, 0, c.stream>>>(c.g, src, nc, fx, o8, o4);
-    else if (prec == WD_H16N) gauge_f64_to_16_kernel<Fmt16::H16><<<grid, 256, 0, c.stream>>>(c.g, src, nc, fx, o8, o4);
-    else gauge_f64_to_16_kernel<Fmt16::B16><<<grid, 256, 0, c.stream>>>(c.g, src, nc, fx, o8, o4);
+    if (prec == WD_Q16) gauge_f64_to_16_kernel<Fmt16::Q16><<<grid, 256, 0, c.stream>>>(c.g, src, nc, o8, o4);
+    else if (prec == WD_H16N) gauge_f64_to_16_kernel<Fmt16::H16><<<grid, 256, 0, c.stream>>>(c.g, src, nc, o8, o4);
+    else gauge_f64_to_16_kernel<Fmt16::B16><<<grid, 256, 0, c.stream>>>(c.g, src, nc, o8, o4);
   }
   WD_CK_LAUNCH(ctx, "gauge conversion");
   return WD_OK;
@@ -904,6 +926,7 @@ wd_status wd_destroy(wd_ctx* ctx) {
   dev_free(c.sb_full[0]);
   dev_free(c.sb_full[1]);
   dev_free((void*&)c.gfix);
+  drop_fixed_links(c);
   batch_release(c);
   if (c.host_pinned) cudaFreeHost(c.host_pinned);
   delete ctx;
@@ -938,8 +961,9 @@ wd_status wd_load_gauge_opt(wd_ctx* ctx, const double* U, int is_device, int rec
     dev_free(c.gauge[p]);
     dev_free(c.gauge4[p]);
   }
+  drop_fixed_links(c);
   dev_free((void*&)c.gfix);
-  c.gauge_loaded = false;
+  c.gauge_loaded = c.fixed_ok = false;
   c.g.tfix = 0;
   const size_t lex_bytes = (size_t)2 * c.g.Vh * 72 * sizeof(double);
   const double* src = U;
@@ -975,23 +999,16 @@ wd_status wd_load_gauge_opt(wd_ctx* ctx, const double* U, int is_device, int rec
   const int nc = recon / 2;
   if (st == WD_OK) st = dev_alloc(ctx, &c.gauge[WD_F64], (size_t)8 * nc * c.g.stride * sizeof(double2));
   if (st == WD_OK) {
-    // fixed-point links; a field with an element above kFixedLinkMax (not
-    // SU(3)) or not finite is packed again as doubles
     unsigned* nbad = reinterpret_cast<unsigned*>(c.scalars);
     unsigned h_nbad = 0;
-    const int grid = grid_for(c, 2 * c.g.Vh, 256);
     cudaError_t e = cudaMemsetAsync(nbad, 0, sizeof(unsigned), c.stream);
-    gauge_pack_f64_kernel<<<grid, 256, 0, c.stream>>>(c.g, src, (double2*)c.gauge[WD_F64], nc, nbad);
+    gauge_pack_f64_kernel<<<grid_for(c, 2 * c.g.Vh, 256), 256, 0, c.stream>>>(c.g, src, (double2*)c.gauge[WD_F64],
+                                                                               nc, nbad);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(&h_nbad, nbad, sizeof(unsigned), cudaMemcpyDeviceToHost, c.stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c.stream);
-    c.gauge_fixed = h_nbad == 0;
-    if (e == cudaSuccess && h_nbad) {
-      gauge_pack_f64_kernel<<<grid, 256, 0, c.stream>>>(c.g, src, (double2*)c.gauge[WD_F64], nc, nullptr);
-      e = cudaGetLastError();
-      if (e == cudaSuccess) e = cudaStreamSynchronize(c.stream);
-    }
+    c.fixed_ok = h_nbad == 0;
     if (e != cudaSuccess) st = cuda_err(ctx, e, "gauge pack");
   }
   if (staging) cudaFree(staging);
@@ -999,6 +1016,7 @@ wd_status wd_load_gauge_opt(wd_ctx* ctx, const double* U, int is_device, int rec
   if (st == WD_OK) {
     c.gauge_loaded = true;
     c.g.tfix = temporal_gauge;
+    if (!c.fixed_lazy) make_fixed_links(c);
   } else {
     dev_free((void*&)c.gfix);
   }

@@ -663,8 +663,8 @@ template <typename R, class In, class G, class Dag, class Epi>
 void launch_dslash_mrhs(const Geom& g, const BatchLaunch& bl, const In& in, const G& gauge, int parity, Dag dagger,
                         const Epi& epi, const BatchArgs& ba, cudaStream_t s) {
   if constexpr (std::is_same<G, GaugeF64>::value) {
-    if (gauge.fixed) {
-      launch_dslash_mrhs<R>(g, bl, in, GaugeX64{(const int4*)gauge.p, gauge.stride, gauge.recon}, parity, dagger, epi,
+    if (gauge.fx) {
+      launch_dslash_mrhs<R>(g, bl, in, GaugeX64{gauge.fx, gauge.stride, gauge.recon, gauge.p}, parity, dagger, epi,
                             ba, s);
       return;
     }

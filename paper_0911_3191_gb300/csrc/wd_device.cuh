@@ -526,22 +526,13 @@ __device__ __forceinline__ void su3_from8(const float (&p)[8], float (&u)[18]) {
 }
 
 // --------------------------------------------------------- fixed-point links
-// The FP64 links are kept as 64-bit integers u 2^60, each as two signed 32-bit
-// limbs (high, low), for the integer-pipe dslash of wd_fixed.cuh, when every
-// element of the field satisfies |u| <= kFixedLinkMax (SU(3) links do); other
-// fields keep the doubles.  Both take the same 16 bytes per complex number.
+// Beside the FP64 links a context keeps a copy as 64-bit integers u 2^60, each as
+// two signed 32-bit limbs (high, low), for the integer-pipe dslash of wd_fixed.cuh,
+// when every element of the field satisfies |u| <= kFixedLinkMax (SU(3) links do).
+// Both take the same 16 bytes per complex number.  Only that dslash reads it: the
+// links of the other precisions, the slab faces and the sites that it leaves to FP64
+// come from the doubles, since an element below 2^-8 is not exact in the integers.
 constexpr double kFixedLinkMax = 1.125;
-// v 2^e as a double, rounded to nearest, on the integer pipe
-__device__ __forceinline__ double fx_to_double(long long v, int e) {
-  const long long m = v >> 63;
-  unsigned long long a = (unsigned long long)((v ^ m) - m);
-  const int n = __clzll((long long)a);
-  a <<= (n & 63);
-  const unsigned long long f = (a >> 11) + ((a >> 10) & 1ull);
-  unsigned long long bits = ((unsigned long long)(unsigned)(1023 + 62 - n + e) << 52) + f;
-  if (v == 0) bits = 0;
-  return __longlong_as_double((long long)(bits | ((unsigned long long)m & 0x8000000000000000ull)));
-}
 
 // u 2^60, rounded to nearest (|u| <= kFixedLinkMax), as (high limb, low limb)
 __device__ __forceinline__ int2 fx_link(double u) {
@@ -552,14 +543,6 @@ __device__ __forceinline__ int2 fx_link(double u) {
   const long long v = w < 0 ? -(long long)a : (long long)a;
   return make_int2((int)(v >> 32) + (int)((unsigned)v >> 31), (int)v);
 }
-__device__ __forceinline__ double fx_link_value(int h, int l) { return fx_to_double(((long long)h << 32) + l, -60); }
-
-// one complex number of the FP64 links as doubles, from either form
-__device__ __forceinline__ double2 link_value(double2 d, bool fixed) {
-  if (!fixed) return d;
-  const int4 w = *reinterpret_cast<const int4*>(&d);
-  return make_double2(fx_link_value(w.x, w.y), fx_link_value(w.z, w.w));
-}
 
 struct GaugeF64 {
   using real = double;
@@ -567,8 +550,8 @@ struct GaugeF64 {
   static constexpr double kScale = 1.0;
   const double2* p;
   int stride;
-  int recon;   // 12 or 18
-  bool fixed;  // the words are fixed-point links
+  int recon;       // 12 or 18
+  const int4* fx;  // their fixed-point copy, or null
   template <bool R8, typename R>
   __device__ __forceinline__ void load_scaled(int parity, int mu, int h, double (&u)[18], R& w) const {
     load_scaled_slot<R8>(parity * 4 + mu, h, u, w);
@@ -588,14 +571,14 @@ struct GaugeF64 {
     const double2* b = p + (size_t)slot * nc * stride + h;
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
-      const double2 d = link_value(ld_link(b + (size_t)c * stride), fixed);
+      const double2 d = ld_link(b + (size_t)c * stride);
       u[2 * c] = d.x;
       u[2 * c + 1] = d.y;
     }
     if (recon == 18) {
 #pragma unroll
       for (int c = 6; c < 9; ++c) {
-        const double2 d = link_value(ld_link(b + (size_t)c * stride), fixed);
+        const double2 d = ld_link(b + (size_t)c * stride);
         u[2 * c] = d.x;
         u[2 * c + 1] = d.y;
       }

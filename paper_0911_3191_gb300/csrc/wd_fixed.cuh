@@ -81,14 +81,15 @@ __device__ __forceinline__ double fx_sum_value(long long v, int e) {
 }
 
 // The FP64 links in this form: the words of GaugeF64, each double replaced by
-// its two limbs (h first).
+// its two limbs (h first), and the doubles themselves for the sites left to FP64.
 struct GaugeX64 {
   using real = double;
   static constexpr bool kScaled = false;
   const int4* p;
   int stride;
   int recon;
-  __device__ __forceinline__ GaugeF64 f64() const { return GaugeF64{(const double2*)p, stride, recon, true}; }
+  const double2* d;
+  __device__ __forceinline__ GaugeF64 f64() const { return GaugeF64{d, stride, recon, nullptr}; }
 };
 
 // Staging of one hop per thread, as in wd_async.cuh: the neighbour's spinor and

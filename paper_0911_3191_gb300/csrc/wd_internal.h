@@ -133,7 +133,9 @@ struct Ctx {
   void* gauge[5];       // by wd_prec: F64 double2; F32 float4; 16-bit: uint4 part
   void* gauge4[5];      // 16-bit: uint2 part
   bool gauge_loaded;
-  bool gauge_fixed;     // the FP64 copy holds fixed-point links (wd_fixed.cuh)
+  bool fixed_ok;        // the fixed-point form of wd_fixed.cuh takes the FP64 links
+  bool fixed_lazy;      // its copy is made on request (make_fixed_links), not at loading
+  void* gauge_fx;       // the fixed-point copy, or nullptr
   // temporal gauge (wd_load_gauge_opt): G(x) as [parity][9][stride] double2,
   // or nullptr; c.g.tfix is set with it
   double2* gfix;
@@ -171,6 +173,12 @@ struct Ctx {
   std::string last_error;
 };
 
+// The fixed-point copy of the FP64 links (wd_api.cu): made when the form takes them
+// (fixed_ok) and the copy is at most a quarter of the free device memory.  Solver
+// graphs captured with it are not to be launched after a drop.
+size_t fixed_link_bytes(const Ctx& c);
+void make_fixed_links(Ctx& c);
+void drop_fixed_links(Ctx& c);
 void batch_release(Ctx& c);  // frees the batched-solve workspace (wd_solve_batch.cu)
 
 // helpers

@@ -1129,13 +1129,13 @@ struct Tr<WD_F64> {
   using R = double;
   static size_t bytes(int stride) { return align256(192 * (size_t)stride); }
   static S view(const void* p, const Geom& g, size_t rs = 0) { return S{(double2*)p, g.stride, rs}; }
-  static G gauge(const Ctx& c) { return G{(const double2*)c.gauge[WD_F64], c.g.stride, c.recon, c.gauge_fixed}; }
+  static G gauge(const Ctx& c) { return G{(const double2*)c.gauge[WD_F64], c.g.stride, c.recon, (const int4*)c.gauge_fx}; }
   // T-slab faces (wd_slab.cuh)
   using Fc = FaceF64;
   static size_t face_bytes(int fs) { return align256(96 * (size_t)fs); }
   static Fc face(const void* p, int fs) { return Fc{(const double2*)p, fs}; }
   static size_t link_face_bytes(const Ctx& c, int fs) { return align256((size_t)2 * (c.recon / 2) * 16 * fs); }
-  static LinkFace<G> link_face(const Ctx& c, const void* p, int fs) { return {G{(const double2*)p, fs, c.recon, false}}; }
+  static LinkFace<G> link_face(const Ctx& c, const void* p, int fs) { return {G{(const double2*)p, fs, c.recon, nullptr}}; }
   static void pack_faces(const Ctx& c, void* lo, void* hi, const void* in, int fs, int dagger, int grid,
                          cudaStream_t s) {
     pack_faces_f64_kernel<<<grid, 256, 0, s>>>(c.g, (const double2*)in, c.g.stride, (double2*)lo, (double2*)hi, fs,
@@ -1143,7 +1143,7 @@ struct Tr<WD_F64> {
   }
   static void pack_link_face(const Ctx& c, void* out, int fs, int grid, cudaStream_t s) {
     pack_link_face_kernel<double2><<<grid, 256, 0, s>>>(c.g, (const double2*)c.gauge[WD_F64], c.recon / 2,
-                                                        c.g.stride, (double2*)out, fs, c.gauge_fixed);
+                                                        c.g.stride, (double2*)out, fs);
   }
 };
 template <>
@@ -1278,8 +1278,8 @@ void launch_dslash(const Ctx& c, const In& in, const G& gauge, int parity, Dag d
   // sub: the context's geometry with a narrower output-site range
   const Geom& geo = sub ? *sub : c.g;
   if constexpr (std::is_same<G, GaugeF64>::value) {
-    if (gauge.fixed) {
-      launch_dslash<R>(c, in, GaugeX64{(const int4*)gauge.p, gauge.stride, gauge.recon}, parity, dagger, epi, s, sub);
+    if (gauge.fx) {
+      launch_dslash<R>(c, in, GaugeX64{gauge.fx, gauge.stride, gauge.recon, gauge.p}, parity, dagger, epi, s, sub);
       return;
     }
   }

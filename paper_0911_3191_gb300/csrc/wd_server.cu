@@ -256,6 +256,7 @@ void release_workspace(Pool& pl, size_t& used) {
   if (pl.ws) cudaFree(pl.ws);
   if (pl.small) cudaFree(pl.small);
   if (pl.hctl) cudaFreeHost(pl.hctl);
+  if (pl.ctx) drop_fixed_links(pl.ctx->c);
   pl.ws = pl.small = nullptr;
   pl.hctl = nullptr;
   used -= pl.ws_bytes;
@@ -265,8 +266,8 @@ void release_workspace(Pool& pl, size_t& used) {
 }
 
 // Workspace for `cap` slots: the batch views of wd_batch.cuh plus one FP64
-// full source field per slot.
-wd_status alloc_workspace(wd_server* sv, Pool& pl, int cap) {
+// full source field per slot, and (fixed) the fixed-point links.
+wd_status alloc_workspace(wd_server* sv, Pool& pl, int cap, bool fixed) {
   Ctx& c = pl.ctx->c;
   const int prec = sv->p.inner_precision;
   const size_t f64 = fbytes(c, WD_F64), fin = fbytes(c, prec);
@@ -283,7 +284,8 @@ wd_status alloc_workspace(wd_server* sv, Pool& pl, int cap) {
   // land after the slots' control blocks are initialised
   WS_CK(sv, cudaMemsetAsync(pl.small, 0, sm, c.stream));
   WS_CK(sv, cudaMallocHost((void**)&pl.hctl, (size_t)cap * sizeof(SolverCtl)));
-  pl.ws_bytes = ws + sm;
+  if (fixed) make_fixed_links(c);
+  pl.ws_bytes = ws + sm + (c.gauge_fx ? fixed_link_bytes(c) : 0);
   sv->used += pl.ws_bytes;
   pl.capacity = cap;
   pl.slot_req.assign(cap, -1);
@@ -558,13 +560,17 @@ wd_status pool_progress(wd_server* s, Pool& pl, int& waiting_for_memory, bool& d
     const size_t left = s->p.budget_bytes ? (s->p.budget_bytes > s->used ? s->p.budget_bytes - s->used : 0)
                                           : (size_t)-1;
     const size_t share = s->p.budget_bytes ? left / (size_t)std::max(1, waiting_for_memory) : left;
+    // the fixed-point links, where they take a quarter of it at most: an FP64 dslash
+    // in a third of the time is worth more than the slots there would be for them
+    const size_t fx = c.fixed_ok && fixed_link_bytes(c) <= share / 4 ? fixed_link_bytes(c) : 0;
     int cap = s->p.max_slots;
-    while (cap > 0 && s->p.budget_bytes && slot_bytes(c, prec) * cap + small_bytes(c, cap, s->p.rhs_tile) > share)
+    while (cap > 0 && s->p.budget_bytes &&
+           slot_bytes(c, prec) * cap + small_bytes(c, cap, s->p.rhs_tile) + fx > share)
       --cap;
     if (cap < 1 && s->p.budget_bytes && slot_bytes(c, prec) + small_bytes(c, 1, s->p.rhs_tile) <= left) cap = 1;
     if (cap >= 1) {
       --waiting_for_memory;
-      wd_status st = alloc_workspace(s, pl, cap);
+      wd_status st = alloc_workspace(s, pl, cap, fx > 0);
       if (st != WD_OK) return st;
       did_work = true;
     }
@@ -724,6 +730,7 @@ wd_status wd_server_add_gauge(wd_server* s, const int dims[4], int t_antiperiodi
     cudaStreamDestroy(st);
     return serr(s, WD_ERR_BUDGET, "gauge field does not fit the memory budget");
   }
+  c.fixed_lazy = true;  // its fixed-point links come and go with the slots' memory
   r = wd_load_gauge_opt(pl.ctx, U, 0, recon, s->p.gauge_flags);
   if (r == WD_OK) r = wd_internal_ensure_gauge(pl.ctx, ip);
   if (r != WD_OK) {

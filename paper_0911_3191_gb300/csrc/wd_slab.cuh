@@ -22,8 +22,6 @@
 // exactly the values the sender's field holds.
 #pragma once
 
-#include <type_traits>
-
 #include "wd_device.cuh"
 
 namespace wd {
@@ -247,11 +245,10 @@ static __global__ void pack_faces_16_kernel(Geom g, const uint4* in, const float
 }
 
 // Link face: U_4 of the last slice, both parities, in the gauge copy's own
-// words (FP64 links as doubles: a rank's neighbour may keep the other form).  `words` 16-byte (or 8-byte) words per link in the gauge layout
+// words.  `words` 16-byte (or 8-byte) words per link in the gauge layout
 // [parity * 4 + mu][words][stride] are copied to [parity][words][fs].
 template <class W>
-__global__ void pack_link_face_kernel(Geom g, const W* gauge, int words, int stride, W* out, int fs,
-                                      bool fixed = false) {
+__global__ void pack_link_face_kernel(Geom g, const W* gauge, int words, int stride, W* out, int fs) {
   const int ts = g.XhYZ;
   const int n = 2 * ts * words;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -259,9 +256,7 @@ __global__ void pack_link_face_kernel(Geom g, const W* gauge, int words, int str
     const int rest = i / ts;
     const int w = rest % words, q = rest / words;
     const int h = hf + ts * (g.T - 1);
-    W v = gauge[((size_t)(q * 4 + 3) * words + w) * stride + h];
-    if constexpr (std::is_same<W, double2>::value) v = link_value(v, fixed);
-    out[((size_t)q * words + w) * fs + hf] = v;
+    out[((size_t)q * words + w) * fs + hf] = gauge[((size_t)(q * 4 + 3) * words + w) * stride + h];
   }
 }
 
