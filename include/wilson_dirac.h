@@ -104,6 +104,10 @@ size_t wd_field_bytes(const wd_ctx *ctx, wd_prec prec);
  * u 2^60 for the FP64 dslash on the integer units, as many bytes again as the
  * FP64 copy, unless that is more than a quarter of the free device memory;
  * without them the FP64 dslash takes about three times as long.
+ * Either way every complex component of an FP64 dslash is right to 2^-44 of
+ * the sum of the |u| |psi| that feed it (2^-49 as a rule, and 2^-53 of the
+ * largest neighbour component over a whole field); with recon = 12 the
+ * elements of the rebuilt row, by either route, to a few 2^-53 of 1.
  * Replaces any previous gauge field. */
 wd_status wd_load_gauge(wd_ctx *ctx, const double *U, int is_device, int recon);
 

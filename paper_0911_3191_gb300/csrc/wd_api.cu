@@ -53,8 +53,8 @@ __global__ void mark_done_kernel(SolverCtl* ctl) {
 }
 
 // ---- gauge field: host layout -> even-odd structure of arrays (S1); nbad
-// counts the links with an element the fixed-point form does not take, row c of
-// 12-real storage included
+// counts the links that the fixed-point form does not take, row c of 12-real
+// storage included
 __global__ void gauge_pack_f64_kernel(Geom g, const double* lex, double2* out, int nc, unsigned* nbad) {
   const int n = 2 * g.Vh;
   unsigned bad = 0;
@@ -79,6 +79,16 @@ __global__ void gauge_pack_f64_kernel(Geom g, const double* lex, double2* out, i
       bool ok = true;
 #pragma unroll
       for (int k = 0; k < 18; ++k) ok = ok && fabs(r[k]) <= kFixedLinkMax;  // false for a NaN
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {  // a unit vector's sum is 1 at least
+        double row = 0, col = 0;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          row += fabs(r[6 * c + 2 * j]) + fabs(r[6 * c + 2 * j + 1]);
+          col += fabs(r[6 * j + 2 * c]) + fabs(r[6 * j + 2 * c + 1]);
+        }
+        ok = ok && row >= kFixedLinkMin && col >= kFixedLinkMin;
+      }
       bad += !ok;
     }
   }

@@ -528,11 +528,12 @@ __device__ __forceinline__ void su3_from8(const float (&p)[8], float (&u)[18]) {
 // --------------------------------------------------------- fixed-point links
 // Beside the FP64 links a context keeps a copy as 64-bit integers u 2^60, each as
 // two signed 32-bit limbs (high, low), for the integer-pipe dslash of wd_fixed.cuh,
-// when every element of the field satisfies |u| <= kFixedLinkMax (SU(3) links do).
+// when every element of the field satisfies |u| <= kFixedLinkMax and the parts of no
+// row or column add up to less than kFixedLinkMin (SU(3) links do both).
 // Both take the same 16 bytes per complex number.  Only that dslash reads it: the
 // links of the other precisions, the slab faces and the sites that it leaves to FP64
 // come from the doubles, since an element below 2^-8 is not exact in the integers.
-constexpr double kFixedLinkMax = 1.125;
+constexpr double kFixedLinkMax = 1.125, kFixedLinkMin = 0.99;
 
 // u 2^60, rounded to nearest (|u| <= kFixedLinkMax), as (high limb, low limb)
 __device__ __forceinline__ int2 fx_link(double u) {

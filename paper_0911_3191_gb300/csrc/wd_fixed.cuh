@@ -3,13 +3,12 @@
 // An SM quarter of GB300 takes one FP64 warp instruction every 67 cycles
 // (measured), but a 32 x 32 + 64-bit integer multiply-add every 4.2 and an
 // integer add, logic or shift instruction every 2.4.  The FP64 stencil takes 614
-// FP64 instructions a site and is bound by that pipe alone.  Here every number of
-// a hop is a 64-bit integer, a product of two takes three integer multiply-adds,
-// and nothing is rounded more coarsely than in FP64.  24^3 x 64, temporal gauge,
-// 18 reals: 471 -> 145 us a dslash (its bytes take 81 us); 12-real general links
-// of 20 x 14 x 22 x 38, M_hat: 459 -> 129 us; 8^3 x 16: 27 -> 14 us.  What bounds
-// it now is the issue of 6100 integer instructions per 32 sites: the multiplier
-// is 59 % busy and the other integer pipe 45 %, which add up rather than overlap.
+// FP64 instructions a site and is bound by that pipe alone (24^3 x 64, temporal
+// gauge, 18 reals: 471 us).  Here every number of a hop is a 64-bit integer, and a
+// product of two takes three integer multiply-adds: 148 us (its bytes take 81);
+// M_hat with 12-real general links of 20 x 14 x 22 x 38 130 us; 8^3 x 16, four
+// warps per 32 sites, 5.9 us.  No pipe is full: 12 warps per SM (168 registers)
+// leave the latencies of 6200 dependent integer instructions per 32 sites in sight.
 //
 //  * A link element u, |u| <= 1, is the integer u 2^60 (converted once, when
 //    the links are loaded).  A double of at least 2^-8 is exact in it, a
@@ -21,9 +20,23 @@
 //    [-2^31, 2^31).  Of a product's limbs ah bh, (ah bl + al bh) 2^-32 and
 //    al bl 2^-64, the last is left out: at most a quarter of the unit 2^(E-1078)
 //    in which the sums are kept.
-//  * The 24 sums are 64-bit integers of that unit, 2^-55 of the largest
-//    neighbour component, where FP64 rounds every partial sum at 2^-53 of
-//    itself.  They are rounded once, to the double they become.
+//  * The 24 sums are 64-bit integers of that unit, rounded once, to the double they
+//    become.
+//
+// Accuracy.  B = 2^(E-1023) is one to four times the largest neighbour component.
+// The sums are off by 23 units of 2^-55 B at most (a hop: 1.5 dropped limbs, 0.5 the
+// middle sums' rounding, 0.6 the cut numbers; one the shifts to a larger E) and by
+// one unit as a rule: over Gaussian fields 0.8e-16 of the largest component against
+// 1.5e-16 for FP64 arithmetic.  FP64 rounds each component relative to what feeds
+// it, though, sum |u| |psi|, which may be far less than B.  So each spin collects the
+// smallest colour of every row that feeds it (fixed_weight), and a site with a spin
+// that gets less than 2^-6 B is computed in FP64 (dslash_site).  What is left is
+// right to 2^-44 of sum |u| |psi| in every complex component, and as a rule to
+// 2^-49, the bound that FP64's 15 roundings have.  No site of Gaussian fields goes
+// that way, 5e-4 of a point source's solution at kappa 0.12, and the fronts of its
+// first iterates.  The weights take 2 % of the dslash (144.6 -> 148.0 us at
+// 24^3 x 64), the FP64 sites 3 % of twelve point sources' batch on 16^3 x 32.
+// (A third row rebuilt from 12 reals is right to a few 2^-53 of 1, here and in FP64.)
 //
 // E is known only when all neighbours are, so it is a running maximum: a hop
 // that raises it shifts the sums down.  Starting one above the first hop's
@@ -32,7 +45,7 @@
 // most 6 x 1.125 x 2^56, and a middle sum stays below 12 x 1.125 x 2^59.
 //
 // Sites whose neighbours hold an infinity, a NaN, or only numbers outside
-// 2^-830 .. 2^870 are computed by dslash_site in FP64 as before.
+// 2^-830 .. 2^870 are computed by dslash_site in FP64 as well.
 #pragma once
 
 #include "wd_async.cuh"
@@ -41,6 +54,7 @@
 namespace wd {
 
 constexpr int kFixedMinExp = 192, kFixedMaxExp = 1892;  // biased exponents E of the fixed-point path
+constexpr int kFixedWeak = 1 << 21;  // 2^-6 of the common exponent, in the unit of the high words (fixed_weight)
 
 struct Fx {
   int h, l;  // h * 2^32 + l
@@ -66,10 +80,15 @@ __device__ __forceinline__ unsigned long long fx_shr(unsigned long long v, int s
   asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));
   return r;
 }
-__device__ __forceinline__ long long fx_sar(long long v, int s) {
-  long long r;
-  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));
+__device__ __forceinline__ int fx_shr32(int v, int s) {  // v >= 0; 0 for any count of 32 and more
+  int r;
+  asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(s));
   return r;
+}
+// v 2^-s rounded to nearest, |v| < 2^62
+__device__ __forceinline__ long long fx_round_sar(long long v, int s) {
+  s = min(s, 62);
+  return (v + ((1ll << s) >> 1)) >> s;
 }
 
 // v 2^e by the conversion of the FP64 pipe (otherwise idle here) and an
@@ -282,14 +301,18 @@ __device__ __forceinline__ void fixed_issue_link(FixedSlots& sm, const GaugeX64&
 // reconstruct() of row s: the upper row s of a hop, and the lower row that the
 // projector makes of it.  CONJ: the row is that of the conjugate (backward hops,
 // see dslash_site_fixed)
+// weak[s] collects the weight (fixed_weight) of the rows that feed output spin s.
 template <int MU, int S_, bool CONJ, int ROW>
-__device__ __forceinline__ void fixed_add(const long long (&gr)[3], const long long (&gi)[3], long long (&a)[24]) {
+__device__ __forceinline__ void fixed_add(const long long (&gr)[3], const long long (&gi)[3], int weight,
+                                          long long (&a)[24], int (&weak)[4]) {
   constexpr int S = (MU == 1) ? -S_ : S_;
   constexpr int up = (MU == 3 && S_ < 0) ? 12 + 6 * ROW : 6 * ROW;
   constexpr int lo = (MU == 2) ? 12 + 6 * ROW : 18 - 6 * ROW;
   // lower row = t g (y) or t i g (x, z): x: -S for both rows, y: -S, S, z: -S, S
   constexpr int t = (MU == 0 || ROW == 0) ? -S : S;
   constexpr int ci = CONJ ? -1 : 1;
+  weak[up / 6] += weight;
+  if constexpr (MU != 3) weak[lo / 6] += weight;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     a[up + 2 * c] += gr[c];
@@ -302,6 +325,20 @@ __device__ __forceinline__ void fixed_add(const long long (&gr)[3], const long l
       a[lo + 2 * c + 1] += t * gr[c];
     }
   }
+}
+
+// The smallest colour of a row of h, by its larger part, in the unit of the high
+// words: whatever the row of the link, no less than that (times sum |u| >= 1)
+// goes into each colour that the row feeds.
+__device__ __forceinline__ int fixed_weight(const long long (&hr)[3], const long long (&hi)[3]) {
+  int w[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) w[c] = max(abs((int)(hr[c] >> 32)), abs((int)(hi[c] >> 32)));
+  return __vimin3_s32(w[0], w[1], w[2]);
+}
+// An output spin that so little feeds that the unit of the sums may show in it
+__device__ __forceinline__ bool fixed_is_weak(const int (&weak)[4]) {
+  return min(min(weak[0], weak[1]), min(weak[2], weak[3])) < kFixedWeak;
 }
 
 // A site whose neighbours are zero (false: its sums are right), or hold numbers
@@ -381,12 +418,14 @@ __device__ __forceinline__ void fixed_su3(const FixedSlots& sm, int step_i, int 
 }
 
 // the sums move to the exponent of a hop that needs a larger one
-__device__ __forceinline__ void fixed_raise(float m, int& E, int& top, long long (&acc)[24]) {
+__device__ __forceinline__ void fixed_raise(float m, int& E, int& top, long long (&acc)[24], int (&weak)[4]) {
   const int e = fx_exponent(m);
   top = max(top, e);
   if (e > E) {
 #pragma unroll
-    for (int q = 0; q < 24; ++q) acc[q] = fx_sar(acc[q], e - E);
+    for (int q = 0; q < 24; ++q) acc[q] = fx_round_sar(acc[q], e - E);
+#pragma unroll
+    for (int s = 0; s < 4; ++s) weak[s] = fx_shr32(weak[s], e - E);
     E = e;
   }
 }
@@ -403,11 +442,11 @@ __device__ __forceinline__ void fixed_raise(float m, int& E, int& top, long long
 // they are converted, and the result's as they are added.
 //
 // The hops k0 .. k1 - 1 of a site (0, 8: all), in the unit of E; top: the largest
-// exponent met.
+// exponent met; weak: what feeds each output spin.
 template <bool DAGGER, bool TFIX>
 __device__ __forceinline__ void fixed_hops(const Geom& g, const SpinorF64& in, const GaugeX64& gauge, FixedSlots& sm,
                                            int h, int parity, int k0, int k1, int& E, int& top,
-                                           long long (&acc)[24]) {
+                                           long long (&acc)[24], int (&weak)[4]) {
   constexpr int SF = DAGGER ? +1 : -1;  // the projector sign of the forward hops
   const int tid = threadIdx.x;
   int x, y, z, t;
@@ -415,6 +454,8 @@ __device__ __forceinline__ void fixed_hops(const Geom& g, const SpinorF64& in, c
   const bool last = (t == g.T - 1), first = (t == 0);
 #pragma unroll
   for (int k = 0; k < 24; ++k) acc[k] = 0;
+#pragma unroll
+  for (int s = 0; s < 4; ++s) weak[s] = 0;
   E = kFixedMinExp;
   top = 0;
   const int n = fixed_neighbour(g, h, x, y, z, t, k0);
@@ -435,7 +476,7 @@ __device__ __forceinline__ void fixed_hops(const Geom& g, const SpinorF64& in, c
         m = fx_max(m, w.y, w.w);
       }
       if (k == k0) E = max(fx_exponent(m), kFixedMinExp) + 1;
-      fixed_raise(m, E, top, acc);
+      fixed_raise(m, E, top, acc, weak);
     }
     // rows 0, 1 and their partners: row 0 joins spin 3 (x, y) or 2 (z), row 1
     // the other; a real part joins a real one (y) or an imaginary one (x, z)
@@ -462,6 +503,7 @@ __device__ __forceinline__ void fixed_hops(const Geom& g, const SpinorF64& in, c
         hi[s][c] = fx_number(w.z, w.w, e4, cj) + fx_number(vi.x, vi.y, e4, fi);
       }
     }
+    const int w0 = fixed_weight(hr[0], hi[0]), w1 = fixed_weight(hr[1], hi[1]);
     // the next hop's spinor takes the slots just read
     int nn = 0;
     if (k + 1 < k1) {
@@ -475,9 +517,9 @@ __device__ __forceinline__ void fixed_hops(const Geom& g, const SpinorF64& in, c
     fixed_su3(sm, step_i, step_j, hr, hi, gr, gi);
     if (k + 1 < k1 && !(TFIX && k == 5 && !last)) fixed_issue_link(sm, gauge, parity, h, nn, k + 1);
     cp_commit();
-#define WD_FIXED_ADD(MU, S, CONJ)                          \
-  fixed_add<MU, S, CONJ, 0>(gr[0], gi[0], acc);            \
-  fixed_add<MU, S, CONJ, 1>(gr[1], gi[1], acc)
+#define WD_FIXED_ADD(MU, S, CONJ)                                \
+  fixed_add<MU, S, CONJ, 0>(gr[0], gi[0], w0, acc, weak);        \
+  fixed_add<MU, S, CONJ, 1>(gr[1], gi[1], w1, acc, weak)
     switch (k) {
       case 0: WD_FIXED_ADD(0, SF, false); break;
       case 1: WD_FIXED_ADD(0, -SF, true); break;
@@ -499,7 +541,7 @@ __device__ __forceinline__ void fixed_hops(const Geom& g, const SpinorF64& in, c
         m = fx_max(m, w.y, w.w);
       }
       if (k == k0) E = max(fx_exponent(m), kFixedMinExp) + 1;
-      fixed_raise(m, E, top, acc);
+      fixed_raise(m, E, top, acc, weak);
     }
     const bool unit = TFIX && (fwd ? !last : !first);
     const int fm = (g.tbc_anti && (fwd ? last : first)) ? -1 : 0;
@@ -511,6 +553,7 @@ __device__ __forceinline__ void fixed_hops(const Geom& g, const SpinorF64& in, c
       hr[q / 3][q % 3] = fx_number(w.x, w.y, E + 3, fm);
       hi[q / 3][q % 3] = fx_number(w.z, w.w, E + 3, cj);
     }
+    const int w0 = fixed_weight(hr[0], hi[0]), w1 = fixed_weight(hr[1], hi[1]);
     int nn = 0;
     if (fwd) {
       nn = fixed_neighbour(g, h, x, y, z, t, 7);
@@ -548,10 +591,10 @@ __device__ __forceinline__ void fixed_hops(const Geom& g, const SpinorF64& in, c
 template <bool DAGGER, bool TFIX, bool PAIR>
 __device__ __forceinline__ void dslash_site_fixed(const Geom& g, const SpinorF64& in, const GaugeX64& gauge,
                                                   FixedSlots& sm, int h, int parity, double (&out)[24]) {
-  int E, top;
+  int E, top, weak[4];
   long long acc[24];
-  fixed_hops<DAGGER, TFIX>(g, in, gauge, sm, h, parity, 0, 8, E, top, acc);
-  if (top < kFixedMinExp || top > kFixedMaxExp) {
+  fixed_hops<DAGGER, TFIX>(g, in, gauge, sm, h, parity, 0, 8, E, top, acc, weak);
+  if (top < kFixedMinExp || top > kFixedMaxExp || fixed_is_weak(weak)) {
     double slow[24];  // its address is taken on this path only
     if (dslash_site_outside<DAGGER, TFIX, PAIR>(g, in, gauge, h, parity, top, slow)) {
 #pragma unroll
@@ -575,17 +618,18 @@ __device__ __forceinline__ bool dslash_site_fixed_split(const Geom& g, const Spi
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, h = h0 + lane;
   const bool ok = h < h_end;
   if (ok) {
-    int E, top;
+    int E, top, weak[4];
     long long acc[24];
-    fixed_hops<DAGGER, TFIX>(g, in, gauge, sm, h, parity, 2 * w, 2 * w + 2, E, top, acc);
+    fixed_hops<DAGGER, TFIX>(g, in, gauge, sm, h, parity, 2 * w, 2 * w + 2, E, top, acc, weak);
 #pragma unroll
     for (int c = 0; c < 12; ++c)
       *reinterpret_cast<longlong2*>(&sm.sp[c][tid]) = make_longlong2(acc[2 * c], acc[2 * c + 1]);
     sm.lk[0][tid] = make_int4(E, top, 0, 0);
+    sm.lk[4][tid] = make_int4(weak[0], weak[1], weak[2], weak[3]);
   }
   __syncthreads();
   double* fin = reinterpret_cast<double*>(&sm.lk[1][0]);  // [24][32]
-  int top = 0;
+  int top = 0, weak[4] = {0, 0, 0, 0};
   if (ok) {
     int e[4], E = 0;
 #pragma unroll
@@ -601,16 +645,24 @@ __device__ __forceinline__ bool dslash_site_fixed_split(const Geom& g, const Spi
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const longlong2 v = *reinterpret_cast<const longlong2*>(&sm.sp[3 * w + c][lane + 32 * q]);
-        r += fx_sar(v.x, E - e[q]);
-        i += fx_sar(v.y, E - e[q]);
+        r += fx_round_sar(v.x, E - e[q]);
+        i += fx_round_sar(v.y, E - e[q]);
       }
       fin[(6 * w + 2 * c) * 32 + lane] = fx_sum_value(r, E - 1078);
       fin[(6 * w + 2 * c + 1) * 32 + lane] = fx_sum_value(i, E - 1078);
     }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int4 v = sm.lk[4][lane + 32 * q];
+      weak[0] += fx_shr32(v.x, E - e[q]);
+      weak[1] += fx_shr32(v.y, E - e[q]);
+      weak[2] += fx_shr32(v.z, E - e[q]);
+      weak[3] += fx_shr32(v.w, E - e[q]);
+    }
   }
   __syncthreads();
   if (!ok || w != 0) return false;
-  if (top < kFixedMinExp || top > kFixedMaxExp) {
+  if (top < kFixedMinExp || top > kFixedMaxExp || fixed_is_weak(weak)) {
     double slow[24];
     if (dslash_site_outside<DAGGER, TFIX, PAIR>(g, in, gauge, h, parity, top, slow)) {
 #pragma unroll

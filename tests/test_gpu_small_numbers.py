@@ -43,3 +43,84 @@ def test_small_link_elements_of_derived_links(prec, unit, recon, small):
     odd = parity_sites(DIMS, 1)
     assert np.abs(want[odd]).max() > 4 * bound
     assert np.abs(got - want)[odd].max() <= bound
+
+
+# --------------------------------------------- FP64: spins and colours of very different size
+def _fields(dims, parity, seed, spread):
+    """Device field (12, sites of the parity) of numbers 2^-k, k up to `spread`, by site, spin and colour, in the
+    basis and order of device fields, and the same as (T, Z, Y, X, 4, 3) with zeros on the other parity."""
+    rng = np.random.default_rng(seed)
+    full = rng.normal(size=(li.volume(dims), 4, 3)) + 1j * rng.normal(size=(li.volume(dims), 4, 3))
+    full *= np.exp2(-spread * rng.random((li.volume(dims), 4, 3)))
+    sites = parity_sites(dims, parity)
+    out = np.zeros_like(full)
+    out[sites] = full[sites]
+    return full[sites].reshape(-1, 12).T, out.reshape(*dims[::-1], 4, 3)
+
+
+def _feeds(U, psi, dims, dagger):
+    """Sum of |u| |psi| over the terms of each output: a spatial hop adds to a spin itself and its partner, a
+    temporal one twice the spins that its projector keeps."""
+    a, u = np.abs(psi), np.abs(U).reshape(*dims[::-1], 4, 3, 3)
+    out = np.zeros_like(a)
+    for mu in range(4):
+        for fwd in (True, False):
+            if fwd:
+                h = np.einsum("...ij,...sj->...si", u[..., mu, :, :], np.roll(a, -1, 3 - mu))
+            else:
+                h = np.roll(np.einsum("...ji,...sj->...si", u[..., mu, :, :], a), 1, 3 - mu)
+            if mu == 3:
+                keep = slice(2, 4) if fwd != dagger else slice(0, 2)
+                out[..., keep, :] += 2 * h[..., keep, :]
+            else:
+                partner = [3, 2, 1, 0] if mu < 2 else [2, 3, 0, 1]
+                out += h + h[..., partner, :]
+    return out.reshape(-1, 12)
+
+
+def _raw_dslash(U, dims, raw, dagger, recon):
+    """(sites of parity 1, 12) complex: the stored numbers of D applied to a device field."""
+    import paper_0911_3191_gb300 as m
+    import torch
+    vh, st = raw.shape[1], (raw.shape[1] + 31) // 32 * 32
+    buf = np.zeros((12, st, 2))
+    buf[:, :vh, 0], buf[:, :vh, 1] = raw.real, raw.imag
+    wd = m.WilsonDirac(dims)
+    wd.load_gauge(U, recon=recon)
+    o = wd.new_field(m.F64)
+    wd.dslash(o, torch.from_numpy(buf).cuda().view(torch.uint8).reshape(-1), 1, dagger, m.F64)
+    out = o.cpu().numpy()[: 192 * st].view(np.float64).reshape(12, st, 2)[:, :vh]
+    wd.close()
+    return (out[..., 0] + 1j * out[..., 1]).T
+
+
+# one thread per site and four warps per 32 sites
+@pytest.mark.parametrize("dims", [(4, 6, 8, 10), (16, 14, 12, 18)])
+@pytest.mark.parametrize("recon,dagger", [(18, False), (12, True)])
+@pytest.mark.parametrize("spread", [0, 6, 25, 90, "spin", "colour"])
+def test_fp64_by_component(dims, recon, dagger, spread):
+    """Every spin and colour is right to the sum of the |u| |psi| that feed it, however small beside the others.
+    A field with a link that the integer form does not take is computed in FP64 throughout: its result is the
+    reference away from that link.
+    18 reals: 23 units of 2^-55 of the common exponent at most in a real part, and what feeds a component is at least
+    2^-6 of it, or the site is computed in FP64: 23 sqrt(2) 2^-49, and FP64's 2^-48.  12 reals: the third row, which
+    both rebuild, is right to a few 2^-53 absolute, which is 64 times as much of a component fed by 2^-6."""
+    U = li.gauge(dims, 0.7, 1600)
+    raw, psi = _fields(dims, 0, 2601, spread if isinstance(spread, int) else 0)
+    if isinstance(spread, str):  # one spin (colour) 1e-18 of the others, links that do not mix it with them
+        small = (np.arange(12) // 3 != 1) if spread == "spin" else (np.arange(12) % 3 == 1)
+        raw = raw * np.where(small, 1e-18, 1.0)[:, None]
+        psi = (psi.reshape(-1, 12) * np.where(small, 1e-18, 1.0)).reshape(psi.shape)
+        U = U * np.eye(3)
+        U /= np.abs(U).sum(-1, keepdims=True)
+    if recon == 12:
+        U[:, :, 2] = np.cross(U[:, :, 0], U[:, :, 1]).conj()
+    V = U.copy()
+    V[37, 2] *= 1.5
+    got, want = _raw_dslash(U, dims, raw, dagger, recon), _raw_dslash(V, dims, raw, dagger, recon)
+    feeds, feeds2 = _feeds(U, psi, dims, dagger), _feeds(V, psi, dims, dagger)
+    odd = parity_sites(dims, 1)
+    away = (feeds == feeds2).all(axis=1)[odd]
+    assert away.sum() >= len(odd) - 2
+    bound = (2.0 ** -43.8 if recon == 18 else 2.0 ** -40) * feeds[odd]
+    assert (np.abs(got - want) <= bound)[away].all(), np.nanmax(np.abs(got - want)[away] / feeds[odd][away])
