@@ -1159,8 +1159,29 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 __device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
-  const double i = 1.0 / (b.x * b.x + b.y * b.y);  // one division: some ten dependent FP64 operations
+  const double d = b.x * b.x + b.y * b.y;
+  return make_double2((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
+}
+// biased exponent of the larger part
+__device__ __forceinline__ int cexponent(double2 a) {
+  return max(__double2hiint(a.x) & 0x7fffffff, __double2hiint(a.y) & 0x7fffffff) >> 20;
+}
+// 2^-448 <= |a| < 2^449: |a|^2, its reciprocal and products of the two with such numbers are normal
+__device__ __forceinline__ bool cmoderate(double2 a) { return (unsigned)(cexponent(a) - 575) < 896u; }
+// a / b by one reciprocal, where that neither overflows nor is lost: one rounding
+// more than cdiv, and one division fewer (some ten dependent FP64 operations)
+__device__ __forceinline__ double2 cdiv_r(double2 a, double2 b) {
+  if (!cmoderate(a) || !cmoderate(b)) return cdiv(a, b);
+  const double i = 1.0 / (b.x * b.x + b.y * b.y);
   return make_double2((a.x * b.x + a.y * b.y) * i, (a.y * b.x - a.x * b.y) * i);
+}
+// (a / b) (c / d) as (a c) / (b d): one division for four, and no more roundings
+// (two products, the quotient's sums, reciprocal and product) than two quotients
+// and their product have
+__device__ __forceinline__ double2 cratio(double2 a, double2 b, double2 c, double2 d) {
+  const double2 n = cmul(a, c), m = cmul(b, d);
+  if (cmoderate(n) && cmoderate(m)) return cdiv_r(n, m);
+  return cmul(cdiv(a, b), cdiv(c, d));
 }
 __device__ __forceinline__ bool cfinite(double2 a) { return isfinite(a.x) && isfinite(a.y); }
 

@@ -126,7 +126,7 @@ struct FinBicgIter {
     ctl->rr = rr;
     ctl->rho_prev = ctl->rho;
     ctl->rho = rho_new;
-    ctl->beta = cdiv(cmul(rho_new, ctl->alpha), cmul(ctl->rho_prev, ctl->omega));
+    ctl->beta = cratio(rho_new, ctl->rho_prev, ctl->alpha, ctl->omega);
     decide_update(ctl, (rho_new.x == 0.0 && rho_new.y == 0.0) ? 0.0 : rr, ctl->stop2);
   }
 };
@@ -155,7 +155,7 @@ struct FinRelupBicg {
       ctl->beta = make_double2(0.0, 0.0);
     } else {
       ctl->rho = rho;
-      ctl->beta = cdiv(cmul(rho, ctl->alpha), cmul(ctl->rho_prev, ctl->omega));
+      ctl->beta = cratio(rho, ctl->rho_prev, ctl->alpha, ctl->omega);
     }
     if (r2 <= ctl->stop2) { ctl->status = WD_OK; ctl->done = 1; }
     else if (ctl->iter >= ctl->max_iter) ctl_fail(ctl, WD_ERR_NOT_CONVERGED);

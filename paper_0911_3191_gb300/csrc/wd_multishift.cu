@@ -208,27 +208,28 @@ struct FinMsIter {
     const double rn = sqrt(t[2]);
     if (!isfinite(rn) || !cfinite(rho_new)) { ms_fail(m, WD_ERR_NUMERIC); return; }
     const double2 alpha = m->alpha, omega = m->omega;
-    const double2 beta = cmul(cdiv(alpha, omega), cdiv(rho_new, m->rho));
+    const double2 beta = cratio(alpha, omega, rho_new, m->rho);
+    // (the quotients here are FP32 in the end)
     for (int k = 0; k < m->n; ++k) {
       ShiftCoef q{};
       if (m->active[k]) {
         const double sg = m->tau[k];
         const double2 fz = m->fz[k], gz = m->gz[k], pz = m->pz[k];
         const double2 f_next = c_add(fz, cmul(c_scale(sg, alpha), gz));
-        const double2 alpha_s = cdiv(cmul(alpha, fz), f_next);
+        const double2 alpha_s = cdiv_r(cmul(alpha, fz), f_next);
         const double2 one_ws = c_add(make_double2(1.0, 0.0), c_scale(sg, omega));
-        const double2 omega_s = cdiv(omega, one_ws);
+        const double2 omega_s = cdiv_r(omega, one_ws);
         const double2 pi_next = cmul(pz, one_ws);
-        const double2 ratio = cdiv(fz, f_next);
+        const double2 ratio = cdiv_r(fz, f_next);
         const double2 beta_s = cmul(beta, cmul(ratio, ratio));
-        const double2 qq = cdiv(cmul(beta_s, omega_s), alpha_s);
+        const double2 qq = cdiv_r(cmul(beta_s, omega_s), alpha_s);
         const double2 pf = cmul(pz, f_next);
         q.ax = c_f2(alpha_s);
-        q.as = c_f2(cdiv(omega_s, pf));
-        q.c1 = c_f2(cdiv(make_double2(1.0, 0.0), cmul(pi_next, f_next)));
+        q.as = c_f2(cdiv_r(omega_s, pf));
+        q.c1 = c_f2(cdiv_r(make_double2(1.0, 0.0), cmul(pi_next, f_next)));
         q.c2 = c_f2(beta_s);
-        q.c3 = c_f2(cdiv(c_scale(-1.0, qq), cmul(pz, fz)));
-        q.c4 = c_f2(cdiv(qq, pf));
+        q.c3 = c_f2(cdiv_r(c_scale(-1.0, qq), cmul(pz, fz)));
+        q.c4 = c_f2(cdiv_r(qq, pf));
         q.active = 1;
         m->gz[k] = c_add(f_next, cmul(beta, gz));
         m->fz[k] = f_next;

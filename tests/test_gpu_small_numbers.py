@@ -124,3 +124,21 @@ def test_fp64_by_component(dims, recon, dagger, spread):
     assert away.sum() >= len(odd) - 2
     bound = (2.0 ** -43.8 if recon == 18 else 2.0 ** -40) * feeds[odd]
     assert (np.abs(got - want) <= bound)[away].all(), np.nanmax(np.abs(got - want)[away] / feeds[odd][away])
+
+
+@pytest.mark.parametrize("exp2", [-264, -240])
+def test_solver_coefficients_of_a_small_source(exp2):
+    """|b|^2 about 2^-513 (2^-465): the square in the complex divisions is below 2^-1024, which is a number but its
+    reciprocal is not."""
+    import paper_0911_3191_gb300 as m
+    U = li.gauge(DIMS, 0.4, 1700)
+    b = li.gaussian_spinor(DIMS, 2700)
+    assert -514 < np.log2(np.linalg.norm(b) ** 2) - 528 < -512
+    wd = m.WilsonDirac(DIMS)
+    wd.load_gauge(U)
+    for graph in (False, True):
+        x = np.zeros_like(b)
+        r = wd.solve(x, b * 2.0 ** exp2, 0.12, tol=0.05, solver=0, inner_precision=0, use_graph=graph, max_iter=50,
+                     check=False)
+        assert r.status == 0 and oracle.true_residual(x * 2.0 ** -exp2, b, U, DIMS, 0.12) <= 0.05, r
+    wd.close()
