@@ -193,12 +193,17 @@ __device__ __forceinline__ int fx_exponent(float m) { return (int)(__float_as_ui
 // pipe bounds.  A vector becomes integers of 58 bits in the unit of its largest
 // exponent, each split into two signed halves; a product is three 32-bit
 // multiply-adds (12 cycles or so of an SM quarter, an FP64 one 67), the product of
-// the low halves (2^-58 of the two largest components' product) dropped, and a
-// site's 24 products are added exactly.  Cutting, dropping and rounding leave less
-// than FP64 products and sums do.
+// the low halves dropped, and a site's 24 products are added exactly.
+//
+// Cutting (48), dropping (6) and rounding are at most 55 units of 2^-114 to 2^-116
+// of 2^58 x 2^58, the two vectors' units; 24 FP64 multiply-adds may be off by 24 x
+// 2^-53 of the sum of |w| |a|.  So the integers are no worse wherever that sum is
+// 2^54.2 units or more, as a norm's always is (2^56), and the products of vectors
+// whose large components do not meet are left to FP64 (fx_products).
 constexpr int kFxSiteMinExp = 600, kFxSiteMaxExp = 1500;  // (biased) squares and scales stay normal doubles
+constexpr int kFxDense = 5 << 18;  // 2^54.3 units as products of the halves' upper 12 bits
 // biased exponent of the largest of 24 doubles; 24 zeros, as most sites of a point
-// source are, count as in range
+// source are, count as in range, with an exponent of their own
 __device__ __forceinline__ int fx_site_exp(const double (&x)[24]) {
   float m = 0.f;
 #pragma unroll
@@ -209,7 +214,8 @@ __device__ __forceinline__ int fx_site_exp(const double (&x)[24]) {
     for (int k = 0; k < 24; ++k) lo |= (unsigned)__double2loint(x[k]);
     return lo ? 0 : kFxSiteMinExp;
   }
-  return (int)(__float_as_uint(m) >> 20);
+  const int e = (int)(__float_as_uint(m) >> 20);
+  return e == kFxSiteMinExp ? 0 : e;
 }
 __device__ __forceinline__ bool fx_site_ok(int e) { return e >= kFxSiteMinExp && e <= kFxSiteMaxExp; }
 struct FxSite {
@@ -254,6 +260,21 @@ __device__ __forceinline__ double2 fx_dot(const FxSite& w, const FxSite& a) {
     im.add(-w.h[k + 1], -w.l[k + 1], a.h[k], a.l[k]);
   }
   return make_double2(re.value(w.e, a.e), im.value(w.e, a.e));
+}
+
+// the larger part of complex number k, the upper 12 bits of its upper half
+__device__ __forceinline__ int fx_part(const FxSite& a, int k) { return max(abs(a.h[2 * k]), abs(a.h[2 * k + 1])) >> 17; }
+// |a|^2 and <w, a>, or false where FP64 has to form them
+__device__ __forceinline__ bool fx_products(const double (&wv)[24], const double (&av)[24], double& norm2, double2& dot) {
+  const int ea = fx_site_exp(av), ew = fx_site_exp(wv);
+  if (!fx_site_ok(ea) || !fx_site_ok(ew)) return false;
+  const FxSite a(av, ea), w(wv, ew);
+  int met = 0;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) met += fx_part(w, k) * fx_part(a, k);
+  norm2 = fx_norm2(a);
+  dot = fx_dot(w, a);
+  return met >= kFxDense || ea == kFxSiteMinExp || ew == kFxSiteMinExp;
 }
 
 __device__ __forceinline__ int fixed_neighbour(const Geom& g, int h, int x, int y, int z, int t, int k) {

@@ -838,6 +838,14 @@ struct OpBicgFinal {
   __device__ __forceinline__ OpBicgFinal at(int q) const {
     return OpBicgFinal{xh.at(q), p.at(q), r.at(q), t.at(q), rt.at(q), ctl + q, rs, fin.at(q)};
   }
+  __device__ static void load_again(const SpinorF64& f, int h, double (&v)[24]) {
+    const volatile double* q = reinterpret_cast<const volatile double*>(f.p);
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+      v[2 * c] = q[2 * ((size_t)c * f.stride + h)];
+      v[2 * c + 1] = q[2 * ((size_t)c * f.stride + h) + 1];
+    }
+  }
   __device__ __forceinline__ void operator()(int h, double* red) const {
     using R = typename S::real;
     const double2 al = ctl->alpha, om = ctl->omega;
@@ -853,15 +861,18 @@ struct OpBicgFinal {
     r.store_get(h, sv);
     rt.load(h, wv);
     if constexpr (sizeof(R) == 8) {
-      const int ea = fx_site_exp(sv), ew = fx_site_exp(wv);
-      if (fx_site_ok(ea) && fx_site_ok(ew)) {
-        const FxSite a(sv, ea), w(wv, ew);
-        const double2 d = fx_dot(w, a);
-        red[0] += fx_norm2(a);
+      double n2;
+      double2 d;
+      if (fx_products(wv, sv, n2, d)) {
+        red[0] += n2;
         red[1] += d.x;
         red[2] += d.y;
         return;
       }
+      // read again, by loads that see the store and that the compiler does not
+      // take for the first ones: kept, they would need the integers' registers
+      load_again(r, h, sv);
+      load_again(rt, h, wv);
     }
     R n = 0, re = 0, im = 0;
 #pragma unroll
