@@ -508,12 +508,12 @@ __global__ void __launch_bounds__(kDslashBlock, (DslashOccupancy<R, In, Epi::NRE
 // partner is computed alone.
 // 128 x 4 threads of the 48 KB ring fit an SM; the fp16 temporal-gauge hops
 // spill there and are 1-2 % faster at 3 blocks, the others 2-5 % at 4.
-template <class In, int NRED, bool TFIX>
+template <class In, bool TFIX>
 struct PairOccupancy {
   static constexpr int kMinBlocks = (TFIX && !In::kPairedHops) ? 3 : 4;
 };
 template <bool DAGGER, bool TFIX, class In, class G, class Epi>
-__global__ void __launch_bounds__(kDslashBlock, (PairOccupancy<In, Epi::NRED, TFIX>::kMinBlocks))
+__global__ void __launch_bounds__(kDslashBlock, (PairOccupancy<In, TFIX>::kMinBlocks))
     dslash_rhs_pair_kernel(Geom g, In in, G gauge, int parity, Epi epi, BatchArgs ba) {
   pdl_wait();
   constexpr int NR = Epi::NRED > 0 ? Epi::NRED : 1;
