@@ -337,8 +337,8 @@ wd_status wd_solve_multishift_device(wd_ctx *ctx, int n, void *x, const void *b,
  * batched solver above).  Requests that arrive while others are running are
  * admitted at the next step as slots and memory free up; every device
  * allocation is charged against budget_bytes, the integer copy of the FP64
- * links (wd_load_gauge) among a field's solver slots: it is made with them when
- * it takes at most a quarter of their memory.  Each gauge field has its own
+ * links (wd_load_gauge) with a field's solver slots: it is made as soon as they
+ * leave room for it and for one slot of every waiting field.  Each gauge field has its own
  * CUDA stream, so solves on different volumes overlap on the device.  A
  * request's iterates follow the same kernel sequence alone and in a mix. */
 typedef struct wd_server wd_server;

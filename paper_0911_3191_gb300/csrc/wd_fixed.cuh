@@ -8,7 +8,7 @@
 // product of two takes three integer multiply-adds: 148 us (its bytes take 81);
 // M_hat with 12-real general links of 20 x 14 x 22 x 38 130 us; 8^3 x 16, four
 // warps per 32 sites, 5.9 us.  No pipe is full: 12 warps per SM (168 registers)
-// leave the latencies of 6200 dependent integer instructions per 32 sites in sight.
+// leave the latencies of 6300 dependent integer instructions per 32 sites in sight.
 //
 //  * A link element u, |u| <= 1, is the integer u 2^60 (converted once, when
 //    the links are loaded).  A double of at least 2^-8 is exact in it, a

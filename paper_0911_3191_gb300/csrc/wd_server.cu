@@ -266,8 +266,8 @@ void release_workspace(Pool& pl, size_t& used) {
 }
 
 // Workspace for `cap` slots: the batch views of wd_batch.cuh plus one FP64
-// full source field per slot, and (fixed) the fixed-point links.
-wd_status alloc_workspace(wd_server* sv, Pool& pl, int cap, bool fixed) {
+// full source field per slot.
+wd_status alloc_workspace(wd_server* sv, Pool& pl, int cap) {
   Ctx& c = pl.ctx->c;
   const int prec = sv->p.inner_precision;
   const size_t f64 = fbytes(c, WD_F64), fin = fbytes(c, prec);
@@ -284,8 +284,7 @@ wd_status alloc_workspace(wd_server* sv, Pool& pl, int cap, bool fixed) {
   // land after the slots' control blocks are initialised
   WS_CK(sv, cudaMemsetAsync(pl.small, 0, sm, c.stream));
   WS_CK(sv, cudaMallocHost((void**)&pl.hctl, (size_t)cap * sizeof(SolverCtl)));
-  if (fixed) make_fixed_links(c);
-  pl.ws_bytes = ws + sm + (c.gauge_fx ? fixed_link_bytes(c) : 0);
+  pl.ws_bytes = ws + sm;
   sv->used += pl.ws_bytes;
   pl.capacity = cap;
   pl.slot_req.assign(cap, -1);
@@ -319,11 +318,38 @@ wd_status alloc_workspace(wd_server* sv, Pool& pl, int cap, bool fixed) {
   pl.bl = pool_shape(c, cap, sv->p.rhs_tile);
   mark_free_kernel<<<(cap + 127) / 128, 128, 0, c.stream>>>(b.ctl, cap);
   WS_CK(sv, cudaGetLastError());
-  if (sv->p.use_graph) {
-    cudaError_t e = build_batch_loop_graph(c, prec, b, pl.bl, &pl.graph, &pl.exec, &pl.hu, &pl.hl);
+  WS_CK(sv, cudaStreamSynchronize(c.stream));
+  return WD_OK;
+}
+
+// memory of n slots
+size_t slots_bytes(const wd_server* sv, const Ctx& c, int n) {
+  return slot_bytes(c, sv->p.inner_precision) * n + small_bytes(c, n, sv->p.rhs_tile);
+}
+
+// Before a step of a pool with slots: the fixed-point links (an FP64 dslash in a
+// third of the time) as soon as the budget has them beside one slot for every pool
+// that waits, and the loop's graph when it is missing or was captured without them.
+wd_status ensure_links_and_graph(wd_server* sv, Pool& pl) {
+  Ctx& c = pl.ctx->c;
+  if (!c.gauge_fx && c.fixed_ok) {
+    size_t need = sv->used + fixed_link_bytes(c);
+    for (const Pool& q : sv->pools)
+      if (!q.queue.empty() && !q.capacity) need += slots_bytes(sv, q.ctx->c, 1);
+    if (!sv->p.budget_bytes || need <= sv->p.budget_bytes) make_fixed_links(c);
+    if (c.gauge_fx) {
+      pl.ws_bytes += fixed_link_bytes(c);
+      sv->used += fixed_link_bytes(c);
+      if (pl.exec) cudaGraphExecDestroy(pl.exec);
+      if (pl.graph) cudaGraphDestroy(pl.graph);
+      pl.exec = nullptr;
+      pl.graph = nullptr;
+    }
+  }
+  if (sv->p.use_graph && !pl.exec) {
+    cudaError_t e = build_batch_loop_graph(c, sv->p.inner_precision, pl.bb, pl.bl, &pl.graph, &pl.exec, &pl.hu, &pl.hl);
     if (e != cudaSuccess) return serr(sv, WD_ERR_CUDA, std::string("pool graph: ") + cudaGetErrorString(e));
   }
-  WS_CK(sv, cudaStreamSynchronize(c.stream));
   return WD_OK;
 }
 
@@ -559,18 +585,22 @@ wd_status pool_progress(wd_server* s, Pool& pl, int& waiting_for_memory, bool& d
     // slot memory: what the budget has left, shared with the other pools that wait
     const size_t left = s->p.budget_bytes ? (s->p.budget_bytes > s->used ? s->p.budget_bytes - s->used : 0)
                                           : (size_t)-1;
-    const size_t share = s->p.budget_bytes ? left / (size_t)std::max(1, waiting_for_memory) : left;
-    // the fixed-point links, where they take a quarter of it at most: an FP64 dslash
-    // in a third of the time is worth more than the slots there would be for them
-    const size_t fx = c.fixed_ok && fixed_link_bytes(c) <= share / 4 ? fixed_link_bytes(c) : 0;
+    // its share: what one slot and the fixed-point links take, and an equal part of
+    // what those of all waiting pools leave; of all there is if they do not fit
+    size_t all = 0;
+    for (const Pool& q : s->pools)
+      if (!q.queue.empty() && !q.capacity)
+        all += slots_bytes(s, q.ctx->c, 1) + (q.ctx->c.fixed_ok ? fixed_link_bytes(q.ctx->c) : 0);
+    const size_t waiting = (size_t)std::max(1, waiting_for_memory);
+    const size_t share = !s->p.budget_bytes ? left
+                         : all <= left      ? slots_bytes(s, c, 1) + (left - all) / waiting
+                                            : left / waiting;
     int cap = s->p.max_slots;
-    while (cap > 0 && s->p.budget_bytes &&
-           slot_bytes(c, prec) * cap + small_bytes(c, cap, s->p.rhs_tile) + fx > share)
-      --cap;
-    if (cap < 1 && s->p.budget_bytes && slot_bytes(c, prec) + small_bytes(c, 1, s->p.rhs_tile) <= left) cap = 1;
+    while (cap > 0 && s->p.budget_bytes && slots_bytes(s, c, cap) > share) --cap;
+    if (cap < 1 && s->p.budget_bytes && slots_bytes(s, c, 1) <= left) cap = 1;
     if (cap >= 1) {
       --waiting_for_memory;
-      wd_status st = alloc_workspace(s, pl, cap, fx > 0);
+      wd_status st = alloc_workspace(s, pl, cap);
       if (st != WD_OK) return st;
       did_work = true;
     }
@@ -587,6 +617,7 @@ wd_status pool_progress(wd_server* s, Pool& pl, int& waiting_for_memory, bool& d
   int n = 0;
   for (long long id : pl.slot_req) n += (id >= 0);
   if (!n) return WD_OK;
+  if (wd_status lst = ensure_links_and_graph(s, pl); lst != WD_OK) return lst;
   // up to iters_per_step lockstep iterations, then an event marks the end
   if (!pl.start_ev) WS_CK(s, cudaEventCreate(&pl.start_ev));
   if (!pl.done_ev) WS_CK(s, cudaEventCreate(&pl.done_ev));
@@ -773,9 +804,7 @@ wd_status wd_server_submit(wd_server* s, int gauge_id, const double* b, double* 
     const Pool& pl = s->pools[gauge_id];
     size_t fixed = 0;
     for (const Pool& q : s->pools) fixed += q.fixed_bytes;
-    if (s->p.budget_bytes &&
-        fixed + slot_bytes(pl.ctx->c, s->p.inner_precision) + small_bytes(pl.ctx->c, 1, s->p.rhs_tile) >
-            s->p.budget_bytes)
+    if (s->p.budget_bytes && fixed + slots_bytes(s, pl.ctx->c, 1) > s->p.budget_bytes)
       return serr(s, WD_ERR_BUDGET, "one solver slot for this lattice exceeds the memory budget");
   }
   const size_t field = (size_t)2 * s->pools[gauge_id].ctx->c.g.Vh * 24 * sizeof(double);
