@@ -75,7 +75,7 @@ FP64_PEAK_TFLOPS = 1.252
 # (precision, link reals, lattice, temporal gauge).  KERNEL_SOURCES_SHA is the
 # hash of the kernel sources the counters were taken on (kernel_sources_sha());
 # when the sources differ, the bench reports traffic as null.
-KERNEL_SOURCES_SHA = "1d35d5902bb5bfe7"
+KERNEL_SOURCES_SHA = "9310aed4479d49ae"
 NCU_TRAFFIC_BYTES = {("f64", 18, "24x24x24x64", True): 5.224e+08, ("q16", 12, "24x24x24x64", True): 9.118e+07}
 
 

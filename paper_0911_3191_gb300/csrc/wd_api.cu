@@ -87,7 +87,7 @@ __global__ void gauge_pack_f64_kernel(Geom g, const double* lex, double2* out, i
           row += fabs(r[6 * c + 2 * j]) + fabs(r[6 * c + 2 * j + 1]);
           col += fabs(r[6 * j + 2 * c]) + fabs(r[6 * j + 2 * c + 1]);
         }
-        ok = ok && row >= kFixedLinkMin && col >= kFixedLinkMin;
+        ok = ok && fmin(row, col) >= kFixedLinkMin && fmax(row, col) <= kFixedLinkSum;
       }
       bad += !ok;
     }

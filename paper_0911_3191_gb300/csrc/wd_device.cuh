@@ -526,19 +526,19 @@ __device__ __forceinline__ void su3_from8(const float (&p)[8], float (&u)[18]) {
 }
 
 // --------------------------------------------------------- fixed-point links
-// Beside the FP64 links a context keeps a copy as 64-bit integers u 2^60, each as
+// Beside the FP64 links a context keeps a copy as 64-bit integers u 2^61, each as
 // two signed 32-bit limbs (high, low), for the integer-pipe dslash of wd_fixed.cuh,
-// when every element of the field satisfies |u| <= kFixedLinkMax and the parts of no
-// row or column add up to less than kFixedLinkMin (SU(3) links do both).
+// when every element of the field satisfies |u| <= kFixedLinkMax and the parts of
+// each row and column add up to kFixedLinkMin .. kFixedLinkSum (1 .. sqrt(6) in SU(3)).
 // Both take the same 16 bytes per complex number.  Only that dslash reads it: the
 // links of the other precisions, the slab faces and the sites that it leaves to FP64
-// come from the doubles, since an element below 2^-8 is not exact in the integers.
-constexpr double kFixedLinkMax = 1.125, kFixedLinkMin = 0.99;
+// come from the doubles, since an element below 2^-9 is not exact in the integers.
+constexpr double kFixedLinkMax = 1.125, kFixedLinkMin = 0.99, kFixedLinkSum = 3.5;
 
-// u 2^60, rounded to nearest (|u| <= kFixedLinkMax), as (high limb, low limb)
+// u 2^61, rounded to nearest (|u| <= kFixedLinkMax), as (high limb, low limb)
 __device__ __forceinline__ int2 fx_link(double u) {
   const long long w = __double_as_longlong(u);
-  const int s = 1026 - (int)((w >> 52) & 0x7ff);
+  const int s = 1025 - (int)((w >> 52) & 0x7ff);
   const unsigned long long m = ((unsigned long long)w << 11) | 0x8000000000000000ull;
   unsigned long long a = s > 64 ? 0ull : ((m >> (s - 1)) + 1) >> 1;
   const long long v = w < 0 ? -(long long)a : (long long)a;

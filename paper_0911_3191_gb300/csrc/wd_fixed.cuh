@@ -10,39 +10,39 @@
 // warps per 32 sites, 5.9 us.  No pipe is full: 12 warps per SM (168 registers)
 // leave the latencies of 6300 dependent integer instructions per 32 sites in sight.
 //
-//  * A link element u, |u| <= 1, is the integer u 2^60 (converted once, when
-//    the links are loaded).  A double of at least 2^-8 is exact in it, a
-//    smaller one is off by at most 2^-61.
+//  * A link element u, |u| <= 1, is the integer u 2^61 (converted once, when
+//    the links are loaded).  A double of at least 2^-9 is exact in it, a
+//    smaller one is off by at most 2^-62.
 //  * The spinors of a site's neighbours share one exponent E (|x| < 2^(E-1023)
 //    for all of their components): x is the integer x 2^(59-(E-1023)), so a
 //    projected component, a sum of two, is below 2^60.
 //  * Both are kept as two signed 32-bit limbs, a = ah 2^32 + al with al in
 //    [-2^31, 2^31).  Of a product's limbs ah bh, (ah bl + al bh) 2^-32 and
-//    al bl 2^-64, the last is left out: at most a quarter of the unit 2^(E-1078)
+//    al bl 2^-64, the last is left out: at most a quarter of the unit 2^(E-1079)
 //    in which the sums are kept.
 //  * The 24 sums are 64-bit integers of that unit, rounded once, to the double they
 //    become.
 //
 // Accuracy.  B = 2^(E-1023) is one to four times the largest neighbour component.
-// The sums are off by 23 units of 2^-55 B at most (a hop: 1.5 dropped limbs, 0.5 the
-// middle sums' rounding, 0.6 the cut numbers; one the shifts to a larger E) and by
-// one unit as a rule: over Gaussian fields 0.8e-16 of the largest component against
-// 1.5e-16 for FP64 arithmetic.  FP64 rounds each component relative to what feeds
-// it, though, sum |u| |psi|, which may be far less than B.  So each spin collects the
-// smallest colour of every row that feeds it (fixed_weight), and a site with a spin
-// that gets less than 2^-6 B is computed in FP64 (dslash_site).  What is left is
-// right to 2^-44 of sum |u| |psi| in every complex component, and as a rule to
-// 2^-49, the bound that FP64's 15 roundings have.  No site of Gaussian fields goes
-// that way, 5e-4 of a point source's solution at kappa 0.12, and the fronts of its
-// first iterates.  The weights take 2 % of the dslash (144.6 -> 148.0 us at
-// 24^3 x 64), the FP64 sites 3 % of twelve point sources' batch on 16^3 x 32.
-// (A third row rebuilt from 12 reals is right to a few 2^-53 of 1, here and in FP64.)
+// The sums are off by 25 units of 2^-56 B at most (a hop: 1.5 dropped limbs, 0.5 the
+// middle sums' rounding, 1.0 the cut numbers; one the shifts to a larger E) and by
+// one unit as a rule; FP64 rounds each component relative to what feeds it, sum |u|
+// |psi|, which is more than B in ordinary fields but may be far less.  So each spin
+// collects the smallest colour of every row that feeds it (fixed_weight), and a site
+// with a spin that gets less than 2^-7 B is computed in FP64 (dslash_site).  What is
+// left is right to 2^-43 of sum |u| |psi| in every complex component, and as a rule
+// to 2^-49, the bound that FP64's 15 roundings have.  No site of Gaussian fields
+// goes that way, 2e-4 of a point source's solution at kappa 0.12, and the fronts of
+// its first iterates.  The weights take 2 % of the dslash (144.6 -> 148.0 us at
+// 24^3 x 64), the FP64 sites 1 % of twelve point sources' batch on
+// 16^3 x 32.
+// (A third row rebuilt from 12 reals is right to a few 2^-53 of 1 in FP64.)
 //
 // E is known only when all neighbours are, so it is a running maximum: a hop
 // that raises it shifts the sums down.  Starting one above the first hop's
-// exponent makes that rare.  Sums cannot overflow: with |u| <= 1.125 (the rule
-// by which links take this form, kFixedLinkMax) each of the eight hops adds at
-// most 6 x 1.125 x 2^56, and a middle sum stays below 12 x 1.125 x 2^59.
+// exponent makes that rare.  Sums cannot overflow: where the parts of a row add up
+// to 3.5 (kFixedLinkSum, a rule by which links take this form), each of the eight
+// hops adds at most 3.5 x 2^57, and a middle sum stays below 3.5 x 2^60 + 6 x 2^59.
 //
 // Sites whose neighbours hold an infinity, a NaN, or only numbers outside
 // 2^-830 .. 2^870 are computed by dslash_site in FP64 as well.
@@ -54,7 +54,7 @@
 namespace wd {
 
 constexpr int kFixedMinExp = 192, kFixedMaxExp = 1892;  // biased exponents E of the fixed-point path
-constexpr int kFixedWeak = 1 << 21;  // 2^-6 of the common exponent, in the unit of the high words (fixed_weight)
+constexpr int kFixedWeak = 1 << 20;  // 2^-7 of the common exponent, in the unit of the high words (fixed_weight)
 
 struct Fx {
   int h, l;  // h * 2^32 + l
@@ -123,7 +123,7 @@ struct FixedSlots {
 
 // a b + c d - e f - g q of link elements, as a link element
 __device__ __forceinline__ long long fx_minor(Fx a, Fx b, Fx c, Fx d, Fx e, Fx f, Fx g, Fx q) {
-  long long hp = fx_mad(a.h, b.h, 0), mp = fx_mad(a.h, b.l, 1ll << 27);
+  long long hp = fx_mad(a.h, b.h, 0), mp = fx_mad(a.h, b.l, 1ll << 28);
   mp = fx_mad(a.l, b.h, mp);
   hp = fx_mad(c.h, d.h, hp);
   mp = fx_mad(c.h, d.l, mp);
@@ -133,7 +133,7 @@ __device__ __forceinline__ long long fx_minor(Fx a, Fx b, Fx c, Fx d, Fx e, Fx f
   hq = fx_mad(g.h, q.h, hq);
   mq = fx_mad(g.h, q.l, mq);
   mq = fx_mad(g.l, q.h, mq);
-  return ((hp - hq) << 4) + ((mp - mq) >> 28);
+  return ((hp - hq) << 3) + ((mp - mq) >> 29);
 }
 
 // row c = (a x b)^* of a 12-real link, written to its slots
@@ -159,7 +159,7 @@ __device__ __forceinline__ void fx_row3(FixedSlots& sm) {
 // common exponent, e4 = E + 4: |x| 2^(59-(E-1023)) cut to an integer, 0 for a
 // denormal or a zero, times the sign of x and of the mask `flip` (0 or -1).  A
 // negative number is the one's complement of its magnitude, one unit (2^-59 of
-// the largest component, a sixteenth of the unit of the sums) too low; a zero
+// the largest component, an eighth of the unit of the sums) too low; a zero
 // stays zero in the sums, which round.
 __device__ __forceinline__ unsigned fx_xor3(unsigned a, unsigned b, unsigned c) {
   unsigned r;
@@ -362,11 +362,11 @@ __device__ __forceinline__ bool fixed_is_weak(const int (&weak)[4]) {
   return min(min(weak[0], weak[1]), min(weak[2], weak[3])) < kFixedWeak;
 }
 
-// A site whose neighbours are zero (false: its sums are right), or hold numbers
-// the fixed-point form does not take (out = (D in)(h) in FP64).  Not inlined:
-// the FP64 arithmetic would be in every kernel that has the fixed-point one.
+// A site whose neighbours are zero (out = 0), or hold numbers the fixed-point form
+// does not take or would not keep (out = (D in)(h) in FP64).  Not inlined: the FP64
+// arithmetic would be in every kernel that has the fixed-point one.
 template <bool DAGGER, bool TFIX, bool PAIR>
-__device__ __noinline__ bool dslash_site_outside(Geom g, SpinorF64 in, GaugeX64 gauge, int h,
+__device__ __noinline__ void dslash_site_outside(Geom g, SpinorF64 in, GaugeX64 gauge, int h,
                                                  int parity, int top, double (&out)[24]) {
   if (top < kFixedMinExp) {
     int x, y, z, t;
@@ -381,10 +381,13 @@ __device__ __noinline__ bool dslash_site_outside(Geom g, SpinorF64 in, GaugeX64 
         const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(in.p + (size_t)c * in.stride + nb[k]));
         any |= (v.x | v.y) & 0x7fffffffffffffffull;
       }
-    if (any == 0) return false;
+    if (any == 0) {
+#pragma unroll
+      for (int k = 0; k < 24; ++k) out[k] = 0.0;
+      return;
+    }
   }
   dslash_site<DAGGER, TFIX, false, PAIR>(g, in, gauge.f64(), h, parity, out);
-  return true;
 }
 
 // U h: the limbs of the two rows of h, the link in its slots read by rows (step
@@ -586,8 +589,8 @@ __device__ __forceinline__ void fixed_hops(const Geom& g, const SpinorF64& in, c
     if (unit) {
 #pragma unroll
       for (int q = 0; q < 6; ++q) {
-        gr[q / 3][q % 3] = (hr[q / 3][q % 3] + 8) >> 4;
-        gi[q / 3][q % 3] = (hi[q / 3][q % 3] + 8) >> 4;
+        gr[q / 3][q % 3] = (hr[q / 3][q % 3] + 4) >> 3;
+        gi[q / 3][q % 3] = (hi[q / 3][q % 3] + 4) >> 3;
       }
     } else {
       if (gauge.recon == 12) fx_row3(sm);
@@ -617,14 +620,13 @@ __device__ __forceinline__ void dslash_site_fixed(const Geom& g, const SpinorF64
   fixed_hops<DAGGER, TFIX>(g, in, gauge, sm, h, parity, 0, 8, E, top, acc, weak);
   if (top < kFixedMinExp || top > kFixedMaxExp || fixed_is_weak(weak)) {
     double slow[24];  // its address is taken on this path only
-    if (dslash_site_outside<DAGGER, TFIX, PAIR>(g, in, gauge, h, parity, top, slow)) {
+    dslash_site_outside<DAGGER, TFIX, PAIR>(g, in, gauge, h, parity, top, slow);
 #pragma unroll
-      for (int k = 0; k < 24; ++k) out[k] = slow[k];
-      return;
-    }
+    for (int k = 0; k < 24; ++k) out[k] = slow[k];
+    return;
   }
 #pragma unroll
-  for (int k = 0; k < 24; ++k) out[k] = fx_sum_value(acc[k], E - 1078);
+  for (int k = 0; k < 24; ++k) out[k] = fx_sum_value(acc[k], E - 1079);
 }
 
 // The same with four warps for 32 sites, warp w taking the two hops of direction
@@ -669,8 +671,8 @@ __device__ __forceinline__ bool dslash_site_fixed_split(const Geom& g, const Spi
         r += fx_round_sar(v.x, E - e[q]);
         i += fx_round_sar(v.y, E - e[q]);
       }
-      fin[(6 * w + 2 * c) * 32 + lane] = fx_sum_value(r, E - 1078);
-      fin[(6 * w + 2 * c + 1) * 32 + lane] = fx_sum_value(i, E - 1078);
+      fin[(6 * w + 2 * c) * 32 + lane] = fx_sum_value(r, E - 1079);
+      fin[(6 * w + 2 * c + 1) * 32 + lane] = fx_sum_value(i, E - 1079);
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -685,11 +687,10 @@ __device__ __forceinline__ bool dslash_site_fixed_split(const Geom& g, const Spi
   if (!ok || w != 0) return false;
   if (top < kFixedMinExp || top > kFixedMaxExp || fixed_is_weak(weak)) {
     double slow[24];
-    if (dslash_site_outside<DAGGER, TFIX, PAIR>(g, in, gauge, h, parity, top, slow)) {
+    dslash_site_outside<DAGGER, TFIX, PAIR>(g, in, gauge, h, parity, top, slow);
 #pragma unroll
-      for (int k = 0; k < 24; ++k) out[k] = slow[k];
-      return true;
-    }
+    for (int k = 0; k < 24; ++k) out[k] = slow[k];
+    return true;
   }
 #pragma unroll
   for (int k = 0; k < 24; ++k) out[k] = fin[k * 32 + lane];

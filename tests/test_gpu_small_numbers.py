@@ -102,9 +102,9 @@ def test_fp64_by_component(dims, recon, dagger, spread):
     """Every spin and colour is right to the sum of the |u| |psi| that feed it, however small beside the others.
     A field with a link that the integer form does not take is computed in FP64 throughout: its result is the
     reference away from that link.
-    18 reals: 23 units of 2^-55 of the common exponent at most in a real part, and what feeds a component is at least
-    2^-6 of it, or the site is computed in FP64: 23 sqrt(2) 2^-49, and FP64's 2^-48.  12 reals: the third row, which
-    both rebuild, is right to a few 2^-53 absolute, which is 64 times as much of a component fed by 2^-6."""
+    18 reals: 25 units of 2^-56 of the common exponent at most in a real part, and what feeds a component is at least
+    2^-7 of it, or the site is computed in FP64: 25 sqrt(2) 2^-49, and FP64's 2^-48.  12 reals: the third row, which
+    both rebuild, is right to a few 2^-53 absolute, which is 128 times as much of a component fed by 2^-7."""
     U = li.gauge(dims, 0.7, 1600)
     raw, psi = _fields(dims, 0, 2601, spread if isinstance(spread, int) else 0)
     if isinstance(spread, str):  # one spin (colour) 1e-18 of the others, links that do not mix it with them
@@ -122,8 +122,22 @@ def test_fp64_by_component(dims, recon, dagger, spread):
     odd = parity_sites(dims, 1)
     away = (feeds == feeds2).all(axis=1)[odd]
     assert away.sum() >= len(odd) - 2
-    bound = (2.0 ** -43.8 if recon == 18 else 2.0 ** -40) * feeds[odd]
+    bound = (2.0 ** -43.7 if recon == 18 else 2.0 ** -40) * feeds[odd]
     assert (np.abs(got - want) <= bound)[away].all(), np.nanmax(np.abs(got - want)[away] / feeds[odd][away])
+
+
+@pytest.mark.parametrize("dims", [(4, 6, 8, 10), (16, 14, 12, 18)])
+@pytest.mark.parametrize("recon", [12, 18])
+def test_negative_zeros(dims, recon):
+    """-0.0 beside -0.0 gives zeros, and beside numbers what +0.0 gives, to a unit in the last place of the largest."""
+    raw, _ = _fields(dims, 0, 2602, 0)
+    U = li.gauge(dims, 0.7, 1601)
+    assert (_raw_dslash(U, dims, np.full_like(raw, complex(-0.0, -0.0)), False, recon) == 0).all()
+    zero = np.random.default_rng(51).random(raw.shape[1]) < 0.5
+    plus, minus = raw.copy(), raw.copy()
+    plus[:, zero], minus[:, zero] = 0.0, complex(-0.0, -0.0)
+    a, b = _raw_dslash(U, dims, plus, False, recon), _raw_dslash(U, dims, minus, False, recon)
+    assert np.abs(a - b).max() <= 2.0 ** -50 * np.abs(raw).max()
 
 
 @pytest.mark.parametrize("exp2", [-264, -240])
