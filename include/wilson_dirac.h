@@ -101,10 +101,11 @@ size_t wd_field_bytes(const wd_ctx *ctx, wd_prec prec);
  * nine entries (FP64 only).  Lower-precision copies (FP32; Q16 codes
  * rint(u*32767); fp16; bf16) are derived from the FP64 copy on first use.
  * SU(3) links (each real at most 1.125, the reals of a row or column together
- * 0.99 to 3.5) are also kept as 64-bit integers u 2^61 for the FP64 dslash on the integer units, as many bytes again as the
- * FP64 copy, unless that is more than a quarter of the free device memory;
- * without them the FP64 dslash takes about three times as long.
- * Either way every complex component of an FP64 dslash is right to 2^-43 of
+ * 0.99 to 3.5) are also kept as 64-bit integers u 2^61 for the FP64 dslash on
+ * the integer units, as many bytes again as the FP64 copy, unless that is more
+ * than a quarter of the free device memory; without them the FP64 dslash takes
+ * about three times as long.
+ * Either way every complex component of an FP64 dslash is right to 2^-44 of
  * the sum of the |u| |psi| that feed it (2^-49 as a rule, and 2^-53 of the
  * largest neighbour component over a whole field); with recon = 12 the
  * elements of the rebuilt row, by either route, to a few 2^-53 of 1.

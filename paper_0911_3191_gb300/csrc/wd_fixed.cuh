@@ -5,9 +5,9 @@
 // integer add, logic or shift instruction every 2.4.  The FP64 stencil takes 614
 // FP64 instructions a site and is bound by that pipe alone (24^3 x 64, temporal
 // gauge, 18 reals: 471 us).  Here every number of a hop is a 64-bit integer, and a
-// product of two takes three integer multiply-adds: 148 us (its bytes take 81);
-// M_hat with 12-real general links of 20 x 14 x 22 x 38 130 us; 8^3 x 16, four
-// warps per 32 sites, 5.9 us.  No pipe is full: 12 warps per SM (168 registers)
+// product of two takes three integer multiply-adds: 149 us (its bytes take 81);
+// M_hat with 12-real general links of 20 x 14 x 22 x 38 132 us; 8^3 x 16, four
+// warps per 32 sites, 6.0 us.  No pipe is full: 12 warps per SM (168 registers)
 // leave the latencies of 6300 dependent integer instructions per 32 sites in sight.
 //
 //  * A link element u, |u| <= 1, is the integer u 2^61 (converted once, when
@@ -29,13 +29,13 @@
 // one unit as a rule; FP64 rounds each component relative to what feeds it, sum |u|
 // |psi|, which is more than B in ordinary fields but may be far less.  So each spin
 // collects the smallest colour of every row that feeds it (fixed_weight), and a site
-// with a spin that gets less than 2^-7 B is computed in FP64 (dslash_site).  What is
-// left is right to 2^-43 of sum |u| |psi| in every complex component, and as a rule
-// to 2^-49, the bound that FP64's 15 roundings have.  No site of Gaussian fields
-// goes that way, 2e-4 of a point source's solution at kappa 0.12, and the fronts of
-// its first iterates.  The weights take 2 % of the dslash (144.6 -> 148.0 us at
-// 24^3 x 64), the FP64 sites 1 % of twelve point sources' batch on
-// 16^3 x 32.
+// with a spin that gets less than 2^-6 B is computed in FP64 (dslash_site_weak).
+// What is left is right to 2^-44 of sum |u| |psi| in every complex component, and as
+// a rule to 2^-50, inside the 2^-49 that FP64's 15 roundings may add up to.  No site
+// of Gaussian fields goes that way, 5e-4 of a point source's solution at kappa 0.12,
+// and the fronts of its first iterates.  The weights take 3 % of the dslash (144.5 ->
+// 149.1 us at 24^3 x 64, 5.7 -> 6.0 at 8^3 x 16), the FP64 sites 0.3 % of twelve point
+// sources' batch on 16^3 x 32 (4 % when each was left to its own thread).
 // (A third row rebuilt from 12 reals is right to a few 2^-53 of 1 in FP64.)
 //
 // E is known only when all neighbours are, so it is a running maximum: a hop
@@ -54,7 +54,12 @@
 namespace wd {
 
 constexpr int kFixedMinExp = 192, kFixedMaxExp = 1892;  // biased exponents E of the fixed-point path
-constexpr int kFixedWeak = 1 << 20;  // 2^-7 of the common exponent, in the unit of the high words (fixed_weight)
+// Weak sites of a warp that its lanes compute together, one after the other; more
+// are computed by their own threads at a time.  8^3 x 16, 18 (12) reals: 3.1 us (3.9)
+// a site against 27 us (33) for all of a warp's; 24^3 x 64 with every site weak 1614
+// us (2180) against 632 (797), which crosses at ten.
+constexpr int kFixedShared = 8;
+constexpr int kFixedWeak = 1 << 21;  // 2^-6 of the common exponent, in the unit of the high words (fixed_weight)
 
 struct Fx {
   int h, l;  // h * 2^32 + l
@@ -357,13 +362,14 @@ __device__ __forceinline__ int fixed_weight(const long long (&hr)[3], const long
   for (int c = 0; c < 3; ++c) w[c] = max(abs((int)(hr[c] >> 32)), abs((int)(hi[c] >> 32)));
   return __vimin3_s32(w[0], w[1], w[2]);
 }
+__device__ __forceinline__ bool fixed_is_outside(int top) { return top < kFixedMinExp || top > kFixedMaxExp; }
 // An output spin that so little feeds that the unit of the sums may show in it
 __device__ __forceinline__ bool fixed_is_weak(const int (&weak)[4]) {
   return min(min(weak[0], weak[1]), min(weak[2], weak[3])) < kFixedWeak;
 }
 
 // A site whose neighbours are zero (out = 0), or hold numbers the fixed-point form
-// does not take or would not keep (out = (D in)(h) in FP64).  Not inlined: the FP64
+// does not take (out = (D in)(h) in FP64).  Not inlined: the FP64
 // arithmetic would be in every kernel that has the fixed-point one.
 template <bool DAGGER, bool TFIX, bool PAIR>
 __device__ __noinline__ void dslash_site_outside(Geom g, SpinorF64 in, GaugeX64 gauge, int h,
@@ -388,6 +394,133 @@ __device__ __noinline__ void dslash_site_outside(Geom g, SpinorF64 in, GaugeX64 
     }
   }
   dslash_site<DAGGER, TFIX, false, PAIR>(g, in, gauge.f64(), h, parity, out);
+}
+
+// Site h in FP64 by the warp's lanes 0 .. n - 1, all of which call this with the
+// same site (a site with a spin that little feeds): one part (re, im) of one row of
+// one hop per lane, 24 FP64 instructions each (56 with a third row to rebuild) and
+// 7 for the sums, against some 614 in a row by the site's own thread, 20 us that
+// the others of a launch then wait for.  The parts pass through the warp's spinor
+// slots (216 doubles, 64 to a row of slots).  Not inlined: its registers would be in
+// every kernel.
+struct FixedScratch {
+  FixedSlots& sm;
+  int first;  // the warp's first thread
+  __device__ __forceinline__ double& operator[](int i) const {
+    return reinterpret_cast<double*>(&sm.sp[i >> 6][first])[i & 63];
+  }
+};
+template <bool DAGGER, bool TFIX>
+__device__ __noinline__ void dslash_site_weak(Geom g, SpinorF64 in, GaugeF64 gauge, FixedSlots& sm, int h, int parity,
+                                              int n) {
+  const int lane = threadIdx.x & 31;
+  const unsigned lanes = 0xffffffffu >> (32 - n);
+  const FixedScratch sc{sm, (int)threadIdx.x - lane};
+  const int nc = gauge.recon >> 1;
+  int x, y, z, t;
+  site_coords(g, h, parity, x, y, z, t);
+  __syncwarp(lanes);  // the slots are read
+#pragma unroll 1
+  for (int role = lane; role < 32; role += n) {
+    const int k = role >> 2, row = (role >> 1) & 1, part = role & 1, mu = k >> 1;
+    const bool fwd = (k & 1) == 0;
+    const bool minus = fwd != DAGGER;  // S = -1
+    const int nb = fixed_neighbour(g, h, x, y, z, t, k);
+    // h = p + s q (y) or p + s i q (x, z), or twice p: its two parts in the order
+    // that this part of the product takes them
+    const int up = mu < 3 ? row : row + (minus ? 2 : 0);
+    const int lo = mu == 2 ? 2 + row : 3 - row;  // the spin that joins a row, and that it gives
+    const bool edge = mu == 3 && (fwd ? t == g.T - 1 : t == 0);
+    const double s = minus != (row == 1 && mu != 0) ? -1.0 : 1.0;
+    const double sr = mu == 1 ? s : -s, f = (edge && g.tbc_anti) ? -2.0 : 2.0;
+    double a[3], b[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double2 p = __ldg(in.p + (size_t)(3 * up + c) * in.stride + nb);
+      double hr, hi;
+      if (mu < 3) {
+        const double2 q = __ldg(in.p + (size_t)(3 * lo + c) * in.stride + nb);
+        hr = fma(sr, mu == 1 ? q.x : q.y, p.x);
+        hi = fma(s, mu == 1 ? q.y : q.x, p.y);
+      } else {
+        hr = f * p.x;
+        hi = f * p.y;
+      }
+      a[c] = part ? hi : hr;
+      b[c] = part ? hr : -hi;
+    }
+    double v[3];
+    if (TFIX && mu == 3 && !edge) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) v[c] = a[c];
+    } else {
+      const double2* l = gauge.p + (size_t)((fwd ? parity : 1 - parity) * 4 + mu) * nc * gauge.stride + (fwd ? h : nb);
+      double u[18];
+#pragma unroll
+      for (int e = 0; e < 9; ++e) {
+        const double2 d = e < nc ? __ldg(l + (size_t)e * gauge.stride) : make_double2(0.0, 0.0);
+        u[2 * e] = d.x;
+        u[2 * e + 1] = d.y;
+      }
+      if (nc == 6) reconstruct_row3(u);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        v[c] = 0.0;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          const int e = 2 * (3 * c + j), et = 2 * (3 * j + c);  // U, or U^dag
+          v[c] = fma(fwd ? u[e] : u[et], a[j], v[c]);
+          v[c] = fma(fwd ? u[e + 1] : -u[et + 1], b[j], v[c]);
+        }
+      }
+    }
+    // to its own spin, and (spatial hops) to the other: s' v (y), or s' i v (x, z)
+    const bool m1 = mu == 0 ? !minus : mu == 1 ? minus == (row == 0) : minus != (row == 0);
+    const int to = mu == 1 ? part : 1 - part;
+    const bool m2 = m1 != (mu != 1 && part == 1);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      sc[24 * k + 6 * up + 2 * c + part] = v[c];
+      if (mu < 3) sc[24 * k + 6 * lo + 2 * c + to] = m2 ? -v[c] : v[c];
+    }
+  }
+  __syncwarp(lanes);
+  for (int q = lane; q < 24; q += n) {
+    double v = sc[24 * ((q >= 12) != DAGGER ? 6 : 7) + q];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) v += sc[24 * k + q];
+    sc[192 + q] = v;
+  }
+  __syncwarp(lanes);
+}
+
+// out of the lanes in `todo`, whose sites are weakly fed, computed in FP64; the
+// warp's lanes 0 .. n - 1 have consecutive sites
+template <bool DAGGER, bool TFIX, bool PAIR>
+__device__ __forceinline__ void dslash_weak_sites(const Geom& g, const SpinorF64& in, const GaugeX64& gauge,
+                                                  FixedSlots& sm, int h, int parity, int n, unsigned todo,
+                                                  double (&out)[24]) {
+  const int lane = threadIdx.x & 31;
+  if (__popc(todo) > kFixedShared) {
+    if (todo >> lane & 1u) {
+      double slow[24];
+      dslash_site_outside<DAGGER, TFIX, PAIR>(g, in, gauge, h, parity, kFixedMinExp, slow);
+#pragma unroll
+      for (int k = 0; k < 24; ++k) out[k] = slow[k];
+    }
+    return;
+  }
+  while (todo) {
+    const int l = __ffs(todo) - 1;
+    todo &= todo - 1;
+    dslash_site_weak<DAGGER, TFIX>(g, in, gauge.f64(), sm, h - lane + l, parity, n);
+    if (lane == l) {
+      const FixedScratch sc{sm, (int)threadIdx.x - lane};
+#pragma unroll
+      for (int k = 0; k < 24; ++k) out[k] = sc[192 + k];
+    }
+    __syncwarp(0xffffffffu >> (32 - n));
+  }
 }
 
 // U h: the limbs of the two rows of h, the link in its slots read by rows (step
@@ -611,22 +744,25 @@ __device__ __forceinline__ void fixed_hops(const Geom& g, const SpinorF64& in, c
 #undef WD_FIXED_ADD
 }
 
-// out = (D in)(h) for this thread's site
+// out = (D in)(h) for this thread's site; the warp's lanes 0 .. n - 1 have one
 template <bool DAGGER, bool TFIX, bool PAIR>
 __device__ __forceinline__ void dslash_site_fixed(const Geom& g, const SpinorF64& in, const GaugeX64& gauge,
-                                                  FixedSlots& sm, int h, int parity, double (&out)[24]) {
+                                                  FixedSlots& sm, int h, int parity, int n, double (&out)[24]) {
   int E, top, weak[4];
   long long acc[24];
   fixed_hops<DAGGER, TFIX>(g, in, gauge, sm, h, parity, 0, 8, E, top, acc, weak);
-  if (top < kFixedMinExp || top > kFixedMaxExp || fixed_is_weak(weak)) {
+  const bool outside = fixed_is_outside(top);
+  if (outside) {
     double slow[24];  // its address is taken on this path only
     dslash_site_outside<DAGGER, TFIX, PAIR>(g, in, gauge, h, parity, top, slow);
 #pragma unroll
     for (int k = 0; k < 24; ++k) out[k] = slow[k];
-    return;
-  }
+  } else {
 #pragma unroll
-  for (int k = 0; k < 24; ++k) out[k] = fx_sum_value(acc[k], E - 1079);
+    for (int k = 0; k < 24; ++k) out[k] = fx_sum_value(acc[k], E - 1079);
+  }
+  const unsigned todo = __ballot_sync(0xffffffffu >> (32 - n), !outside && fixed_is_weak(weak));
+  dslash_weak_sites<DAGGER, TFIX, PAIR>(g, in, gauge, sm, h, parity, n, todo, out);
 }
 
 // The same with four warps for 32 sites, warp w taking the two hops of direction
@@ -652,7 +788,8 @@ __device__ __forceinline__ bool dslash_site_fixed_split(const Geom& g, const Spi
   }
   __syncthreads();
   double* fin = reinterpret_cast<double*>(&sm.lk[1][0]);  // [24][32]
-  int top = 0, weak[4] = {0, 0, 0, 0};
+  const int n = min(32, h_end - h0);
+  int top = 0;
   if (ok) {
     int e[4], E = 0;
 #pragma unroll
@@ -674,26 +811,25 @@ __device__ __forceinline__ bool dslash_site_fixed_split(const Geom& g, const Spi
       fin[(6 * w + 2 * c) * 32 + lane] = fx_sum_value(r, E - 1079);
       fin[(6 * w + 2 * c + 1) * 32 + lane] = fx_sum_value(i, E - 1079);
     }
+    int feeds = 0;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int4 v = sm.lk[4][lane + 32 * q];
-      weak[0] += fx_shr32(v.x, E - e[q]);
-      weak[1] += fx_shr32(v.y, E - e[q]);
-      weak[2] += fx_shr32(v.z, E - e[q]);
-      weak[3] += fx_shr32(v.w, E - e[q]);
-    }
+    for (int q = 0; q < 4; ++q) feeds += fx_shr32(reinterpret_cast<const int*>(&sm.lk[4][lane + 32 * q])[w], E - e[q]);
+    const unsigned weak_w = __ballot_sync(0xffffffffu >> (32 - n), feeds < kFixedWeak && !fixed_is_outside(top));
+    if (lane == 0) reinterpret_cast<unsigned*>(&sm.lk[5][0])[w] = weak_w;
   }
   __syncthreads();
   if (!ok || w != 0) return false;
-  if (top < kFixedMinExp || top > kFixedMaxExp || fixed_is_weak(weak)) {
+  if (fixed_is_outside(top)) {
     double slow[24];
     dslash_site_outside<DAGGER, TFIX, PAIR>(g, in, gauge, h, parity, top, slow);
 #pragma unroll
     for (int k = 0; k < 24; ++k) out[k] = slow[k];
-    return true;
-  }
+  } else {
 #pragma unroll
-  for (int k = 0; k < 24; ++k) out[k] = fin[k * 32 + lane];
+    for (int k = 0; k < 24; ++k) out[k] = fin[k * 32 + lane];
+  }
+  const int4 f = sm.lk[5][0];
+  dslash_weak_sites<DAGGER, TFIX, PAIR>(g, in, gauge, sm, h, parity, n, (unsigned)(f.x | f.y | f.z | f.w), out);
   return true;
 }
 
@@ -712,7 +848,8 @@ __device__ __forceinline__ void dslash_sites_fixed(const Geom& g, const SpinorF6
     }
   } else {
     for (int h = h_begin + blockIdx.x * blockDim.x + threadIdx.x; h < h_end; h += gridDim.x * blockDim.x) {
-      dslash_site_fixed<DAGGER, TFIX, kPair>(g, in, gauge, sm, h, parity, acc);
+      dslash_site_fixed<DAGGER, TFIX, kPair>(g, in, gauge, sm, h, parity, min(32, h_end - h + (int)(threadIdx.x & 31)),
+                                             acc);
       epi(h, acc, red);
     }
   }
