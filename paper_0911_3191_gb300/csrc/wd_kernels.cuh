@@ -1306,8 +1306,8 @@ void launch_dslash(const Ctx& c, const In& in, const G& gauge, int parity, Dag d
     // window of the lattice and find their neighbours in L2, where looping blocks
     // drift apart.  Against 2 waves (temporal gauge) and 16 per SM (general links):
     // Q16 948 -> 878 and 1021 -> 965 us, bf16 880 -> 835 and 978 -> 875, fp16 977 ->
-    // 901 and 1022 -> 980; 48^3 x 96 bf16 general 307 -> 273; FP64 32^3 x 64 345 ->
-    // 331; nothing on 24^3 x 64, which L2 holds.  FP32: one wave of resident blocks
+    // 901 and 1022 -> 980; 48^3 x 96 bf16 general 307 -> 273; FP64 32^3 x 64 347 ->
+    // 334; nothing on 24^3 x 64, which L2 holds.  FP32: one wave of resident blocks
     // (48^3 x 96 401 us against 410 without a loop and 491 at 16 per SM; general
     // links 461, 463, 547).  Fused reductions, whose partial sums grow with the
     // blocks: one wave in 16 bit (two: the 24^3 x 64 solve 0.1 % slower), 16 per SM
@@ -1318,11 +1318,11 @@ void launch_dslash(const Ctx& c, const In& in, const G& gauge, int parity, Dag d
     static const int per_sm = kMany ? 16 : resident_blocks(k, kDslashBlock);
     const int n = geo.h_end - geo.h_begin;
     // Split kernels (a site over four warps) up to one block of 128 sites per
-    // SM.  FP64 in fixed point, 152 SMs, back to back: 2048 and 4096 sites 13.4 ->
-    // 5.7 us, 8192 13.2 -> 7.1, 16384 13.4 -> 12.2, 32768 17.2 against 18.1, 65536
-    // 30.2 against 32.4.  With fused reductions, whose FP64 arithmetic one warp of the
-    // four does, half as far: <r_tilde, v> at 4096 sites 18.1 -> 11.1 us, 8192
-    // 18.2 -> 12.5, 16384 18.6 against 20.9.  Not compiled for general FP64 links
+    // SM.  FP64 in fixed point, 152 SMs, back to back: 2048 and 4096 sites 14.1 ->
+    // 5.8 us, 8192 13.8 -> 7.2, 16384 14.0 -> 12.3, 32768 17.3 against 18.3, 65536
+    // 30.8 against 32.5.  With fused reductions, whose FP64 arithmetic one warp of the
+    // four does, half as far: <r_tilde, v> at 4096 sites 19.2 -> 11.4 us, 8192
+    // 19.2 -> 12.8, 16384 19.1 against 21.5.  Not compiled for general FP64 links
     // and 8-number links.
     if constexpr (!std::is_same<G, GaugeF64>::value && !kR8) {
       constexpr int kSites = (sizeof(R) == 8 && Epi::NRED > 0) ? kDslashBlock / 2 : kDslashBlock;
